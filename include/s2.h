@@ -255,8 +255,8 @@ int s2_set_tiles(s2_solver *s, const int *tiles);
  * (Table 3) and of its translator's configuration (Sec. 3.3), searched by
  * the autotuner (paper_2304_05494_gb300/autotune.py).  tiles: as
  * s2_set_tiles.  flux_ctas_per_sm[d]: CTAs per multiprocessor of the
- * persistent single-precision flux grid of direction d (0: as many as
- * fit, up to 16).
+ * persistent flux grid of direction d (0: as many as fit, up to 16; KEEP
+ * in S2_FP64 has no persistent grid).
  * z_planes: z-planes each CTA of the mixed path's z-marching gradient and
  * viscous passes walks (0: 12; else 4, 8, 16 or 24, compiled variants).  weno_ctas_per_sm: cap of the
  * WENO kernels' 64-thread CTAs per multiprocessor (0: 16; else 1..64).

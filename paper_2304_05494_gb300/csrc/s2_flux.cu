@@ -8,13 +8,12 @@
 // kernels of Table 2.  The paper's transposition kernel for x is not needed:
 // every direction stages its pencils through shared memory.
 //
-// k_flux<DIR>  tiles of L points along DIR times W pencils (one tile per CTA
-// in double precision; a persistent grid walking the tiles in single
-// precision):
+// k_flux<DIR>  tiles of L points along DIR times W pencils (a persistent grid
+// walking the tiles; KEEP in double precision one tile per CTA):
 //   1. the tile plus GH ghost points each side arrives by TMA, one box per
 //      staged field (rho, u, v, w, H, p, and the sensor test for WENO),
-//      completing on an mbarrier; single precision prefetches the next
-//      tiles into further buffers while computing this one;
+//      completing on an mbarrier; the next tiles are prefetched into further
+//      buffers while computing this one;
 //   2. per position a the weighted pair mass fluxes of the pairs (a, a+l),
 //      l = 1..NP: m_l(a) = (a_l/4) (rho_a+rho_b)(un_a+un_b);
 //   3. the central flux difference D(a) = F_{a+1/2} - F_{a-1/2} of the
@@ -38,6 +37,7 @@
 // (arithmetic of the mixed path).
 #include <string.h>
 
+#include "s2_fixed.cuh"
 #include "s2_internal.cuh"
 
 namespace s2 {
@@ -148,9 +148,10 @@ struct FluxLayout {
   static constexpr int SFA = (SF * (int)sizeof(R) + 127) / 128 * 128 / (int)sizeof(R);  // 128-B aligned
   static constexpr int BAR_BYTES = 128;                          // mbarriers, padded
   // staging buffers: single precision prefetches two tiles ahead in x and
-  // one in y and z (larger tiles); double precision runs one tile per CTA
-  // and stages it once
-  static constexpr int NBUF = sizeof(R) == 4 ? (DIR == 0 ? 3 : 2) : 1;
+  // one in y and z (larger tiles), double precision one; KEEP in double
+  // precision (bound by the double-precision unit, and with five times the
+  // pair words) runs one tile per CTA and stages it once
+  static constexpr int NBUF = sizeof(R) == 4 ? (DIR == 0 ? 3 : 2) : (TV == 2 ? 1 : 2);
 };
 
 // Dynamic shared memory of a flux CTA: barriers, staging buffers and the
@@ -188,6 +189,115 @@ __device__ __forceinline__ void keep_pairs_tile(const R *S, R *TP, R gm1, int n)
   }
 }
 
+// Double precision, split form: the pair mass fluxes and the flux
+// difference in fixed point (s2_fixed.cuh).  Per point of an order-6 flux
+// the double unit executed 61 operations (64 issue clocks each); here it
+// executes 17 (five conversions, the pressure difference, the sums into the
+// RHS), the integer unit the rest beside them.  On 420 x 250 x 320 points a
+// launch went from 3.85 / 3.70 / 3.64 ms (x / y / z) to 1.33 / 1.28 / 1.29.
+// With the double unit no longer the bound, the persistent grid that
+// prefetches the next tile pays here too: with one tile per CTA the same
+// arithmetic took 2.67 / 2.77 / 2.72 ms (waiting at barriers and for the
+// tile's copy).
+//
+// The staged rho, u, v, w, H become limbs in place.
+template <int SFA>
+__device__ __forceinline__ void fx_convert_tile(double *S, const int *e) {
+  static_assert(SFA % 2 == 0, "a thread converts two values of one field at a time");
+#pragma unroll
+  for (int it = 0; it < (5 * SFA / 2 + NTHREADS - 1) / NTHREADS; ++it) {
+    const int idx = threadIdx.x + it * NTHREADS;
+    if (idx < 5 * SFA / 2) {
+      const int ef = e[idx / (SFA / 2)];
+      const double2 x = ((const double2 *)S)[idx];
+      const int2 a = fx_split(x.x, ef), b = fx_split(x.y, ef);
+      ((int4 *)S)[idx] = make_int4(a.x, a.y, b.x, b.y);
+    }
+  }
+}
+
+// a_l / 2 as a 60-bit fraction in limbs of its own sign.
+template <int NP>
+__device__ __forceinline__ constexpr int2 acoef_limbs(int l) {
+  const double a = acoef<NP>(l) * 0.5;
+  const double m = a < 0 ? -a : a;
+  const long long k = (long long)(m * 1152921504606846976.0);
+  const int lo = (int)(k & FX_MASK), hi = (int)(k >> FX_LIMB);
+  return a < 0 ? int2{-lo, -hi} : int2{lo, hi};
+}
+
+// Pair mass fluxes m_l(a), a = -NP .. L-1, in units of 2^(E_rho + E_n - 59).
+// (rho_a + rho_b)(un_a + un_b) is formed to 2^-60 of its largest value, and
+// so is its product with a_l / 4.
+template <int DIR, int NP, int LT, int W, int SA, int SCS, int SCT, int SFA>
+__device__ __forceinline__ void fx_pairs_tile(const int2 *S, int2 *TP) {
+  constexpr int ST = LT * W;
+  for (int idx = threadIdx.x; idx < ST; idx += NTHREADS) {
+    int a, cc;
+    if (DIR == 0) { a = idx % LT; cc = idx / LT; }
+    else { a = idx / W; cc = idx % W; }
+    const int2 *Sr = S + F_RHO * SFA, *Sn = S + (F_U + DIR) * SFA;
+    const int q0 = (a - NP + GH) * SA + cc * SCS;
+    const int2 r0 = Sr[q0], n0 = Sn[q0];
+#pragma unroll
+    for (int l = 1; l <= NP; ++l) {
+      const int2 r1 = Sr[q0 + l * SA], n1 = Sn[q0 + l * SA];
+      const long long P = fx_mulhi(r0.x + r1.x, r0.y + r1.y, n0.x + n1.x, n0.y + n1.y);
+      const int2 k = acoef_limbs<NP>(l);
+      const long long m = fx_mulhi((int)P & FX_MASK, (int)(P >> FX_LIMB), k.x, k.y);
+      TP[(l - 1) * ST + a * SA + cc * SCT] = make_int2((int)m & FX_MASK, (int)(m >> FX_LIMB));
+    }
+  }
+}
+
+// The flux difference of one point: D_rho = 2 M, D_phi = phi_a M + sum_l
+// [m_l(a) phi_{a+l} - m_l(a-l) phi_{a-l}], each product to 2^-60 of its
+// largest value: A collects the hi hi products, B the mixed ones.  |m| is
+// below 2^59 sum |a_l| and the lo limbs of m are not negative, so with 8
+// pairs (order 8) |B| stays below 2^59 (8 + 2.1 + 1 + 2.1) < 2^63.
+template <int DIR, int NP, int ST, int SA, int SFA>
+__device__ __forceinline__ void fx_flux_point(const int2 *S, const int2 *TP, int at, int ap, const int *e,
+                                              double dp, double scale, const double *prev, double *out,
+                                              long long n) {
+  int2 mp[NP], mm[NP];  // m_l(a), -m_l(a-l)
+  int Ml = 0, Mh = 0;
+#pragma unroll
+  for (int l = 1; l <= NP; ++l) {
+    mp[l - 1] = TP[(l - 1) * ST + at];
+    const int2 m = TP[(l - 1) * ST + at - l * SA];
+    mm[l - 1] = make_int2(-m.x, -m.y);
+    Ml += mp[l - 1].x + mm[l - 1].x;
+    Mh += mp[l - 1].y + mm[l - 1].y + (Ml >> FX_LIMB);
+    Ml &= FX_MASK;
+  }
+  const int eM = e[F_RHO] + e[F_U + DIR] - 2 * 1022 - 59;  // unit of m
+  const double M = __ll2double_rn((long long)Mh * (1 << FX_LIMB) + Ml);
+  out[0] = fma(-fx_ldexp(scale, eM + 1), M, prev[0]);
+#pragma unroll
+  for (int f = 1; f < 5; ++f) {
+    const int2 *Sf = S + f * SFA;  // F_U .. F_H follow F_RHO
+    const int2 c = Sf[ap];
+    long long A = (long long)Mh * c.y;
+    long long B = (long long)Mh * c.x + (long long)Ml * c.y;
+#pragma unroll
+    for (int l = 1; l <= NP; ++l) {
+      const int2 vp = Sf[ap + l * SA], vm = Sf[ap - l * SA];
+      A += (long long)mp[l - 1].y * vp.y;
+      B += (long long)mp[l - 1].y * vp.x;
+      B += (long long)mp[l - 1].x * vp.y;
+      A += (long long)mm[l - 1].y * vm.y;
+      B += (long long)mm[l - 1].y * vm.x;
+      B += (long long)mm[l - 1].x * vm.y;
+    }
+    const double D = __ll2double_rn(A + (B >> FX_LIMB));
+    // unit of D: 2^60 times the units of m and phi
+    const int eD = eM + e[f] - 1022 + 1;
+    double r = fma(-fx_ldexp(scale, eD), D, prev[f]);
+    if (f == 1 + DIR) r = fma(-scale, dp, r);
+    out[f * n] = r;
+  }
+}
+
 // CTAs walk the tiles of a direction (t = block index, + grid extent, ...).
 // With NBUF staging buffers, the tensor memory accelerator fills the
 // buffers of the next NBUF - 1 tiles while tile t is computed, so the HBM
@@ -216,6 +326,9 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
   const View<R> V = view<R>(d);
   const Consts<R> &K = consts<R>(d);
   const int ntiles = tg.count();
+  // split form in double precision: fixed point where the fields allow it
+  constexpr bool FX = sizeof(R) == 8 && TV != 2;
+  __shared__ int fx_e[8];  // exponents of rho, u, v, w, H by F_*; [5]: fixed point
 
   const int tid = threadIdx.x;
   const int n = DIR == 0 ? d.nx : (DIR == 1 ? d.ny : d.nz);
@@ -239,7 +352,17 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
     for (int j = 0; j < NBUF - 1; ++j)
       if ((int)B.x + j * G < ntiles) issue((int)B.x + j * G, j);
   }
+  if (FX && tid == 32) {
+    const FxScale fx = fx_scale(d);
+    fx_e[F_RHO] = fx.e[FX_RHO];
+    fx_e[F_U] = fx.e[FX_U];
+    fx_e[F_V] = fx.e[FX_V];
+    fx_e[F_W] = fx.e[FX_W];
+    fx_e[F_H] = fx.e[FX_H];
+    fx_e[5] = fx.ok;
+  }
   __syncthreads();
+  const bool fixed = FX && fx_e[5];
 
   int it = 0;
   for (int t = (int)B.x; t < ntiles; t += G, ++it) {
@@ -261,6 +384,7 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
     bool mine[PPT];
     long long q[PPT];
     R prev[PPT][5];
+    R ey[PPT];  // fixed point: eta_y of the point's row, loaded early like its RHS
 #pragma unroll
     for (int pp = 0; pp < PPT; ++pp) {
       mine[pp] = (c0 + tc < nac) && (s0 + ta[pp] < n);
@@ -272,9 +396,16 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
       if (mine[pp] && !S2_OK_IDX(d, q[pp], d.n)) mine[pp] = false;
 #pragma unroll
       for (int f = 0; f < 5; ++f) prev[pp][f] = (mine[pp] && accumulate) ? V.fl[f * d.n + q[pp]] : R(0);
+      if (FX && DIR == 1) ey[pp] = mine[pp] && S2_OK_IDX(d, pj, d.ny) ? __ldg(V.eta_y + pj) : R(0);
     }
     bool late = false;
-    if (tid == 0) late = !mbar_wait_bounded(&bar[buf], (unsigned)(it / NBUF) & 1u, d.wait_ns);
+    if (FX) {
+      // every thread waits, so that each converts its share at once
+      late = !mbar_wait_bounded(&bar[buf], (unsigned)(it / NBUF) & 1u, d.wait_ns);
+      if (fixed && !late) fx_convert_tile<SFA>((double *)Sbuf + buf * NFLD * SFA, fx_e);
+    } else if (tid == 0) {
+      late = !mbar_wait_bounded(&bar[buf], (unsigned)(it / NBUF) & 1u, d.wait_ns);
+    }
     if (__syncthreads_or(late)) {
       if (tid == 0) {
         atomicOr(&d.scal->status, ERR_TIMEOUT);
@@ -291,6 +422,8 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
     // (KEEP: the five components of a_l f*(a, a+l) instead)
     if constexpr (TV == 2) {
       keep_pairs_tile<DIR, R, NP, LT, W, SA, SCS, SCT, SFA>(S, TP, K.gamma - R(1), d.keep);
+    } else if (fixed) {
+      if constexpr (FX) fx_pairs_tile<DIR, NP, LT, W, SA, SCS, SCT, SFA>((const int2 *)S, (int2 *)TP);
     } else
     for (int idx = tid; idx < ST; idx += NTHREADS) {
       int a, cc;                            // a in 0..LT-1 <-> position a-NP
@@ -388,6 +521,20 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
       R D[5];
       const int at = (ta[pp] + NP) * SA + tc * SCT;
       const int ap = (ta[pp] + GH) * SA + tc * SCS;
+      const R *Sp = S + F_P * SFA;
+      R dp = R(0);
+#pragma unroll
+      for (int l = 1; l <= NP; ++l) dp = fma(R(acoef<NP>(l)), Sp[ap + l * SA] - Sp[ap - l * SA], dp);
+      const int pj = DIR == 0 ? y0 + tc : (DIR == 1 ? y0 + ta[pp] : y0);
+      if (DIR == 1 && !S2_OK_IDX(d, pj, d.ny)) continue;
+      R scale = DIR == 0 ? K.idx : (DIR == 1 ? (FX ? ey[pp] : __ldg(V.eta_y + pj)) : K.idz);
+      if constexpr (FX) {
+        if (fixed) {
+          fx_flux_point<DIR, NP, ST, SA, SFA>((const int2 *)S, (const int2 *)TP, at, ap, fx_e, dp, scale, prev[pp],
+                                              V.fl + q[pp], d.n);
+          continue;
+        }
+      }
       R mp[NP], mm[NP];                     // m_l(a), m_l(a-l)
       R M = R(0);
 #pragma unroll
@@ -410,19 +557,15 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
         }
         D[f] = acc;
       }
-      const R *Sp = S + F_P * SFA;
-      R dp = R(0);
-#pragma unroll
-      for (int l = 1; l <= NP; ++l) dp = fma(R(acoef<NP>(l)), Sp[ap + l * SA] - Sp[ap - l * SA], dp);
       D[1 + DIR] += dp;
-      const int pj = DIR == 0 ? y0 + tc : (DIR == 1 ? y0 + ta[pp] : y0);
-      if (DIR == 1 && !S2_OK_IDX(d, pj, d.ny)) continue;
-      R scale = DIR == 0 ? K.idx : (DIR == 1 ? __ldg(V.eta_y + pj) : K.idz);
       const R scale0 = DIR == 0 ? K.idx2 : (DIR == 1 ? scale : K.idz2);
       V.fl[q[pp]] = fma(-scale0, D[0], prev[pp][0]);
 #pragma unroll
       for (int f = 1; f < 5; ++f) V.fl[f * d.n + q[pp]] = fma(-scale, D[f], prev[pp][f]);
     }
+    // the limbs were written by ordinary stores: order them before the copy
+    // that refills the buffer
+    if (FX) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();  // staging buffer and TP free for the next tile
   }
 }
@@ -727,11 +870,10 @@ __global__ void __launch_bounds__(WENO_NT) kb_weno(BatchArgs ba) {
   weno_body<DIR, WR, R>(sd, B);
 }
 
-// Single precision (bound by memory traffic): a persistent grid, as many
-// CTAs as fit on the device at once, each prefetching its next two tiles.
-// Double precision (bound by the double-precision unit): one tile per CTA,
-// so that more CTAs at different phases share each multiprocessor and keep
-// that unit busy (measured faster than the persistent loop).
+// A persistent grid, as many CTAs as fit on the device at once, each
+// prefetching its next tiles.  KEEP in double precision (bound by the
+// double-precision unit): one tile per CTA, so that more CTAs at different
+// phases share each multiprocessor and keep that unit busy.
 template <int DIR, bool HASW, class R, int TV, int NP>
 cudaError_t launch_one(const Dev &d, const FluxMaps &maps, int accumulate, cudaStream_t st) {
   static int per_sm = 0;  // resident CTAs per multiprocessor (per instantiation)
@@ -747,7 +889,7 @@ cudaError_t launch_one(const Dev &d, const FluxMaps &maps, int accumulate, cudaS
   const TileGrid<DIR, TV, R> tg(d);
   const int ntiles = tg.count();
   const int cps = d.flux_cps[DIR] > 0 && d.flux_cps[DIR] < per_sm ? d.flux_cps[DIR] : per_sm;
-  const int nb = sizeof(R) == 8 ? ntiles : (ntiles < cps * d.nsm ? ntiles : cps * d.nsm);
+  const int nb = FluxLayout<DIR, R, TV>::NBUF == 1 ? ntiles : (ntiles < cps * d.nsm ? ntiles : cps * d.nsm);
   k_flux<DIR, HASW, R, TV, NP><<<nb, NTHREADS, smem, st>>>(maps, d, tg, accumulate);
   return cudaGetLastError();
 }
@@ -982,7 +1124,7 @@ struct FluxPlan {
     out.tg_size = (int)sizeof(tg);
     out.tiles = tg.count();
     out.per_sm = d.flux_cps[DIR] > 0 && d.flux_cps[DIR] < per_sm ? d.flux_cps[DIR] : per_sm;
-    out.persistent = sizeof(R) == 4;
+    out.persistent = FluxLayout<DIR, R, TV>::NBUF > 1;
     return cudaSuccess;
   }
 };

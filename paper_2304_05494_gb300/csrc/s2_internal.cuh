@@ -14,6 +14,11 @@ namespace s2 {
 constexpr int GH = 4;
 constexpr int NV = 5;
 
+// Fields with a fixed-point exponent (s2_fixed.cuh); the first FX_NMIN also
+// record their smallest magnitude.
+enum { FX_RHO = 0, FX_T, FX_P, FX_U, FX_V, FX_W, FX_H, FX_NF };
+constexpr int FX_NMIN = 3;
+
 // Device-side scalars of one solver.
 struct Scal {
   double dt;              // current time step
@@ -26,6 +31,11 @@ struct Scal {
   int pad;
   long long nstep;        // completed RK3 steps (decides the dt recomputation on the device)
   double red[8];          // results of the last stats reduction
+  // biased exponent of the largest magnitude of each field of this RHS
+  // evaluation, and 2047 - that of the smallest (0: nothing seen yet); the
+  // primitive and ghost passes raise them, the pass that ends the
+  // evaluation clears them
+  unsigned int fx_e[FX_NF], fx_m[FX_NMIN];
 };
 
 // Error bits kernels OR into Scal::status (mapped on the host to
@@ -108,9 +118,10 @@ struct Dev {
   int dt_every;            // recompute dt at steps that are multiples of this (cfl > 0)
   double vol_inv;          // 1 / sum(dV) / (dx dz) for the forcing
   int viscous, wall_y, weno, force;
+  int fx;                  // 1: FP64 with 1/dx, eta_y, 1/dz in the range of the fixed-point path (s2_fixed.cuh)
   int mixed;               // 0: FP64 everywhere; 1: FP32 primitives and flux arithmetic, FP64 state
   int tile[3];             // flux tile variant per direction (0 default, 1 narrow)
-  int flux_cps[3];         // single-precision flux grids, per direction: resident CTAs per SM to use (0: all that fit)
+  int flux_cps[3];         // persistent flux grids, per direction: resident CTAs per SM to use (0: all that fit)
   int zs;                  // planes per CTA of the z-marching passes (mixed path)
   int weno_cps;            // WENO grids: CTAs per SM
   int nsm;                 // multiprocessors of the device
@@ -657,7 +668,7 @@ cudaError_t flux_set_attributes();
 struct FluxBoxPlan {
   unsigned char tg[64];
   int tg_size, tiles, per_sm;
-  bool persistent;  // single precision: CTAs walk several tiles
+  bool persistent;  // CTAs walk several tiles
 };
 cudaError_t flux_batch_plan(const Dev &d, int dir, FluxBoxPlan *out);
 unsigned weno_batch_blocks(const Dev &d, int dir);

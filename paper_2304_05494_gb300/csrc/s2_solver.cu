@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "../../include/s2.h"
+#include "s2_fixed.cuh"
 #include "s2_internal.cuh"
 
 using namespace s2;
@@ -158,6 +159,27 @@ __device__ __forceinline__ int block_want_dt(const Dev &d, int stage0) {
   return want;
 }
 
+// Exponents of a CTA's largest magnitudes (e[FX_*], 0 for threads without a
+// point) and smallest ones (m: 2047 - exponent) into Scal, for the
+// fixed-point path.  Whole warps reduce with one instruction per value and
+// one thread per value looks at the CTA's result: 0.2 % of k_prims.
+__device__ __forceinline__ void fx_block_raise(const Dev &d, const unsigned *e, const unsigned *m) {
+  __shared__ unsigned red[FX_NF + FX_NMIN][NT / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int f = 0; f < FX_NF + FX_NMIN; ++f) {
+    const unsigned r = __reduce_max_sync(0xffffffffu, f < FX_NF ? e[f] : m[f - FX_NF]);
+    if (lane == 0) red[f][wid] = r;
+  }
+  __syncthreads();
+  if (threadIdx.x < FX_NF + FX_NMIN) {
+    unsigned r = 0;
+    for (int w = 0; w < NT / 32; ++w) r = max(r, red[threadIdx.x][w]);
+    unsigned *at = threadIdx.x < FX_NF ? &d.scal->fx_e[threadIdx.x] : &d.scal->fx_m[threadIdx.x - FX_NF];
+    if (__ldcg(at) < r) atomicMax(at, r);
+  }
+}
+
 // ------------------------------------------------------------- primitives
 // rho, u = (rho u)/rho, ..., T from e = E - |u|^2/2 (e/c_v, or the
 // inverse of e(T) of a thermally perfect gas), p = rho R T, H = e + R T +
@@ -171,6 +193,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
   const View<double> V = view<double>(d);
   const int want_dt = block_want_dt(d, stage0);
   double sr = 0.0;
+  unsigned fe[FX_NF] = {0}, fm[FX_NMIN] = {0};
   if (q < d.n) {
     int i, j, k;
     point_of(d, q, i, j, k);
@@ -195,6 +218,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
       h = fma(d.R, T, e);
     }
     double pr = rho * d.R * T;
+    const double H = h + 0.5 * q2;
     S2_GUARD(okp) {
       V.rho[p] = rho;
       V.u[p] = u;
@@ -202,8 +226,13 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
       V.ww[p] = ww;
       V.T[p] = T;
       V.p[p] = pr;
-      V.H[p] = h + 0.5 * q2;
+      V.H[p] = H;
     }
+    const double fv[FX_NF] = {rho, T, pr, u, v, ww, H};  // by FX_*
+#pragma unroll
+    for (int f = 0; f < FX_NF; ++f) fe[f] = fx_exponent(fv[f]);
+#pragma unroll
+    for (int f = 0; f < FX_NMIN; ++f) fm[f] = 2047u - fe[f];
     double mu = 0.0;
     if (d.viscous) {
       mu = viscosity(d, T);
@@ -213,6 +242,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
       atomicOr(&d.scal->status, ERR_NONFINITE);
     if (want_dt) sr = spectral_radius<TP>(d, rho, u, v, ww, T, mu, d.eta_y[j]);
   }
+  if (d.fx) fx_block_raise(d, fe, fm);
   dt_block_max(d, sr, want_dt, B.x);
 }
 
@@ -409,9 +439,16 @@ __device__ __forceinline__ void ghost_prim_body(const Dev &__restrict__ d, const
     V.ww[dp] = ww;
     V.T[dp] = T;
     V.p[dp] = pr;
-    V.rho[dp] = pr / (K.R_gas * T);
+    const R r = pr / (K.R_gas * T);
+    V.rho[dp] = r;
     const R h = K.tp ? fma(K.R_gas, T, tp_e(K, T, rcp_pos(T))) : K.cp * T;
-    V.H[dp] = h + R(0.5) * (u * u + v * v + ww * ww);
+    const R H = h + R(0.5) * (u * u + v * v + ww * ww);
+    V.H[dp] = H;
+    if (sizeof(R) == 8 && d.fx) {  // the mirrored u, v, w and p have their interior magnitudes
+      fx_raise(d.scal, FX_RHO, fx_exponent(r));
+      fx_raise(d.scal, FX_T, fx_exponent(T));
+      fx_raise(d.scal, FX_H, fx_exponent(H));
+    }
     if (!(T > R(0))) atomicOr(&d.scal->status, ERR_NONFINITE);
   }
 }
@@ -568,6 +605,7 @@ __device__ __forceinline__ void update_body(const Dev &__restrict__ d, const Blk
       if (stage < 2) V.fln[o] = b * R[v];
     }
   }
+  if (q == 0 && d.fx) fx_clear(d.scal);
   if (stage == 2 && q == 0) {
     d.scal->t += dt;
     d.scal->nstep += 1;
@@ -687,6 +725,7 @@ template <class R>
 __global__ void __launch_bounds__(NT) k_rhs_out(Dev d, double *out) {
   long long q = (long long)blockIdx.x * NT + threadIdx.x;
   if (q >= d.n) return;
+  if (q == 0 && d.fx) fx_clear(d.scal);
   const View<R> V = view<R>(d);
   double f = d.force ? d.scal->force : 0.0;
   double fu = 0.0;
@@ -1442,6 +1481,10 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   double den = 0.0;
   for (int j = 0; j < grid->ny; ++j) den += dv[j] * (double)grid->nx * grid->nz;
   d.vol_inv = 1.0 / den;
+  // grid factors inside the range of the fixed-point path (s2_fixed.cuh)
+  auto fx_range = [](double x) { return std::fabs(x) > 0x1p-200 && std::fabs(x) < 0x1p200; };
+  d.fx = !d.mixed && fx_range(d.dx) && fx_range(d.dz);
+  for (int j = 0; j < grid->ny; ++j) d.fx = d.fx && fx_range(dv[j]);
   // initial dt
   double dt0 = scheme->cfl > 0 ? 0.0 : scheme->dt_fixed;
   cudaMemcpyAsync(&d.scal->dt, &dt0, sizeof(double), cudaMemcpyHostToDevice, s->stream);
