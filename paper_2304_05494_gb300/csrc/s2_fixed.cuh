@@ -29,8 +29,8 @@ constexpr int FX_LIMB = 30;
 constexpr int FX_MASK = (1 << FX_LIMB) - 1;
 // Biased exponents below the first are raised to it (fields that are zero
 // or tiny everywhere), those above the second take the double path.  The
-// products of three fields and a grid factor (2^-200 .. 2^200 as well) then
-// stay far inside the range of a double.
+// products of three fields and a grid factor (within 2^-100 .. 2^100, or its
+// square) then stay far inside the range of a double.
 constexpr int FX_EMIN = 1023 - 200, FX_EMAX = 1023 + 200;
 constexpr int FX_SPAN = 6;
 
@@ -86,6 +86,68 @@ __device__ __forceinline__ int2 fx_split(double x, int ex) {
 __device__ __forceinline__ long long fx_mulhi(int al, int ah, int bl, int bh) {
   const long long hl = (long long)ah * bl + (long long)al * bh;
   return (long long)ah * bh + (hl >> FX_LIMB);
+}
+
+// Central difference weights of order 2 NP over a common denominator:
+// first derivative c1(l) / D1 (l = 1..NP), second derivative c2(l) / D2
+// (l = 0..NP); W1, W2: bits of the weights' magnitudes added up.
+template <int NP>
+struct FxStencil;
+template <>
+struct FxStencil<1> {
+  static constexpr int D1 = 2, D2 = 1, W1 = 1, W2 = 2;
+  __host__ __device__ static constexpr int c1(int) { return 1; }
+  __host__ __device__ static constexpr int c2(int l) { return l == 0 ? -2 : 1; }
+};
+template <>
+struct FxStencil<2> {
+  static constexpr int D1 = 12, D2 = 12, W1 = 5, W2 = 6;
+  __host__ __device__ static constexpr int c1(int l) { return l == 1 ? 8 : -1; }
+  __host__ __device__ static constexpr int c2(int l) { return l == 0 ? -30 : (l == 1 ? 16 : -1); }
+};
+template <>
+struct FxStencil<3> {
+  static constexpr int D1 = 60, D2 = 180, W1 = 7, W2 = 11;
+  __host__ __device__ static constexpr int c1(int l) { return l == 1 ? 45 : (l == 2 ? -9 : 1); }
+  __host__ __device__ static constexpr int c2(int l) { return l == 0 ? -490 : (l == 1 ? 270 : (l == 2 ? -27 : 2)); }
+};
+template <>
+struct FxStencil<4> {
+  static constexpr int D1 = 840, D2 = 5040, W1 = 11, W2 = 15;
+  __host__ __device__ static constexpr int c1(int l) { return l == 1 ? 672 : (l == 2 ? -168 : (l == 3 ? 32 : -3)); }
+  __host__ __device__ static constexpr int c2(int l) {
+    return l == 0 ? -14350 : (l == 1 ? 8064 : (l == 2 ? -1008 : (l == 3 ? 128 : -9)));
+  }
+};
+
+// v as a double, rounded to nearest (ties away from zero), on the integer
+// unit: the conversion instruction occupies the double unit like a DFMA.
+__device__ __forceinline__ double fx_i2d(long long v) {
+  const long long s = v >> 63;
+  unsigned long long a = (unsigned long long)((v ^ s) - s);
+  const int z = __clzll((long long)a);
+  a <<= z & 63;
+  const unsigned long long m = (a >> 11) + ((a >> 10) & 1);  // bit 52 set
+  const int hi = (int)(m >> 32) + ((1023 + 62 - z) << 20);
+  return a ? __hiloint2double(hi | ((int)(v >> 32) & (int)0x80000000), (int)m) : 0.0;
+}
+
+// (hi 2^30 + lo) unit for the two 64-bit limb sums of a stencil whose
+// weights add up to less than 2^W in magnitude.  Below 2^62 the sum is
+// exact up to the result's own rounding; above (differences of the order of
+// the field's maximum) its last W - 3 bits are cut, which leaves 54 bits,
+// or 50 for the second derivative of order 8, whose terms' own rounding in
+// double precision would be 2^7 times that.
+template <bool HW, int W>
+__device__ __forceinline__ double fx_sum(long long hi, long long lo, double unit) {
+  constexpr int CUT = W > 3 ? W - 3 : 0;
+  const long long t = hi + (lo >> FX_LIMB);
+  const int r = (int)lo & FX_MASK;
+  const bool big = CUT && ((unsigned long long)(t + (1ll << 32)) >> 33) != 0;
+  const int drop = big ? CUT : 0;
+  const long long v = (t << (FX_LIMB - drop)) + (r >> drop);
+  const double u = __hiloint2double(__double2hiint(unit) + (drop << 20), __double2loint(unit));
+  return (HW ? __ll2double_rn(v) : fx_i2d(v)) * u;
 }
 
 // x 2^n, x and the result being normal.

@@ -16,7 +16,7 @@ constexpr int NV = 5;
 
 // Fields with a fixed-point exponent (s2_fixed.cuh); the first FX_NMIN also
 // record their smallest magnitude.
-enum { FX_RHO = 0, FX_T, FX_P, FX_U, FX_V, FX_W, FX_H, FX_NF };
+enum { FX_RHO = 0, FX_T, FX_P, FX_U, FX_V, FX_W, FX_H, FX_TH, FX_NF };
 constexpr int FX_NMIN = 3;
 
 // Device-side scalars of one solver.
@@ -33,9 +33,10 @@ struct Scal {
   double red[8];          // results of the last stats reduction
   // biased exponent of the largest magnitude of each field of this RHS
   // evaluation, and 2047 - that of the smallest (0: nothing seen yet); the
-  // primitive and ghost passes raise them, the pass that ends the
-  // evaluation clears them
+  // primitive, ghost and gradient passes raise them, the pass that ends
+  // the evaluation clears them
   unsigned int fx_e[FX_NF], fx_m[FX_NMIN];
+  unsigned int fx_pad;
 };
 
 // Error bits kernels OR into Scal::status (mapped on the host to
@@ -142,6 +143,10 @@ struct Dev {
   // metrics (length ny): eta_y; a_l eta_y (4/j); b_l eta_y^2 (5/j); eta_yy/eta_y; 1/eta_y
   // (a_l, b_l of the viscous order; the metric itself uses the higher order)
   const double *eta_y, *ay, *by, *ry, *dvy;
+  // units of the fixed-point stencils (s2_fixed.cuh): the derivative of an
+  // integer stencil sum, 1/(D1 h) and 1/(D2 h^2), for x and z and per row
+  const double *fy1, *fy2;
+  double fx1, fx2, fz1, fz2;
   const float *eta_yf, *ayf, *byf, *ryf;  // the same in single precision
   Scal *scal;
   double *part;            // reduction partials
@@ -675,7 +680,7 @@ unsigned weno_batch_blocks(const Dev &d, int dir);
 cudaError_t launch_flux_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const FluxMaps *maps,
                               const void *tgs, int dir, int accumulate, cudaStream_t st);
 cudaError_t launch_weno_batch(const Dev &d0, const BatchArgs &ba, unsigned total, int dir, cudaStream_t st);
-// z-marching passes of the mixed path: grid of one box (x, y, z blocks)
+// gradient and viscous passes: grid of one box (x, y, z blocks)
 void z_pass_grid(const Dev &d, unsigned g[3]);
 // Planes per CTA of the z-marching passes: compiled for 4, 8, 12, 16 and
 // 24 (the forcing partials are sized for the smallest).

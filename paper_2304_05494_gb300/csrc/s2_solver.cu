@@ -51,6 +51,7 @@ struct MetricCoef {
   double am[5], bm[5];  // metric order (the higher of the two)
   double av[5], bv[5];  // viscous order
   int lm, lv;
+  double fx_d1, fx_d2;  // its common denominators (FxStencil)
 };
 // Wray's low-storage RK3 coefficients.
 const double RK_G[3] = {8.0 / 15.0, 5.0 / 12.0, 3.0 / 4.0};
@@ -99,7 +100,7 @@ __device__ void block_sum(double *v) {
 // pre-scaled coefficient tables used by the stencil kernels, in double and
 // in single precision.
 __global__ void k_metric(const double *yn, int ny, double ly, int wall, MetricCoef mc, double *eta_y, double *ay,
-                         double *by, double *ry, double *dvy, float *eta_yf, float *ayf, float *byf, float *ryf) {
+                         double *by, double *ry, double *dvy, double *fy1, double *fy2, float *eta_yf, float *ayf, float *byf, float *ryf) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= ny) return;
   const double *a = mc.am, *b = mc.bm;
@@ -130,6 +131,8 @@ __global__ void k_metric(const double *yn, int ny, double ly, int wall, MetricCo
     by[5 * j + l] = mc.bv[l] * ey * ey;
     byf[5 * j + l] = (float)(mc.bv[l] * ey * ey);
   }
+  fy1[j] = ey / mc.fx_d1;
+  fy2[j] = ey * ey / mc.fx_d2;
   ry[j] = eyy / ey;
   ryf[j] = (float)(eyy / ey);
   dvy[j] = d1;
@@ -164,18 +167,19 @@ __device__ __forceinline__ int block_want_dt(const Dev &d, int stage0) {
 // fixed-point path.  Whole warps reduce with one instruction per value and
 // one thread per value looks at the CTA's result: 0.2 % of k_prims.
 __device__ __forceinline__ void fx_block_raise(const Dev &d, const unsigned *e, const unsigned *m) {
-  __shared__ unsigned red[FX_NF + FX_NMIN][NT / 32];
+  constexpr int NE = FX_TH;  // the fields of the primitive pass
+  __shared__ unsigned red[NE + FX_NMIN][NT / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int f = 0; f < FX_NF + FX_NMIN; ++f) {
-    const unsigned r = __reduce_max_sync(0xffffffffu, f < FX_NF ? e[f] : m[f - FX_NF]);
+  for (int f = 0; f < NE + FX_NMIN; ++f) {
+    const unsigned r = __reduce_max_sync(0xffffffffu, f < NE ? e[f] : m[f - NE]);
     if (lane == 0) red[f][wid] = r;
   }
   __syncthreads();
-  if (threadIdx.x < FX_NF + FX_NMIN) {
+  if (threadIdx.x < NE + FX_NMIN) {
     unsigned r = 0;
     for (int w = 0; w < NT / 32; ++w) r = max(r, red[threadIdx.x][w]);
-    unsigned *at = threadIdx.x < FX_NF ? &d.scal->fx_e[threadIdx.x] : &d.scal->fx_m[threadIdx.x - FX_NF];
+    unsigned *at = threadIdx.x < NE ? &d.scal->fx_e[threadIdx.x] : &d.scal->fx_m[threadIdx.x - NE];
     if (__ldcg(at) < r) atomicMax(at, r);
   }
 }
@@ -193,7 +197,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
   const View<double> V = view<double>(d);
   const int want_dt = block_want_dt(d, stage0);
   double sr = 0.0;
-  unsigned fe[FX_NF] = {0}, fm[FX_NMIN] = {0};
+  unsigned fe[FX_TH] = {0}, fm[FX_NMIN] = {0};
   if (q < d.n) {
     int i, j, k;
     point_of(d, q, i, j, k);
@@ -228,9 +232,9 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
       V.p[p] = pr;
       V.H[p] = H;
     }
-    const double fv[FX_NF] = {rho, T, pr, u, v, ww, H};  // by FX_*
+    const double fv[FX_TH] = {rho, T, pr, u, v, ww, H};  // by FX_*
 #pragma unroll
-    for (int f = 0; f < FX_NF; ++f) fe[f] = fx_exponent(fv[f]);
+    for (int f = 0; f < FX_TH; ++f) fe[f] = fx_exponent(fv[f]);
 #pragma unroll
     for (int f = 0; f < FX_NMIN; ++f) fm[f] = 2047u - fe[f];
     double mu = 0.0;
@@ -489,7 +493,9 @@ __device__ __forceinline__ void ghost_aux_body(const Dev &__restrict__ d, const 
     long long q = ((long long)sk * d.ny + sj) * d.nx + si;
     if (!S2_OK_IDX(d, q, d.n)) return;
     R ux = V.g[0 * d.n + q], vy = V.g[4 * d.n + q], wz = V.g[8 * d.n + q];
-    V.div[dp] = -ux + vy - wz;
+    const R dv = -ux + vy - wz;
+    V.div[dp] = dv;
+    if (sizeof(R) == 8 && d.fx) fx_raise(d.scal, FX_TH, fx_exponent(dv));
   }
 }
 
@@ -1383,6 +1389,7 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   // s2_rhs stages its double output in fln when that is double, else here
   s->rhs_stage = d.mixed ? A(NV * nn) : (double *)d.fln;
   double *eta = A(grid->ny), *ay = A(4 * grid->ny), *by = A(5 * grid->ny), *ry = A(grid->ny), *dvy = A(grid->ny);
+  double *fy = A(2 * grid->ny);
   float *etaf = (float *)dalloc(s, sizeof(float) * grid->ny), *ayf = (float *)dalloc(s, sizeof(float) * 4 * grid->ny);
   float *byf = (float *)dalloc(s, sizeof(float) * 5 * grid->ny), *ryf = (float *)dalloc(s, sizeof(float) * grid->ny);
   if (!etaf || !ayf || !byf || !ryf) ok = false;
@@ -1426,6 +1433,8 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.by = by;
   d.ry = ry;
   d.dvy = dvy;
+  d.fy1 = fy;
+  d.fy2 = fy + grid->ny;
   d.eta_yf = etaf;
   d.ayf = ayf;
   d.byf = byf;
@@ -1463,8 +1472,16 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
       mc.av[l] = A1_ORD[mc.lv][l];
       mc.bv[l] = B2_ORD[mc.lv][l];
     }
+    const double den1[5] = {0, FxStencil<1>::D1, FxStencil<2>::D1, FxStencil<3>::D1, FxStencil<4>::D1};
+    const double den2[5] = {0, FxStencil<1>::D2, FxStencil<2>::D2, FxStencil<3>::D2, FxStencil<4>::D2};
+    mc.fx_d1 = den1[d.npv];
+    mc.fx_d2 = den2[d.npv];
+    d.fx1 = 1.0 / (d.dx * mc.fx_d1);
+    d.fz1 = 1.0 / (d.dz * mc.fx_d1);
+    d.fx2 = 1.0 / (d.dx * d.dx * mc.fx_d2);
+    d.fz2 = 1.0 / (d.dz * d.dz * mc.fx_d2);
     k_metric<<<(grid->ny + 127) / 128, 128, 0, s->stream>>>(ynd, grid->ny, grid->ly, d.wall_y, mc, eta, ay, by, ry,
-                                                             dvy, etaf, ayf, byf, ryf);
+                                                             dvy, fy, fy + grid->ny, etaf, ayf, byf, ryf);
     e = cudaGetLastError();
   }
   std::vector<double> dv(grid->ny);
@@ -1482,7 +1499,7 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   for (int j = 0; j < grid->ny; ++j) den += dv[j] * (double)grid->nx * grid->nz;
   d.vol_inv = 1.0 / den;
   // grid factors inside the range of the fixed-point path (s2_fixed.cuh)
-  auto fx_range = [](double x) { return std::fabs(x) > 0x1p-200 && std::fabs(x) < 0x1p200; };
+  auto fx_range = [](double x) { return std::fabs(x) > 0x1p-100 && std::fabs(x) < 0x1p100; };
   d.fx = !d.mixed && fx_range(d.dx) && fx_range(d.dz);
   for (int j = 0; j < grid->ny; ++j) d.fx = d.fx && fx_range(dv[j]);
   // initial dt
@@ -1935,15 +1952,10 @@ int group_setup(BatchGroup &g) {
     const unsigned ngb = (unsigned)((nghost + NT - 1) / NT);
     set(BC_PRIMS, b, nb, 1, 1);
     set(BC_GHOST, b, ngb, 1, 1);
-    if (d.mixed) {
-      unsigned zg[3];
-      z_pass_grid(d, zg);
-      set(BC_GRAD, b, zg[0], zg[1], zg[2]);
-      set(BC_VISC, b, zg[0], zg[1], zg[2]);
-    } else {
-      set(BC_GRAD, b, nb, 1, 1);
-      set(BC_VISC, b, nb, 1, 1);
-    }
+    unsigned zg[3];
+    z_pass_grid(d, zg);
+    set(BC_GRAD, b, zg[0], zg[1], zg[2]);
+    set(BC_VISC, b, zg[0], zg[1], zg[2]);
     for (int dir = 0; dir < 3; ++dir) {
       const FluxBoxPlan &pl = plans[3 * b + dir];
       unsigned c = (unsigned)pl.tiles;

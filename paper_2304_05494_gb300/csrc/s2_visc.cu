@@ -24,6 +24,7 @@
 // (arithmetic of the mixed path).
 #include <type_traits>
 
+#include "s2_fixed.cuh"
 #include "s2_internal.cuh"
 
 namespace s2 {
@@ -225,56 +226,28 @@ __global__ void __launch_bounds__(NT) kb_apply(BatchArgs ba) {
   apply_body<R>(sd, B);
 }
 
-template <class R, int NP>
-__device__ __forceinline__ void grad_body(const Dev &__restrict__ d, const Blk &B) {
-  long long q = (long long)B.x * NT + threadIdx.x;
-  if (q >= d.n) return;
-  const View<R> V = view<R>(d);
-  int i, j, k;
-  point_of(d, q, i, j, k);
-  long long p = pidx(d, i, j, k);
-  // the stencils reach p -+ NP sz (z is the largest stride)
-  if (!(S2_OK_IDX(d, p - NP * d.sz, d.np) && S2_OK_IDX(d, p + NP * d.sz, d.np))) return;
-  C5<R> cx, cy, cz;
+// The two passes of the FP64 path at one point in double precision, for
+// fields that the fixed-point stencils below do not take: p and q are its
+// padded and interior offsets.
+template <int NP>
+__device__ __noinline__ void grad_point(const Dev &__restrict__ d, int j, long long p, double *out) {
+  const View<double> V = view<double>(d);
+  C5<double> cx, cy, cz;
   coeffs<NP>(d, V, j, cx, cy, cz);
-  const R *vel[3] = {V.u, V.v, V.ww};
-  R g[3][3];
+  const double *vel[3] = {V.u, V.v, V.ww};
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    g[a][0] = d1<NP>(vel[a], p, 1, cx);
-    g[a][1] = d1<NP>(vel[a], p, d.sy, cy);
-    g[a][2] = d1<NP>(vel[a], p, d.sz, cz);
+    out[3 * a] = d1<NP>(vel[a], p, 1, cx);
+    out[3 * a + 1] = d1<NP>(vel[a], p, d.sy, cy);
+    out[3 * a + 2] = d1<NP>(vel[a], p, d.sz, cz);
   }
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) V.g[(3 * a + b) * d.n + q] = g[a][b];
-  R th = g[0][0] + g[1][1] + g[2][2];
-  V.div[p] = th;
-  if (d.weno) V.sens[p] = sensor_test(consts<R>(d), g, th);
 }
 
-template <class R, int NP>
-__global__ void __launch_bounds__(NT) k_grad(Dev d) {
-  grad_body<R, NP>(d, grid_blk());
-}
-
-template <class R, int NP>
-__global__ void __launch_bounds__(NT) kb_grad(BatchArgs ba) {
-  S2_BATCH_ENTER(ba, sd, B, b_box);
-  grad_body<R, NP>(sd, B);
-}
-
-template <class R, int NP>
-__device__ __forceinline__ void visc_body(const Dev &__restrict__ d, const Blk &B) {
-  long long q = (long long)B.x * NT + threadIdx.x;
-  if (q >= d.n) return;
+template <int NP>
+__device__ __noinline__ void visc_point(const Dev &__restrict__ d, int j, long long p, long long q, double *Rv) {
+  using R = double;
   const View<R> V = view<R>(d);
   const Consts<R> &K = consts<R>(d);
-  int i, j, k;
-  point_of(d, q, i, j, k);
-  long long p = pidx(d, i, j, k);
-  if (!(S2_OK_IDX(d, p - NP * d.sz, d.np) && S2_OK_IDX(d, p + NP * d.sz, d.np))) return;
   C5<R> cx, cy, cz, bx, by, bz;
   coeffs<NP>(d, V, j, cx, cy, cz);
 #pragma unroll
@@ -306,26 +279,311 @@ __device__ __forceinline__ void visc_body(const Dev &__restrict__ d, const Blk &
   const R uv[3] = {__ldg(V.u + p), __ldg(V.v + p), __ldg(V.ww + p)};
   R mom[3], en;
   visc_terms(K, g, lap, gT, lapT, gth, __ldg(V.T + p), __ldg(V.mu + q), __ldg(V.div + p), uv, mom, en);
-  R Rv[NV];
-  Rv[0] = V.fl[q];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) Rv[1 + a] = V.fl[(1 + a) * d.n + q] + mom[a];
-  Rv[4] = V.fl[4 * d.n + q] + en;
+  for (int a = 0; a < 3; ++a) Rv[1 + a] += mom[a];
+  Rv[4] += en;
+}
+
+// --------------------------------------- fixed-point passes (FP64 path)
+// The stencil sums of the gradient and viscous passes in 59-bit fixed point
+// (s2_fixed.cuh).  A CTA owns a 32 x 8 tile of one z-plane: the fields are
+// converted once into shared memory with an NP-point x-y halo; the 2 NP
+// neighbours along z are read from memory (L2) and converted by the thread
+// that needs them.  One plane per CTA keeps small boxes spread over the
+// chip; the double unit stays the bound of the viscous pass, so the
+// repeated conversions along z cost nothing there.
+constexpr int FTX = 32, FTY = 8;
+
+template <int NP>
+struct FxTile {
+  static constexpr int SX = FTX + 2 * NP, SIZE = SX * (FTY + 2 * NP);
+};
+
+// Fields src[0..NF-1] of plane k around (x0, y0) into sm as limbs.
+template <int NP, int NF>
+__device__ __forceinline__ void fx_stage(const Dev &d, const double *const (&src)[NF], const int *e, int x0, int y0,
+                                         int k, int2 (*sm)[FxTile<NP>::SIZE]) {
+  constexpr int SX = FxTile<NP>::SX, SIZE = FxTile<NP>::SIZE;
+#pragma unroll
+  for (int s = 0; s < (SIZE + NT - 1) / NT; ++s) {
+    const int pos = threadIdx.x + s * NT, hy = pos / SX, hx = pos - hy * SX;
+    const int i = x0 - NP + hx, j = y0 - NP + hy;
+    if (pos < SIZE && i < d.nx + GH && j < d.ny + GH) {
+      const long long p = pidx(d, i, j, k);
+      if (S2_OK_IDX(d, p, d.np)) {
+        double x[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) x[f] = __ldg(src[f] + p);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) sm[f][pos] = fx_split(x[f], e[f]);
+      }
+    }
+  }
+}
+
+// Limb sums of the first and second derivative along one direction from the
+// neighbours up[l-1] = f_{+l} and dn[l-1] = f_{-l}.
+template <int NP, bool HW>
+__device__ __forceinline__ double fx_d1(const int2 (&up)[NP], const int2 (&dn)[NP], double unit) {
+  using S = FxStencil<NP>;
+  long long hi = 0, lo = 0;
+#pragma unroll
+  for (int l = 1; l <= NP; ++l) {
+    hi += (long long)S::c1(l) * (up[l - 1].y - dn[l - 1].y);
+    lo += (long long)S::c1(l) * (up[l - 1].x - dn[l - 1].x);
+  }
+  return fx_sum<HW, S::W1>(hi, lo, unit);
+}
+
+template <int NP, bool HW>
+__device__ __forceinline__ double fx_d2(int2 c, const int2 (&up)[NP], const int2 (&dn)[NP], double unit) {
+  using S = FxStencil<NP>;
+  long long hi = (long long)S::c2(0) * c.y, lo = (long long)S::c2(0) * c.x;
+#pragma unroll
+  for (int l = 1; l <= NP; ++l) {
+    hi += (long long)S::c2(l) * (up[l - 1].y + dn[l - 1].y);
+    lo += (long long)S::c2(l) * (up[l - 1].x + dn[l - 1].x);
+  }
+  return fx_sum<HW, S::W2>(hi, lo, unit);
+}
+
+// Neighbours along x (step 1) or y (step SX) in shared memory, along z in
+// memory.
+template <int NP>
+__device__ __forceinline__ void fx_near(const int2 *S, int step, int2 (&up)[NP], int2 (&dn)[NP]) {
+#pragma unroll
+  for (int l = 1; l <= NP; ++l) {
+    up[l - 1] = S[l * step];
+    dn[l - 1] = S[-l * step];
+  }
+}
+template <int NP>
+__device__ __forceinline__ void fx_near_z(const double *f, long long sz, int e, int2 (&up)[NP], int2 (&dn)[NP]) {
+  double a[NP], b[NP];
+#pragma unroll
+  for (int l = 1; l <= NP; ++l) {
+    a[l - 1] = __ldg(f + l * sz);
+    b[l - 1] = __ldg(f - l * sz);
+  }
+#pragma unroll
+  for (int l = 1; l <= NP; ++l) {
+    up[l - 1] = fx_split(a[l - 1], e);
+    dn[l - 1] = fx_split(b[l - 1], e);
+  }
+}
+
+// Velocity gradients (stored), theta = div u and the sensor test.  Bound by
+// the integer unit; the 9 conversions go to the double unit beside it.
+template <int NP>
+__device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Blk &B) {
+  constexpr int SX = FxTile<NP>::SX;
+  __shared__ int2 sm[3][FxTile<NP>::SIZE];
+  __shared__ int ex[4];  // exponents of u, v, w; fixed point or not
+  __shared__ unsigned red[NT / 32];
+  const View<double> V = view<double>(d);
+  const int tid = threadIdx.x, x0 = B.x * FTX, y0 = B.y * FTY, k = B.z;
+  const int i = x0 + tid % FTX, j = y0 + tid / FTX;
+  if (tid == 0) {
+    const FxScale fx = fx_scale(d);
+    ex[0] = fx.e[FX_U];
+    ex[1] = fx.e[FX_V];
+    ex[2] = fx.e[FX_W];
+    ex[3] = fx.ok;
+  }
+  __syncthreads();
+  const double *vel[3] = {V.u, V.v, V.ww};
+  if (ex[3]) fx_stage<NP, 3>(d, vel, ex, x0, y0, k, sm);
+  __syncthreads();
+  unsigned eth = 0;
+  const long long p = pidx(d, i, j, k), q = ((long long)k * d.ny + j) * d.nx + i;
+  // the stencils reach p -+ NP sz (z is the largest stride)
+  if (i < d.nx && j < d.ny && S2_OK_IDX(d, p - NP * d.sz, d.np) && S2_OK_IDX(d, p + NP * d.sz, d.np)) {
+    double g[3][3];
+    if (ex[3]) {
+      const double uy = __ldg(d.fy1 + j);
+      const int c = (tid / FTX + NP) * SX + tid % FTX + NP;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int n = ex[a] - 1022 - 59;  // unit 2^(E - 59)
+        int2 up[NP], dn[NP];
+        fx_near<NP>(sm[a] + c, 1, up, dn);
+        g[a][0] = fx_d1<NP, true>(up, dn, fx_ldexp(d.fx1, n));
+        fx_near<NP>(sm[a] + c, SX, up, dn);
+        g[a][1] = fx_d1<NP, true>(up, dn, fx_ldexp(uy, n));
+        fx_near_z<NP>(vel[a] + p, d.sz, ex[a], up, dn);
+        g[a][2] = fx_d1<NP, true>(up, dn, fx_ldexp(d.fz1, n));
+      }
+    } else {
+      grad_point<NP>(d, j, p, &g[0][0]);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) V.g[(3 * a + b) * d.n + q] = g[a][b];
+    const double th = g[0][0] + g[1][1] + g[2][2];
+    V.div[p] = th;
+    eth = (unsigned)fx_exponent(th);
+    if (d.weno) V.sens[p] = sensor_test(consts<double>(d), g, th);
+  }
+  if (d.fx) {
+    const unsigned r = __reduce_max_sync(0xffffffffu, eth);
+    if ((tid & 31) == 0) red[tid >> 5] = r;
+    __syncthreads();
+    if (tid == 0) {
+      for (int w = 0; w < NT / 32; ++w) eth = max(eth, red[w]);
+      fx_raise(d.scal, FX_TH, (int)eth);
+    }
+  }
+}
+
+// Viscous and heat-flux terms, plus the WENO corrections.  With the stress
+// tensor tau and psi = (omega / T) grad T, each term is mu times
+//   X_a = lap u_a + d_a theta / 3 + psi_b tau_ab / mu   (momentum a)
+//   u_a X_a + tau_ab d_b u_a / mu + (c_p / Pr) (lap T + psi . grad T)
+// so mu enters with the sum into the RHS: 63 double operations per point at
+// order 6 (169 when the stencils were in double precision too).
+template <int NP>
+__device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Blk &B) {
+  constexpr int SX = FxTile<NP>::SX, NF = 5;
+  __shared__ int2 sm[NF][FxTile<NP>::SIZE];
+  __shared__ int ex[NF + 1];  // exponents of u, v, w, T, theta; fixed point or not
+  const View<double> V = view<double>(d);
+  const Consts<double> &K = d.kd;
+  const int tid = threadIdx.x, x0 = B.x * FTX, y0 = B.y * FTY, k = B.z;
+  const int i = x0 + tid % FTX, j = y0 + tid / FTX;
+  if (tid == 0) {
+    const FxScale fx = fx_scale(d);
+    ex[0] = fx.e[FX_U];
+    ex[1] = fx.e[FX_V];
+    ex[2] = fx.e[FX_W];
+    ex[3] = fx.e[FX_T];
+    ex[4] = fx.e[FX_TH];
+    ex[5] = fx.ok;
+  }
+  __syncthreads();
+  const double *src[NF] = {V.u, V.v, V.ww, V.T, V.div};
+  if (ex[5]) fx_stage<NP, NF>(d, src, ex, x0, y0, k, sm);
+  __syncthreads();
+  if (i >= d.nx || j >= d.ny) return;
+  const long long p = pidx(d, i, j, k), q = ((long long)k * d.ny + j) * d.nx + i;
+  if (!(S2_OK_IDX(d, p - NP * d.sz, d.np) && S2_OK_IDX(d, p + NP * d.sz, d.np))) return;
+  double Rv[NV];
+#pragma unroll
+  for (int f = 0; f < NV; ++f) Rv[f] = V.fl[f * d.n + q];
+  if (ex[5]) {
+    const int c = (tid / FTX + NP) * SX + tid % FTX + NP;
+    const double uy1 = __ldg(d.fy1 + j), uy2 = __ldg(d.fy2 + j), ry = __ldg(V.ry + j);
+    const double mu = __ldg(V.mu + q), T = __ldg(V.T + p), th = __ldg(V.div + p);
+    int2 up[NP], dn[NP];
+    // Laplacians of u, v, w, T; gradients of T and theta (a third of it)
+    double lap[4], gT[3], gth[3];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const int n = ex[f] - 1022 - 59;
+      const int2 *S = sm[f] + c;
+      fx_near<NP>(S, 1, up, dn);
+      if (f < 4) lap[f] = fx_d2<NP, false>(S[0], up, dn, fx_ldexp(d.fx2, n));
+      if (f == 3) gT[0] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fx1, n));
+      if (f == 4) gth[0] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fx1, n));
+      fx_near<NP>(S, SX, up, dn);
+      if (f < 4) lap[f] += fx_d2<NP, false>(S[0], up, dn, fx_ldexp(uy2, n));
+      if (f == 3) gT[1] = fx_d1<NP, false>(up, dn, fx_ldexp(uy1, n));
+      if (f == 4) gth[1] = fx_d1<NP, false>(up, dn, fx_ldexp(uy1, n));
+      fx_near_z<NP>(src[f] + p, d.sz, ex[f], up, dn);
+      if (f < 4) lap[f] += fx_d2<NP, false>(S[0], up, dn, fx_ldexp(d.fz2, n));
+      if (f == 3) gT[2] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fz1, n));
+      if (f == 4) gth[2] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fz1, n));
+    }
+    double g[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) g[a][b] = __ldg(V.g + (3 * a + b) * d.n + q);
+    // d2/dy2 = eta_y^2 d2/deta2 + eta_yy d/deta
+    lap[3] = fma(ry, gT[1], lap[3]);
+    const double wT = K.visc_exp * rcp_pos(T);
+    const double psi[3] = {wT * gT[0], wT * gT[1], wT * gT[2]};
+    const double tq = (2.0 / 3.0) * th;
+    double dg[3], X[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) dg[a] = fma(2.0, g[a][a], -tq);
+    const double s01 = g[0][1] + g[1][0], s02 = g[0][2] + g[2][0], s12 = g[1][2] + g[2][1];
+    const double so[3][3] = {{0.0, s01, s02}, {s01, 0.0, s12}, {s02, s12, 0.0}};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      double x = fma(ry, g[a][1], lap[a]);
+      x = fma(gth[a], 1.0 / 3.0, x);
+      x = fma(psi[a], dg[a], x);
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        if (b != a) x = fma(psi[b], so[a][b], x);
+      X[a] = x;
+      Rv[1 + a] = fma(mu, x, Rv[1 + a]);
+    }
+    double e = dg[0] * g[0][0];
+    e = fma(dg[1], g[1][1], e);
+    e = fma(dg[2], g[2][2], e);
+    e = fma(s01, s01, e);
+    e = fma(s02, s02, e);
+    e = fma(s12, s12, e);
+    double h = lap[3];
+    double cpr = K.cp_over_pr;
+    if (K.tp) {
+      // k = mu c_p(T)/Pr: grad k . grad T gains mu (c_p'(T)/Pr) |grad T|^2
+      const double rT = rcp_pos(T);
+      cpr = tp_cp(K, T, rT) * K.inv_pr;
+      const double gT2 = fma(gT[2], gT[2], fma(gT[1], gT[1], gT[0] * gT[0]));
+      e = fma(tp_dcp(K, T, rT) * K.inv_pr, gT2, e);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) h = fma(psi[b], gT[b], h);
+    e = fma(cpr, h, e);
+    e = fma(__ldg(V.u + p), X[0], e);
+    e = fma(__ldg(V.v + p), X[1], e);
+    e = fma(__ldg(V.ww + p), X[2], e);
+    Rv[4] = fma(mu, e, Rv[4]);
+  } else {
+    visc_point<NP>(d, j, p, q, Rv);
+  }
   if (d.weno) weno_correction(d, V, i, j, k, Rv);
   if (d.weno) V.fl[q] = Rv[0];
 #pragma unroll
   for (int f = 1; f < NV; ++f) V.fl[f * d.n + q] = Rv[f];
 }
 
-template <class R, int NP>
-__global__ void __launch_bounds__(NT) k_visc(Dev d) {
-  visc_body<R, NP>(d, grid_blk());
+// One CTA per tile and plane on a linear grid (no extent of a grid
+// dimension limits the box).
+__device__ __forceinline__ Blk fx_blk(const Dev &d) {
+  Blk B = grid_blk();
+  B.nx = (d.nx + FTX - 1) / FTX;
+  B.ny = (d.ny + FTY - 1) / FTY;
+  const unsigned l = B.x, r = l / B.nx;
+  B.x = l - r * B.nx;
+  B.z = r / B.ny;
+  B.y = r - B.z * B.ny;
+  return B;
 }
 
-template <class R, int NP>
-__global__ void __launch_bounds__(NT) kb_visc(BatchArgs ba) {
+template <int NP>
+__global__ void __launch_bounds__(NT, 3) k_grad(const __grid_constant__ Dev d) {
+  grad_fx_body<NP>(d, fx_blk(d));
+}
+
+template <int NP>
+__global__ void __launch_bounds__(NT, 3) kb_grad(BatchArgs ba) {
   S2_BATCH_ENTER(ba, sd, B, b_box);
-  visc_body<R, NP>(sd, B);
+  grad_fx_body<NP>(sd, B);
+}
+
+template <int NP>
+__global__ void __launch_bounds__(NT, 2) k_visc(const __grid_constant__ Dev d) {
+  visc_fx_body<NP>(d, fx_blk(d));
+}
+
+template <int NP>
+__global__ void __launch_bounds__(NT, 2) kb_visc(BatchArgs ba) {
+  S2_BATCH_ENTER(ba, sd, B, b_box);
+  visc_fx_body<NP>(sd, B);
 }
 
 // ------------------------------------------------ z-marching (mixed path)
@@ -668,23 +926,28 @@ __global__ void __launch_bounds__(NT, 2) kb_visc_z(BatchArgs ba) {
 }
 
 
-template <class R>
-void grad_np(const Dev &d, unsigned nb, cudaStream_t st) {
+// Linear grid of the FP64 gradient and viscous passes.
+unsigned fx_blocks(const Dev &d) {
+  return (unsigned)(((d.nx + FTX - 1) / FTX) * (long long)((d.ny + FTY - 1) / FTY) * d.nz);
+}
+
+void grad_np(const Dev &d, cudaStream_t st) {
+  const unsigned nb = fx_blocks(d);
   switch (d.npv) {
-    case 1: k_grad<R, 1><<<nb, NT, 0, st>>>(d); break;
-    case 2: k_grad<R, 2><<<nb, NT, 0, st>>>(d); break;
-    case 3: k_grad<R, 3><<<nb, NT, 0, st>>>(d); break;
-    default: k_grad<R, 4><<<nb, NT, 0, st>>>(d); break;
+    case 1: k_grad<1><<<nb, NT, 0, st>>>(d); break;
+    case 2: k_grad<2><<<nb, NT, 0, st>>>(d); break;
+    case 3: k_grad<3><<<nb, NT, 0, st>>>(d); break;
+    default: k_grad<4><<<nb, NT, 0, st>>>(d); break;
   }
 }
 
-template <class R>
-void visc_np(const Dev &d, unsigned nb, cudaStream_t st) {
+void visc_np(const Dev &d, cudaStream_t st) {
+  const unsigned nb = fx_blocks(d);
   switch (d.npv) {
-    case 1: k_visc<R, 1><<<nb, NT, 0, st>>>(d); break;
-    case 2: k_visc<R, 2><<<nb, NT, 0, st>>>(d); break;
-    case 3: k_visc<R, 3><<<nb, NT, 0, st>>>(d); break;
-    default: k_visc<R, 4><<<nb, NT, 0, st>>>(d); break;
+    case 1: k_visc<1><<<nb, NT, 0, st>>>(d); break;
+    case 2: k_visc<2><<<nb, NT, 0, st>>>(d); break;
+    case 3: k_visc<3><<<nb, NT, 0, st>>>(d); break;
+    default: k_visc<4><<<nb, NT, 0, st>>>(d); break;
   }
 }
 
@@ -708,7 +971,6 @@ static dim3 zgrid(const Dev &d) {
 }
 
 cudaError_t launch_grad(const Dev &d, cudaStream_t st) {
-  unsigned nb = (unsigned)((d.n + NT - 1) / NT);
   if (d.mixed) {
     switch (d.npv) {
       case 1: z_launch<1>([&](auto zs) { k_grad_z<1, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
@@ -717,7 +979,7 @@ cudaError_t launch_grad(const Dev &d, cudaStream_t st) {
       default: z_launch<4>([&](auto zs) { k_grad_z<4, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
     }
   } else {
-    grad_np<double>(d, nb, st);
+    grad_np(d, st);
   }
   return cudaGetLastError();
 }
@@ -741,9 +1003,9 @@ int visc_force_partials(const Dev &d) {
 
 void z_pass_grid(const Dev &d, unsigned g[3]) {
   const dim3 z = zgrid(d);
-  g[0] = z.x;
-  g[1] = z.y;
-  g[2] = z.z;
+  g[0] = d.mixed ? z.x : (d.nx + FTX - 1) / FTX;
+  g[1] = d.mixed ? z.y : (d.ny + FTY - 1) / FTY;
+  g[2] = d.mixed ? z.z : d.nz;
 }
 
 // Batched: every box of a batch group in one launch (instantiation of d0).
@@ -757,10 +1019,10 @@ cudaError_t launch_grad_batch(const Dev &d0, const BatchArgs &ba, unsigned total
     }
   } else {
     switch (d0.npv) {
-      case 1: kb_grad<double, 1><<<total, NT, 0, st>>>(ba); break;
-      case 2: kb_grad<double, 2><<<total, NT, 0, st>>>(ba); break;
-      case 3: kb_grad<double, 3><<<total, NT, 0, st>>>(ba); break;
-      default: kb_grad<double, 4><<<total, NT, 0, st>>>(ba); break;
+      case 1: kb_grad<1><<<total, NT, 0, st>>>(ba); break;
+      case 2: kb_grad<2><<<total, NT, 0, st>>>(ba); break;
+      case 3: kb_grad<3><<<total, NT, 0, st>>>(ba); break;
+      default: kb_grad<4><<<total, NT, 0, st>>>(ba); break;
     }
   }
   return cudaGetLastError();
@@ -776,10 +1038,10 @@ cudaError_t launch_visc_batch(const Dev &d0, const BatchArgs &ba, unsigned total
     }
   } else {
     switch (d0.npv) {
-      case 1: kb_visc<double, 1><<<total, NT, 0, st>>>(ba); break;
-      case 2: kb_visc<double, 2><<<total, NT, 0, st>>>(ba); break;
-      case 3: kb_visc<double, 3><<<total, NT, 0, st>>>(ba); break;
-      default: kb_visc<double, 4><<<total, NT, 0, st>>>(ba); break;
+      case 1: kb_visc<1><<<total, NT, 0, st>>>(ba); break;
+      case 2: kb_visc<2><<<total, NT, 0, st>>>(ba); break;
+      case 3: kb_visc<3><<<total, NT, 0, st>>>(ba); break;
+      default: kb_visc<4><<<total, NT, 0, st>>>(ba); break;
     }
   }
   return cudaGetLastError();
@@ -792,7 +1054,6 @@ cudaError_t launch_apply_batch(const Dev &d0, const BatchArgs &ba, unsigned tota
 }
 
 cudaError_t launch_visc(const Dev &d, cudaStream_t st) {
-  unsigned nb = (unsigned)((d.n + NT - 1) / NT);
   if (d.mixed) {
     switch (d.npv) {
       case 1: z_launch<1>([&](auto zs) { k_visc_z<1, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
@@ -801,7 +1062,7 @@ cudaError_t launch_visc(const Dev &d, cudaStream_t st) {
       default: z_launch<4>([&](auto zs) { k_visc_z<4, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
     }
   } else {
-    visc_np<double>(d, nb, st);
+    visc_np(d, st);
   }
   return cudaGetLastError();
 }
