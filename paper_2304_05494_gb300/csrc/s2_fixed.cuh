@@ -120,35 +120,55 @@ struct FxStencil<4> {
   }
 };
 
-// v as a double, rounded to nearest (ties away from zero), on the integer
-// unit: the conversion instruction occupies the double unit like a DFMA.
-__device__ __forceinline__ double fx_i2d(long long v) {
+// v 2^n as a double, rounded to nearest (ties away from zero), on the
+// integer unit: the conversion instruction occupies the double unit like a
+// DFMA.
+__device__ __forceinline__ double fx_i2d(long long v, int n = 0) {
   const long long s = v >> 63;
   unsigned long long a = (unsigned long long)((v ^ s) - s);
   const int z = __clzll((long long)a);
   a <<= z & 63;
   const unsigned long long m = (a >> 11) + ((a >> 10) & 1);  // bit 52 set
-  const int hi = (int)(m >> 32) + ((1023 + 62 - z) << 20);
+  const int hi = (int)(m >> 32) + (1023 + 62 - z + n) * (1 << 20);
   return a ? __hiloint2double(hi | ((int)(v >> 32) & (int)0x80000000), (int)m) : 0.0;
 }
 
-// (hi 2^30 + lo) unit for the two 64-bit limb sums of a stencil whose
-// weights add up to less than 2^W in magnitude.  Below 2^62 the sum is
-// exact up to the result's own rounding; above (differences of the order of
-// the field's maximum) its last W - 3 bits are cut, which leaves 54 bits,
-// or 50 for the second derivative of order 8, whose terms' own rounding in
-// double precision would be 2^7 times that.
-template <bool HW, int W>
-__device__ __forceinline__ double fx_sum(long long hi, long long lo, double unit) {
+// The limb sums hi 2^30 + lo of a stencil whose weights add up to less than
+// 2^W in magnitude, as an integer times 2^drop.  Below 2^62 the sum is
+// exact; above (differences of the order of the field's maximum) its last
+// W - 3 bits are cut, which leaves at least 54 bits for first derivatives
+// and for Laplacians at least the accuracy of a double-precision sum, whose
+// terms are rounded at 2^(W-2-53) of the field's maximum.
+template <int W>
+__device__ __forceinline__ long long fx_sum(long long hi, long long lo, int &drop) {
   constexpr int CUT = W > 3 ? W - 3 : 0;
   const long long t = hi + (lo >> FX_LIMB);
   const int r = (int)lo & FX_MASK;
-  const bool big = CUT && ((unsigned long long)(t + (1ll << 32)) >> 33) != 0;
-  const int drop = big ? CUT : 0;
-  const long long v = (t << (FX_LIMB - drop)) + (r >> drop);
-  const double u = __hiloint2double(__double2hiint(unit) + (drop << 20), __double2loint(unit));
-  return (HW ? __ll2double_rn(v) : fx_i2d(v)) * u;
+  drop = CUT && ((unsigned long long)(t + (1ll << 32)) >> 33) != 0 ? CUT : 0;
+  return (t << (FX_LIMB - drop)) + (r >> drop);
 }
+
+// Weighted sum of stencil sums (the directions of a Laplacian): each limb
+// sum times a 60-bit fraction k, collected by powers of 2^30.
+struct FxAcc {
+  long long hi = 0, lo = 0, m = 0;
+  __device__ __forceinline__ void add(long long shi, long long slo, int2 k) {
+    const long long t = shi + (slo >> FX_LIMB);
+    const int r = (int)slo & FX_MASK, t0 = (int)t & FX_MASK, t1 = (int)(t >> FX_LIMB);
+    hi += (long long)t1 * k.y;
+    lo += (long long)t1 * k.x;
+    lo += (long long)t0 * k.y;
+    m += (long long)t0 * k.x;
+    m += (long long)r * k.y;
+  }
+};
+
+// Weights 1/(D2 h^2) of the three directions in one row of the grid, as
+// 60-bit fractions of 2^n.
+struct __align__(16) FxLap {
+  int2 x, y, z;
+  int n, pad;
+};
 
 // x 2^n, x and the result being normal.
 __device__ __forceinline__ double fx_ldexp(double x, int n) {

@@ -192,9 +192,9 @@ __device__ __forceinline__ void keep_pairs_tile(const R *S, R *TP, R gm1, int n)
 // Double precision, split form: the pair mass fluxes and the flux
 // difference in fixed point (s2_fixed.cuh).  Per point of an order-6 flux
 // the double unit executed 61 operations (64 issue clocks each); here it
-// executes 17 (five conversions, the pressure difference, the sums into the
-// RHS), the integer unit the rest beside them.  On 420 x 250 x 320 points a
-// launch went from 3.85 / 3.70 / 3.64 ms (x / y / z) to 1.33 / 1.28 / 1.29.
+// executes 12 (the pressure difference and the sums into the RHS), the
+// integer unit the rest beside them.  On 420 x 250 x 320 points a launch
+// went from 3.85 / 3.70 / 3.64 ms (x / y / z) to 1.28 / 1.25 / 1.27.
 // With the double unit no longer the bound, the persistent grid that
 // prefetches the next tile pays here too: with one tile per CTA the same
 // arithmetic took 2.67 / 2.77 / 2.72 ms (waiting at barriers and for the
@@ -271,7 +271,7 @@ __device__ __forceinline__ void fx_flux_point(const int2 *S, const int2 *TP, int
     Ml &= FX_MASK;
   }
   const int eM = e[F_RHO] + e[F_U + DIR] - 2 * 1022 - 59;  // unit of m
-  const double M = __ll2double_rn((long long)Mh * (1 << FX_LIMB) + Ml);
+  const double M = fx_i2d((long long)Mh * (1 << FX_LIMB) + Ml);
   out[0] = fma(-fx_ldexp(scale, eM + 1), M, prev[0]);
 #pragma unroll
   for (int f = 1; f < 5; ++f) {
@@ -289,7 +289,7 @@ __device__ __forceinline__ void fx_flux_point(const int2 *S, const int2 *TP, int
       B += (long long)mm[l - 1].y * vm.x;
       B += (long long)mm[l - 1].x * vm.y;
     }
-    const double D = __ll2double_rn(A + (B >> FX_LIMB));
+    const double D = fx_i2d(A + (B >> FX_LIMB));
     // unit of D: 2^60 times the units of m and phi
     const int eD = eM + e[f] - 1022 + 1;
     double r = fma(-fx_ldexp(scale, eD), D, prev[f]);

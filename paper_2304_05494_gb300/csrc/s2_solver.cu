@@ -52,6 +52,7 @@ struct MetricCoef {
   double av[5], bv[5];  // viscous order
   int lm, lv;
   double fx_d1, fx_d2;  // its common denominators (FxStencil)
+  double fx_x2, fx_z2;  // 1/(D2 dx^2), 1/(D2 dz^2)
 };
 // Wray's low-storage RK3 coefficients.
 const double RK_G[3] = {8.0 / 15.0, 5.0 / 12.0, 3.0 / 4.0};
@@ -100,7 +101,7 @@ __device__ void block_sum(double *v) {
 // pre-scaled coefficient tables used by the stencil kernels, in double and
 // in single precision.
 __global__ void k_metric(const double *yn, int ny, double ly, int wall, MetricCoef mc, double *eta_y, double *ay,
-                         double *by, double *ry, double *dvy, double *fy1, double *fy2, float *eta_yf, float *ayf, float *byf, float *ryf) {
+                         double *by, double *ry, double *dvy, double *fy1, FxLap *fxl, float *eta_yf, float *ayf, float *byf, float *ryf) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= ny) return;
   const double *a = mc.am, *b = mc.bm;
@@ -132,7 +133,20 @@ __global__ void k_metric(const double *yn, int ny, double ly, int wall, MetricCo
     byf[5 * j + l] = (float)(mc.bv[l] * ey * ey);
   }
   fy1[j] = ey / mc.fx_d1;
-  fy2[j] = ey * ey / mc.fx_d2;
+  // Laplacian weights of the row as 60-bit fractions of the power of two
+  // above the largest
+  const double wt[3] = {mc.fx_x2, ey * ey / mc.fx_d2, mc.fx_z2};
+  int n = 0;
+  frexp(fmax(fmax(wt[0], wt[1]), wt[2]), &n);
+  int2 k[3];
+  for (int c = 0; c < 3; ++c) {
+    const long long q = (long long)ldexp(wt[c], 60 - n);
+    k[c] = make_int2((int)q & FX_MASK, (int)(q >> FX_LIMB));
+  }
+  fxl[j].x = k[0];
+  fxl[j].y = k[1];
+  fxl[j].z = k[2];
+  fxl[j].n = n;
   ry[j] = eyy / ey;
   ryf[j] = (float)(eyy / ey);
   dvy[j] = d1;
@@ -1389,7 +1403,9 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   // s2_rhs stages its double output in fln when that is double, else here
   s->rhs_stage = d.mixed ? A(NV * nn) : (double *)d.fln;
   double *eta = A(grid->ny), *ay = A(4 * grid->ny), *by = A(5 * grid->ny), *ry = A(grid->ny), *dvy = A(grid->ny);
-  double *fy = A(2 * grid->ny);
+  double *fy = A(grid->ny);
+  FxLap *fxl = (FxLap *)dalloc(s, sizeof(FxLap) * grid->ny);
+  if (!fxl) ok = false;
   float *etaf = (float *)dalloc(s, sizeof(float) * grid->ny), *ayf = (float *)dalloc(s, sizeof(float) * 4 * grid->ny);
   float *byf = (float *)dalloc(s, sizeof(float) * 5 * grid->ny), *ryf = (float *)dalloc(s, sizeof(float) * grid->ny);
   if (!etaf || !ayf || !byf || !ryf) ok = false;
@@ -1434,7 +1450,7 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.ry = ry;
   d.dvy = dvy;
   d.fy1 = fy;
-  d.fy2 = fy + grid->ny;
+  d.fxl = fxl;
   d.eta_yf = etaf;
   d.ayf = ayf;
   d.byf = byf;
@@ -1478,10 +1494,10 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
     mc.fx_d2 = den2[d.npv];
     d.fx1 = 1.0 / (d.dx * mc.fx_d1);
     d.fz1 = 1.0 / (d.dz * mc.fx_d1);
-    d.fx2 = 1.0 / (d.dx * d.dx * mc.fx_d2);
-    d.fz2 = 1.0 / (d.dz * d.dz * mc.fx_d2);
+    mc.fx_x2 = 1.0 / (d.dx * d.dx * mc.fx_d2);
+    mc.fx_z2 = 1.0 / (d.dz * d.dz * mc.fx_d2);
     k_metric<<<(grid->ny + 127) / 128, 128, 0, s->stream>>>(ynd, grid->ny, grid->ly, d.wall_y, mc, eta, ay, by, ry,
-                                                             dvy, fy, fy + grid->ny, etaf, ayf, byf, ryf);
+                                                             dvy, fy, fxl, etaf, ayf, byf, ryf);
     e = cudaGetLastError();
   }
   std::vector<double> dv(grid->ny);

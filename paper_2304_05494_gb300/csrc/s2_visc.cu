@@ -290,8 +290,9 @@ __device__ __noinline__ void visc_point(const Dev &__restrict__ d, int j, long l
 // converted once into shared memory with an NP-point x-y halo; the 2 NP
 // neighbours along z are read from memory (L2) and converted by the thread
 // that needs them.  One plane per CTA keeps small boxes spread over the
-// chip; the double unit stays the bound of the viscous pass, so the
-// repeated conversions along z cost nothing there.
+// chip.  On 420 x 250 x 320 points at order 6 a launch of the gradient pass
+// went from 3.53 to 1.75 ms (double and integer unit both near 3/4 busy),
+// of the viscous pass from 10.33 to 3.95 ms (double unit).
 constexpr int FTX = 32, FTY = 8;
 
 template <int NP>
@@ -332,11 +333,13 @@ __device__ __forceinline__ double fx_d1(const int2 (&up)[NP], const int2 (&dn)[N
     hi += (long long)S::c1(l) * (up[l - 1].y - dn[l - 1].y);
     lo += (long long)S::c1(l) * (up[l - 1].x - dn[l - 1].x);
   }
-  return fx_sum<HW, S::W1>(hi, lo, unit);
+  int drop;
+  const long long v = fx_sum<S::W1>(hi, lo, drop);
+  return (HW ? __ll2double_rn(v) : fx_i2d(v)) * fx_ldexp(unit, drop);
 }
 
-template <int NP, bool HW>
-__device__ __forceinline__ double fx_d2(int2 c, const int2 (&up)[NP], const int2 (&dn)[NP], double unit) {
+template <int NP>
+__device__ __forceinline__ void fx_d2(FxAcc &acc, int2 c, const int2 (&up)[NP], const int2 (&dn)[NP], int2 k) {
   using S = FxStencil<NP>;
   long long hi = (long long)S::c2(0) * c.y, lo = (long long)S::c2(0) * c.x;
 #pragma unroll
@@ -344,7 +347,7 @@ __device__ __forceinline__ double fx_d2(int2 c, const int2 (&up)[NP], const int2
     hi += (long long)S::c2(l) * (up[l - 1].y + dn[l - 1].y);
     lo += (long long)S::c2(l) * (up[l - 1].x + dn[l - 1].x);
   }
-  return fx_sum<HW, S::W2>(hi, lo, unit);
+  acc.add(hi, lo, k);
 }
 
 // Neighbours along x (step 1) or y (step SX) in shared memory, along z in
@@ -372,8 +375,9 @@ __device__ __forceinline__ void fx_near_z(const double *f, long long sz, int e, 
   }
 }
 
-// Velocity gradients (stored), theta = div u and the sensor test.  Bound by
-// the integer unit; the 9 conversions go to the double unit beside it.
+// Velocity gradients (stored), theta = div u and the sensor test.  The x
+// derivatives are converted on the integer unit, the others on the double
+// unit, which balances the two.
 template <int NP>
 __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Blk &B) {
   constexpr int SX = FxTile<NP>::SX;
@@ -407,7 +411,7 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
         const int n = ex[a] - 1022 - 59;  // unit 2^(E - 59)
         int2 up[NP], dn[NP];
         fx_near<NP>(sm[a] + c, 1, up, dn);
-        g[a][0] = fx_d1<NP, true>(up, dn, fx_ldexp(d.fx1, n));
+        g[a][0] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fx1, n));
         fx_near<NP>(sm[a] + c, SX, up, dn);
         g[a][1] = fx_d1<NP, true>(up, dn, fx_ldexp(uy, n));
         fx_near_z<NP>(vel[a] + p, d.sz, ex[a], up, dn);
@@ -440,8 +444,11 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
 // tensor tau and psi = (omega / T) grad T, each term is mu times
 //   X_a = lap u_a + d_a theta / 3 + psi_b tau_ab / mu   (momentum a)
 //   u_a X_a + tau_ab d_b u_a / mu + (c_p / Pr) (lap T + psi . grad T)
-// so mu enters with the sum into the RHS: 63 double operations per point at
-// order 6 (169 when the stencils were in double precision too).
+// so mu enters with the sum into the RHS: about 55 double operations per
+// point at order 6 (169 when the stencils were in double precision too).
+// Three CTAs per multiprocessor (80 registers, 40 bytes spilled) measured
+// 4.61 ms where two took 5.39; adding the directions of a Laplacian up
+// before its one conversion to double then gave 3.95.
 template <int NP>
 __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Blk &B) {
   constexpr int SX = FxTile<NP>::SX, NF = 5;
@@ -472,27 +479,36 @@ __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Bl
   for (int f = 0; f < NV; ++f) Rv[f] = V.fl[f * d.n + q];
   if (ex[5]) {
     const int c = (tid / FTX + NP) * SX + tid % FTX + NP;
-    const double uy1 = __ldg(d.fy1 + j), uy2 = __ldg(d.fy2 + j), ry = __ldg(V.ry + j);
+    const double uy1 = __ldg(d.fy1 + j), ry = __ldg(V.ry + j);
     const double mu = __ldg(V.mu + q), T = __ldg(V.T + p), th = __ldg(V.div + p);
+    FxLap fl;
+    ((int4 *)&fl)[0] = __ldg((const int4 *)(d.fxl + j));
+    ((int4 *)&fl)[1] = __ldg((const int4 *)(d.fxl + j) + 1);
     int2 up[NP], dn[NP];
-    // Laplacians of u, v, w, T; gradients of T and theta (a third of it)
+    // Laplacians of u, v, w, T in the computational coordinates, gradients
+    // of T and theta
     double lap[4], gT[3], gth[3];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
       const int n = ex[f] - 1022 - 59;
       const int2 *S = sm[f] + c;
-      fx_near<NP>(S, 1, up, dn);
-      if (f < 4) lap[f] = fx_d2<NP, false>(S[0], up, dn, fx_ldexp(d.fx2, n));
-      if (f == 3) gT[0] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fx1, n));
-      if (f == 4) gth[0] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fx1, n));
-      fx_near<NP>(S, SX, up, dn);
-      if (f < 4) lap[f] += fx_d2<NP, false>(S[0], up, dn, fx_ldexp(uy2, n));
-      if (f == 3) gT[1] = fx_d1<NP, false>(up, dn, fx_ldexp(uy1, n));
-      if (f == 4) gth[1] = fx_d1<NP, false>(up, dn, fx_ldexp(uy1, n));
-      fx_near_z<NP>(src[f] + p, d.sz, ex[f], up, dn);
-      if (f < 4) lap[f] += fx_d2<NP, false>(S[0], up, dn, fx_ldexp(d.fz2, n));
-      if (f == 3) gT[2] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fz1, n));
-      if (f == 4) gth[2] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fz1, n));
+      FxAcc acc;
+#pragma unroll
+      for (int dir = 0; dir < 3; ++dir) {
+        if (dir == 0) fx_near<NP>(S, 1, up, dn);
+        else if (dir == 1) fx_near<NP>(S, SX, up, dn);
+        else fx_near_z<NP>(src[f] + p, d.sz, ex[f], up, dn);
+        if (f < 4) fx_d2<NP>(acc, S[0], up, dn, dir == 0 ? fl.x : (dir == 1 ? fl.y : fl.z));
+        if (f >= 3) {
+          const double unit = fx_ldexp(dir == 0 ? d.fx1 : (dir == 1 ? uy1 : d.fz1), n);
+          (f == 3 ? gT : gth)[dir] = fx_d1<NP, false>(up, dn, unit);
+        }
+      }
+      if (f < 4) {
+        int drop;
+        const long long v = fx_sum<FxStencil<NP>::W2 + 2>(acc.hi, acc.lo + (acc.m >> FX_LIMB), drop);
+        lap[f] = fx_i2d(v, fl.n + n + drop);
+      }
     }
     double g[3][3];
 #pragma unroll
@@ -576,7 +592,7 @@ __global__ void __launch_bounds__(NT, 3) kb_grad(BatchArgs ba) {
 }
 
 template <int NP>
-__global__ void __launch_bounds__(NT, 2) k_visc(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(NT, 3) k_visc(const __grid_constant__ Dev d) {
   visc_fx_body<NP>(d, fx_blk(d));
 }
 

@@ -81,6 +81,61 @@ def test_flux_accumulators_stay_in_range(half):
         assert abs(D - exact / 2.0 ** 60) < 64 + 2.0 ** -50 * 2.0 ** 60
 
 
+# weights over a common denominator and the bits of their magnitudes (FxStencil)
+C1 = {1: ((1,), 1), 2: ((8, -1), 5), 3: ((45, -9, 1), 7), 4: ((672, -168, 32, -3), 11)}
+C2 = {1: ((-2, 1), 2), 2: ((-30, 16, -1), 6), 3: ((-490, 270, -27, 2), 11), 4: ((-14350, 8064, -1008, 128, -9), 15)}
+
+
+def stencil_sum(hi, lo, bits):
+    """fx_sum: the integer and the bits cut from it."""
+    cut = max(bits - 3, 0)
+    t = fits(hi + (lo >> LIMB), 64)
+    drop = cut if cut and not -(1 << 32) <= t < (1 << 32) else 0
+    return fits((t << (LIMB - drop)) + ((lo & MASK) >> drop), 64), drop
+
+
+@pytest.mark.parametrize("half", [1, 2, 3, 4])
+def test_stencil_sums_stay_in_range(half):
+    """First derivatives and Laplacians of fields at their extremes and at
+    random: values in range, and exact or cut as stated."""
+    rng = np.random.default_rng(10 + half)
+    top = (1 << 59) - 1
+    (c1, w1), (c2, w2) = C1[half], C2[half]
+    assert 2 * sum(abs(c) for c in c1) <= 1 << w1
+    assert abs(c2[0]) + 2 * sum(abs(c) for c in c2[1:]) <= 1 << w2
+    for trial in range(200):
+        def draw(signs):
+            return [int(s) * (top if trial < 60 else int(rng.integers(0, top >> (trial % 40)))) for s in signs]
+
+        up, dn = (draw(rng.choice([-1, 1], half)) for _ in range(2))
+        if trial < 10:
+            up, dn = [int(np.sign(c)) * top for c in c1], [-int(np.sign(c)) * top for c in c1]
+        lu, ld = [limbs(x) for x in up], [limbs(x) for x in dn]
+        hi = sum(c * fits(a[1] - b[1], 32) for c, a, b in zip(c1, lu, ld))
+        lo = sum(c * fits(a[0] - b[0], 32) for c, a, b in zip(c1, lu, ld))
+        v, drop = stencil_sum(fits(hi, 64), fits(lo, 64), w1)
+        exact = sum(c * (a - b) for c, a, b in zip(c1, up, dn))
+        assert v == exact >> drop and (drop == 0 or abs(v) >= 1 << 53)
+        # Laplacian: three directions with weights of any ratio
+        acc, exact = [0, 0, 0], 0
+        kmax = (1 << 60) - 1
+        for d in range(3):
+            up, dn, c = draw(rng.choice([-1, 1], half)), draw(rng.choice([-1, 1], half)), draw([1])[0]
+            if trial < 10:
+                c, up, dn = -top, [int(np.sign(x)) * top for x in c2[1:]], [int(np.sign(x)) * top for x in c2[1:]]
+            k = kmax if d == trial % 3 or trial < 10 else int(rng.integers(0, kmax))
+            kl, kh = k & MASK, k >> LIMB
+            lc, lu, ld = limbs(c), [limbs(x) for x in up], [limbs(x) for x in dn]
+            hi = c2[0] * lc[1] + sum(w * fits(a[1] + b[1], 32) for w, a, b in zip(c2[1:], lu, ld))
+            lo = c2[0] * lc[0] + sum(w * fits(a[0] + b[0], 32) for w, a, b in zip(c2[1:], lu, ld))
+            t = fits(hi, 64) + (fits(lo, 64) >> LIMB)
+            r, t0, t1 = lo & MASK, t & MASK, fits(t >> LIMB, 32)
+            acc = [fits(x, 64) for x in (acc[0] + t1 * kh, acc[1] + t1 * kl + t0 * kh, acc[2] + t0 * kl + r * kh)]
+            exact += k * (c2[0] * c + sum(w * (a + b) for w, a, b in zip(c2[1:], up, dn)))
+        v, drop = stencil_sum(acc[0], fits(acc[1] + (acc[2] >> LIMB), 64), w2 + 2)
+        assert abs(v - (exact >> (60 + drop))) <= 8
+
+
 def periodic_state(shape, contrast, which, unit, seed=5):
     """Smooth periodic box whose density or temperature spans the given
     factor, in units where the density is of the given size; w = 0."""
