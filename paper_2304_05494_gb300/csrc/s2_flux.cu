@@ -334,6 +334,16 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
   const int n = DIR == 0 ? d.nx : (DIR == 1 ? d.ny : d.nz);
   const int nac = DIR == 0 ? d.ny : d.nx;   // extent across
 
+  // flagged interfaces of a tile, gathered here so that the tile takes its
+  // place in the global list with one atomic: with one per warp, a flow
+  // that flags 19 % of the interfaces (isotropic 256^3, single precision)
+  // spent 1.5 / 1.9 / 1.9 ms per step in x / y / z waiting for that one
+  // address, against 0.61 / 0.66 / 0.65 without flags.  Counter and list
+  // position by tile parity.
+  constexpr int NI = (L + 1) * W;
+  __shared__ unsigned list[HASW ? NI : 1], nlisted[2], listed_at[2];
+  unsigned mycount = 0;  // flagged interfaces after this thread's points
+
   // box origin of a tile in padded coordinates (interior point i sits at i + GH)
   auto issue = [&](int t, int buf) {
     int x0, y0, z0;
@@ -346,6 +356,7 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
   // tile of this CTA's iteration it, its buffer and that buffer's use count
   const int G = (int)B.nx;
   if (tid == 0) {
+    nlisted[0] = nlisted[1] = 0;
     for (int b = 0; b < NBUF; ++b) mbar_init(&bar[b], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -448,8 +459,6 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
     if constexpr (HASW) {
       const R *Ss = S + F_S * SFA;
       const int wr = (d.weno + 1) / 2;
-      constexpr int NI = (L + 1) * W;
-      unsigned long long mycount = 0;
       for (int base = 0; base < NI; base += NTHREADS) {
         int idx = base + tid;
         bool flag = false;
@@ -483,16 +492,27 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
           int lane = tid & 31;
           int leader = __ffs(bal) - 1;
           unsigned off = 0;
-          if (lane == leader) off = atomicAdd(&d.scal->nlist[DIR], (unsigned)__popc(bal));
+          if (lane == leader) off = atomicAdd(&nlisted[it & 1], (unsigned)__popc(bal));
           off = __shfl_sync(0xffffffffu, off, leader);
-          const long long at = (long long)off + __popc(bal & ((1u << lane) - 1u));
-          if (flag && S2_OK_IDX(d, at, d.nslot[DIR])) d.wlist[DIR][at] = (unsigned)slot;
+          if (flag) list[off + __popc(bal & ((1u << lane) - 1u))] = slot;
         }
       }
-      for (int o = 16; o > 0; o >>= 1) mycount += __shfl_xor_sync(0xffffffffu, mycount, o);
-      if ((tid & 31) == 0 && mycount) atomicAdd(&d.scal->wcount, mycount);
     }
     __syncthreads();
+    // the tile's place in the global list, asked for before the arithmetic
+    // below and used after it
+    unsigned place = 0;
+    if (HASW && tid == 0) {
+      if (nlisted[it & 1]) place = atomicAdd(&d.scal->nlist[DIR], nlisted[it & 1]);
+      nlisted[(it + 1) & 1] = 0;  // last read before the barrier that opened this tile
+    }
+    auto flush = [&]() {  // after a barrier that follows listed_at's store
+      if constexpr (HASW) {
+        const unsigned cnt = nlisted[it & 1], at = listed_at[it & 1];
+        for (unsigned m = tid; m < cnt; m += NTHREADS)
+          if (S2_OK_IDX(d, (long long)at + m, d.nslot[DIR])) d.wlist[DIR][at + m] = list[m];
+      }
+    };
 
     // ---- 3. central flux difference of the thread's points -> RHS ----
     if constexpr (TV == 2) {
@@ -512,7 +532,9 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
           V.fl[c * d.n + q[pp]] = fma(-scale2, Dc, prev[pp][c]);
         }
       }
+      if (HASW && tid == 0) listed_at[it & 1] = place;
       __syncthreads();  // staging buffer and TP free for the next tile
+      flush();
       continue;
     }
 #pragma unroll
@@ -566,7 +588,13 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
     // the limbs were written by ordinary stores: order them before the copy
     // that refills the buffer
     if (FX) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (HASW && tid == 0) listed_at[it & 1] = place;
     __syncthreads();  // staging buffer and TP free for the next tile
+    flush();
+  }
+  if constexpr (HASW) {
+    mycount = __reduce_add_sync(0xffffffffu, mycount);
+    if ((tid & 31) == 0 && mycount) atomicAdd(&d.scal->wcount, (unsigned long long)mycount);
   }
 }
 
