@@ -46,6 +46,7 @@ constexpr int ERR_TIMEOUT = 2;  // a bounded wait on an asynchronous copy gave u
 constexpr int ERR_BOUNDS = 4;   // an index left its array (checked build)
 
 struct FxLap;
+struct PowTab;
 
 // Scheme constants in the arithmetic type R of a kernel (double for the
 // FP64 path, float for the flux arithmetic of the mixed path).
@@ -116,6 +117,11 @@ struct Dev {
   double gR;               // gamma R (c^2 = gamma R T)
   int mu_p, mu_q;          // visc_exp = mu_p/mu_q when rational with small terms, else mu_q = 0
   double mu_qm1, mu_qp1;   // mu_q - 1, mu_q + 1
+  // power law on the integer unit (s2_power.cuh): its table (nullptr: not
+  // used), omega (Q58), omega / ln 2 (Q60), largest exponent of T/T_ref
+  const PowTab *powt;
+  long long pow_w, pow_w2;
+  int pow_emax;
   double thr;              // sensor threshold
   double cfl;
   int dt_every;            // recompute dt at steps that are multiples of this (cfl > 0)
@@ -446,10 +452,18 @@ __device__ __forceinline__ R tp_dcp(const Consts<R> &K, R T, R rT) {
   return fma(rT * rT, fma(rT, K.dcc[0], K.dcc[1]), pos);
 }
 
-template <class R>
-__device__ __forceinline__ R tp_e(const Consts<R> &K, R T, R rT) {
+struct TpLog {
+  template <class R>
+  __device__ __forceinline__ R operator()(R x) const {
+    return tp_log(x);
+  }
+};
+
+// (LOG: the logarithm to use)
+template <class R, class LOG = TpLog>
+__device__ __forceinline__ R tp_e(const Consts<R> &K, R T, R rT, LOG ln = LOG()) {
   R e = fma(T, fma(T, fma(T, fma(T, fma(T, K.ecf[6], K.ecf[5]), K.ecf[4]), K.ecf[3]), K.ecf[2]), K.ecf[0] * rT);
-  if (K.ecf[1] != R(0)) e = fma(K.ecf[1], tp_log(T), e);
+  if (K.ecf[1] != R(0)) e = fma(K.ecf[1], ln(T), e);
   return e;
 }
 
@@ -466,13 +480,13 @@ __device__ __forceinline__ R tp_sound2(const Consts<R> &K, R T) {
 // iteration converges quadratically, so the error is then of order tol^2
 // (1e-18 in double, 1e-7 in single precision).  ok is cleared if that
 // does not happen within 24 steps or T leaves T > 0.
-template <class R>
-__device__ __forceinline__ R tp_temperature(const Consts<R> &K, R target, R T, R sR, bool &ok) {
+template <class R, class LOG = TpLog>
+__device__ __forceinline__ R tp_temperature(const Consts<R> &K, R target, R T, R sR, bool &ok, LOG ln = LOG()) {
   const R tol = sizeof(R) == 8 ? R(1e-9) : R(3e-4);
   const R dR = sR - K.R_gas;
   for (int it = 0; it < 24; ++it) {
     const R rT = rcp_pos(T);
-    const R f = fma(sR, T, tp_e(K, T, rT)) - target;
+    const R f = fma(sR, T, tp_e(K, T, rT, ln)) - target;
     const R dT = f * rcp_pos(tp_cp(K, T, rT) + dR);
     T -= dT;
     if (!(T > R(0))) break;

@@ -25,6 +25,7 @@
 #include "../../include/s2.h"
 #include "s2_fixed.cuh"
 #include "s2_internal.cuh"
+#include "s2_power.cuh"
 
 using namespace s2;
 
@@ -231,7 +232,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
       S2_GUARD(okp) T0 = V.T[p];
       if (!positive_finite(T0)) T0 = tp_guess(d.kd, e);
       bool ok = true;
-      T = tp_temperature(d.kd, e, T0, 0.0, ok);
+      T = tp_temperature(d.kd, e, T0, 0.0, ok, FixedLog{d.powt});
       if (!ok) atomicOr(&d.scal->status, ERR_NONFINITE);
       h = fma(d.R, T, e);
     }
@@ -253,7 +254,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
     for (int f = 0; f < FX_NMIN; ++f) fm[f] = 2047u - fe[f];
     double mu = 0.0;
     if (d.viscous) {
-      mu = viscosity(d, T);
+      mu = viscosity_fixed(d, T);
       V.mu[q] = mu;
     }
     if (!positive_finite(rho) || !positive_finite(T) || !finite_bits(q2))
@@ -1403,6 +1404,14 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   // s2_rhs stages its double output in fln when that is double, else here
   s->rhs_stage = d.mixed ? A(NV * nn) : (double *)d.fln;
   double *eta = A(grid->ny), *ay = A(4 * grid->ny), *by = A(5 * grid->ny), *ry = A(grid->ny), *dvy = A(grid->ny);
+  // table of the power law and the logarithm (FP64: mu of viscous runs, the
+  // thermally perfect e(T))
+  std::vector<PowTab> powt(1);
+  if (!d.mixed && (d.viscous || d.kd.tp)) {
+    d.powt = (PowTab *)dalloc(s, sizeof(PowTab));
+    if (!d.powt) ok = false;
+    pow_setup(d, powt[0]);
+  }
   double *fy = A(grid->ny);
   FxLap *fxl = (FxLap *)dalloc(s, sizeof(FxLap) * grid->ny);
   if (!fxl) ok = false;
@@ -1476,6 +1485,8 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
     delete s;
     return S2_ENOMEM;
   }
+  if (e == cudaSuccess && d.powt)
+    e = cudaMemcpyAsync((void *)d.powt, powt.data(), sizeof(PowTab), cudaMemcpyHostToDevice, s->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ynd, yn.data(), sizeof(double) * grid->ny, cudaMemcpyHostToDevice, s->stream);
   if (e == cudaSuccess) {
