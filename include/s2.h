@@ -242,7 +242,8 @@ int s2_stream_states(s2_solver *s, const double *w_in, long long in_stride, doub
                      int count, int nsteps);
 
 /* Flux tile shape per direction: tiles[d] = 0 (64x4 points for x, 32x8
- * for y and z) or 1 (narrower along the direction: 32x8 for x, 16x16 for y
+ * for y and z, or the narrower one where it covers the grid with a quarter
+ * fewer tiles) or 1 (narrower along the direction: 32x8 for x, 16x16 for y
  * and z, for small boxes); single precision doubles each tile along one
  * axis.  Default: (0, 0, 0) for S2_FP64, (0, 1, 1) for S2_MIXED.  Chosen
  * per grid by the autotuner (paper_2304_05494_gb300/autotune.py, the tile
@@ -258,7 +259,8 @@ int s2_set_tiles(s2_solver *s, const int *tiles);
  * persistent flux grid of direction d (0: as many as fit, up to 16; KEEP
  * in S2_FP64 has no persistent grid).
  * z_planes: z-planes each CTA of the mixed path's z-marching gradient and
- * viscous passes walks (0: 12; else 4, 8, 16 or 24, compiled variants).  weno_ctas_per_sm: cap of the
+ * viscous passes walks (0 or 12: chosen from the grid, between 1 and 24;
+ * else 4, 8, 16 or 24, compiled variants).  weno_ctas_per_sm: cap of the
  * WENO kernels' 64-thread CTAs per multiprocessor (0: 16; else 1..64).
  * Takes effect at the next s2_step; results do not depend on it, except
  * that with channel forcing in S2_MIXED the viscous pass sums the forcing
@@ -303,7 +305,7 @@ int s2_get_flags(s2_solver *s, unsigned char *fx, unsigned char *fy, unsigned ch
 #define S2_PROF_VISC 8      /* visflx */
 #define S2_PROF_FORCE 9     /* force_rhs_1 (two kernels) */
 #define S2_PROF_UPDATE 10   /* RK3 update */
-#define S2_PROF_WENO 11     /* WENO flux corrections at flagged interfaces (3 kernels) */
+#define S2_PROF_WENO 11     /* WENO flux corrections at flagged interfaces (1 kernel, or one per direction) */
 #define S2_PROF_APPLY 12    /* adding the WENO corrections (inviscid runs; fused into visc otherwise) */
 #define S2_PROF_KINDS 13
 

@@ -41,6 +41,22 @@
 #include "s2_internal.cuh"
 
 namespace s2 {
+
+constexpr int WENO_NT = 64;  // threads per CTA of the WENO kernels
+
+// CTAs of a direction's WENO corrections: small, so that the flagged
+// interfaces (a count known on the device only, often a few per cent of the
+// slots) spread evenly over the multiprocessors; at most weno_cps on each,
+// or half as many per direction in a launch of all three.  (Isotropic 256^3,
+// 19 % flagged, ms per step for 16 / 24 / 48 per multiprocessor over the
+// three: 3.51 / 2.79 / 2.96; 24 is three times what is resident.)
+unsigned weno_blocks(const Dev &d, int dir, bool all) {
+  const long long need = (d.nslot[dir] + WENO_NT - 1) / WENO_NT;
+  const int cps = d.weno_cps > 0 ? d.weno_cps : 16;
+  const long long cap = (long long)(all ? (cps + 1) / 2 : cps) * d.nsm;
+  return (unsigned)(need < 1 ? 1 : (need < cap ? need : cap));
+}
+
 namespace {
 
 // Central first-derivative coefficients a_l of order 2 NP (l = 1..NP): the
@@ -87,8 +103,14 @@ struct Tile<2, 1> {  // z: 16 along z, 16 columns
 template <int DIR>
 struct Tile<DIR, 2> : Tile<DIR, 0> {};
 
+// Variant 3, x only: rows of at most half a narrow tile (chosen by the
+// default rule alone, Dev::tile = 2).
+template <>
+struct Tile<0, 3> {
+  static constexpr int L = 16, W = 16;
+};
+
 constexpr int NTHREADS = 256;
-constexpr int WENO_NT = 64;  // threads per CTA of the WENO kernels
 enum { F_RHO = 0, F_U, F_V, F_W, F_H, F_P, F_S, NF };
 
 // The tile a kernel of arithmetic type R works on.  Double precision uses
@@ -151,7 +173,7 @@ struct FluxLayout {
   // one in y and z (larger tiles), double precision one; KEEP in double
   // precision (bound by the double-precision unit, and with five times the
   // pair words) runs one tile per CTA and stages it once
-  static constexpr int NBUF = sizeof(R) == 4 ? (DIR == 0 ? 3 : 2) : (TV == 2 ? 1 : 2);
+  static constexpr int NBUF = sizeof(R) == 4 ? (DIR == 0 && TV != 3 ? 3 : 2) : (TV == 2 ? 1 : 2);
 };
 
 // Dynamic shared memory of a flux CTA: barriers, staging buffers and the
@@ -601,6 +623,7 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
 template <int DIR, bool HASW, class R, int TV, int NP>
 __global__ void __launch_bounds__(NTHREADS, 4) k_flux(const __grid_constant__ FluxMaps maps, Dev d,
                                                       const TileGrid<DIR, TV, R> tg, int accumulate) {
+  pdl_wait();
   flux_body<DIR, HASW, R, TV, NP>(maps, d, tg, accumulate, grid_blk());
 }
 
@@ -617,12 +640,17 @@ __global__ void __launch_bounds__(NTHREADS, 4) kb_flux(BatchArgs ba, const FluxM
 // ------------------------------------------------------------------ WENO
 // Reconstruction at i+1/2 from 2r-1 values g[0..2r-2] centred on g[r-1]:
 // Jiang & Shu (r=3), Balsara & Shu (r=4), alpha_k = d_k/(eps+beta_k)^2.
+// Everything but the centre value is formed from the undivided differences
+// d_i = g[i+1] - g[i] and, for the indicators, theirs: the substencil
+// polynomials are q_k = g[r-1] + (a combination of differences)/6 or /12.
 // The normalisation sum alpha_k q_k / sum alpha_k is evaluated with one
 // reciprocal by multiplying through by prod_k (eps+beta_k)^2, and the
-// substencil polynomials' common denominator (6, 12) joins that
-// reciprocal.  The caller passes eps: reconstructing 2 g with eps' = 4 eps
-// gives exactly twice the reconstruction of g with eps (beta is quadratic
-// in g), which lets the flux splitting skip its factor 1/2.
+// polynomials' common denominator joins that reciprocal.  Factors common to
+// eps and all beta_k, and to all alpha_k, cancel: in double precision they
+// are chosen to save multiplications (in single precision they would shift
+// the range in which the products neither overflow nor vanish).  The caller passes eps: reconstructing 2 g with eps' = 4
+// eps gives exactly twice the reconstruction of g with eps (beta is
+// quadratic in g), which lets the flux splitting skip its factor 1/2.
 template <class R>
 __device__ __forceinline__ R recip_pos(R x) {
   return rcp_pos(x);
@@ -630,49 +658,54 @@ __device__ __forceinline__ R recip_pos(R x) {
 
 template <class R>
 __device__ __forceinline__ R weno5(const R *g, R eps) {
-  R q0 = R(2) * g[0] - R(7) * g[1] + R(11) * g[2];
-  R q1 = -g[1] + R(5) * g[2] + R(2) * g[3];
-  R q2 = R(2) * g[2] + R(5) * g[3] - g[4];
-  R t, b0, b1, b2;
-  t = g[0] - R(2) * g[1] + g[2]; b0 = R(13.0 / 12.0) * t * t;
-  t = g[0] - R(4) * g[1] + R(3) * g[2]; b0 += R(0.25) * t * t;
-  t = g[1] - R(2) * g[2] + g[3]; b1 = R(13.0 / 12.0) * t * t;
-  t = g[1] - g[3]; b1 += R(0.25) * t * t;
-  t = g[2] - R(2) * g[3] + g[4]; b2 = R(13.0 / 12.0) * t * t;
-  t = R(3) * g[2] - R(4) * g[3] + g[4]; b2 += R(0.25) * t * t;
-  R s0 = eps + b0, s1 = eps + b1, s2 = eps + b2;
+  const R d0 = g[1] - g[0], d1 = g[2] - g[1], d2 = g[3] - g[2], d3 = g[4] - g[3];
+  // 6 (q_k - g[2])
+  const R q0 = R(5) * d1 - R(2) * d0, q1 = d1 + R(2) * d2, q2 = R(4) * d2 - d3;
+  const R t0 = d1 - d0, t1 = d2 - d1, t2 = d3 - d2;
+  const R u0 = R(3) * d1 - d0, u1 = d1 + d2, u2 = d3 - R(3) * d2;
+  constexpr bool DBL = sizeof(R) == 8;
+  const R e = DBL ? R(4) * eps : eps, c = DBL ? R(13.0 / 3.0) : R(13.0 / 12.0), f = DBL ? R(1) : R(0.25);
+  R s0 = fma(c * t0, t0, fma(f * u0, u0, e));
+  R s1 = fma(c * t1, t1, fma(f * u1, u1, e));
+  R s2 = fma(c * t2, t2, fma(f * u2, u2, e));
   s0 *= s0; s1 *= s1; s2 *= s2;
-  R a0 = R(0.1) * s1 * s2, a1 = R(0.6) * s0 * s2, a2 = R(0.3) * s0 * s1;
-  return (a0 * q0 + a1 * q1 + a2 * q2) * recip_pos(R(6) * (a0 + a1 + a2));
+  const R w = DBL ? R(1) : R(0.1);
+  const R a0 = w * (s1 * s2), a1 = (R(6) * w) * (s0 * s2), a2 = (R(3) * w) * (s0 * s1);
+  return fma(a0 * q0 + a1 * q1 + a2 * q2, recip_pos(R(6) * (a0 + a1 + a2)), g[2]);
 }
 
 template <class R>
 __device__ __forceinline__ R weno7(const R *g, R eps) {
-  R q0 = R(-3) * g[0] + R(13) * g[1] - R(23) * g[2] + R(25) * g[3];
-  R q1 = g[1] - R(5) * g[2] + R(13) * g[3] + R(3) * g[4];
-  R q2 = -g[2] + R(7) * g[3] + R(7) * g[4] - g[5];
-  R q3 = R(3) * g[3] + R(13) * g[4] - R(5) * g[5] + g[6];
-  // smoothness indicators: 240 x the Jiang-Shu measure as sums of squares
-  // of the undivided differences of each 4-point substencil
-  R bk[4];
+  R d[6], e2[5], e3[4];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) d[i] = g[i + 1] - g[i];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) e2[i] = d[i + 1] - d[i];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) e3[i] = e2[i + 1] - e2[i];
+  // 12 (q_k - g[3])
+  const R q0 = R(3) * d[0] - R(10) * d[1] + R(13) * d[2], q1 = R(4) * d[2] - d[1] + R(3) * d[3];
+  const R q2 = d[2] + R(6) * d[3] - d[4], q3 = R(9) * d[3] - R(4) * d[4] + d[5];
+  // smoothness indicators: 240 x the Jiang-Shu measure (in double precision
+  // the measure itself) as sums of squares of the undivided differences of
+  // each 4-point substencil
   const R c10[4] = {R(5.0 / 2.0), R(3.0 / 2.0), R(1.0 / 2.0), R(-1.0 / 2.0)};
   const R c11[4] = {R(11.0 / 6.0), R(1.0 / 3.0), R(-1.0 / 6.0), R(1.0 / 3.0)};
   const R c2[4] = {R(2), R(1), R(0), R(-1)};
+  constexpr bool DBL = sizeof(R) == 8;
+  const R m = DBL ? R(1) : R(240), e = DBL ? eps * R(1.0 / 240.0) : eps;
+  R s[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    R e1 = g[k + 1] - g[k];
-    R e2 = g[k + 2] - R(2) * g[k + 1] + g[k];
-    R e3 = g[k + 3] - R(3) * g[k + 2] + R(3) * g[k + 1] - g[k];
-    R t1 = e1 + c10[k] * e2 + c11[k] * e3;
-    R t2 = e2 + c2[k] * e3;
-    bk[k] = R(240) * t1 * t1 + R(260) * t2 * t2 + R(781.0 / 3.0) * e3 * e3;
+    const R t1 = fma(c11[k], e3[k], fma(c10[k], e2[k], d[k]));
+    const R t2 = k == 2 ? e2[k] : fma(c2[k], e3[k], e2[k]);
+    const R b = fma(m * t1, t1, fma(m * R(13.0 / 12.0) * t2, t2, fma(m * R(781.0 / 720.0) * e3[k], e3[k], e)));
+    s[k] = b * b;
   }
-  R s0 = eps + bk[0], s1 = eps + bk[1], s2 = eps + bk[2], s3 = eps + bk[3];
-  s0 *= s0; s1 *= s1; s2 *= s2; s3 *= s3;
-  R p01 = s0 * s1, p23 = s2 * s3;
-  R a0 = R(1.0 / 35.0) * s1 * p23, a1 = R(12.0 / 35.0) * s0 * p23;
-  R a2 = R(18.0 / 35.0) * p01 * s3, a3 = R(4.0 / 35.0) * p01 * s2;
-  return (a0 * q0 + a1 * q1 + a2 * q2 + a3 * q3) * recip_pos(R(12) * (a0 + a1 + a2 + a3));
+  const R p01 = s[0] * s[1], p23 = s[2] * s[3];
+  const R w = DBL ? R(1) : R(1.0 / 35.0);
+  const R a0 = w * s[1] * p23, a1 = R(12) * w * s[0] * p23, a2 = R(18) * w * p01 * s[3], a3 = R(4) * w * p01 * s[2];
+  return fma(a0 * q0 + a1 * q1 + a2 * q2 + a3 * q3, recip_pos(R(12) * (a0 + a1 + a2 + a3)), g[3]);
 }
 
 // Order 3: two substencils, d = (1/3, 2/3), beta_k = (undivided difference)^2.
@@ -695,7 +728,10 @@ __device__ __forceinline__ R weno_rec(const R *g, R eps) {
   else return weno7<R>(g, eps);
 }
 
-// F_weno - F_central at every listed interface of direction DIR.
+// F_weno - F_central at every listed interface of direction dir.  The
+// direction is a run-time value (strides, and which fields are the normal and
+// tangential velocities), so that one launch serves all three and they share
+// their instructions in the cache.
 //
 // In the frame (normal n, tangents t1, t2) of the interface, with the Roe
 // state (u_n, u_1, u_2, H~, c~), b = gamma-1, h2 = 1/(2 c~^2), the left
@@ -713,27 +749,31 @@ __device__ __forceinline__ R weno_rec(const R *g, R eps) {
 // PA = p h2 b (u_n - u~_n), PB = p h2 c~.  Lax-Friedrichs: each field's
 // dissipation is the largest |eigenvalue| (u_n - c, u_n, u_n + c) over the
 // stencil points.  The result goes back with the right eigenvectors.
-template <int DIR, int WR, class R>
-__device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &B) {
-  constexpr int T1 = (DIR + 1) % 3, T2 = (DIR + 2) % 3;
+template <int WR, class R>
+__device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &B, const int dir) {
   constexpr int NP = 2 * WR;  // stencil points s-WR+1 .. s+WR
   const View<R> V = view<R>(d);
   const Consts<R> &K = consts<R>(d);
-  const unsigned cnt = d.scal->nlist[DIR];
-  const R *vel[3] = {V.u, V.v, V.ww};
+  const unsigned cnt = d.scal->nlist[dir];
+  const int t1 = dir == 2 ? 0 : dir + 1, t2 = dir == 0 ? 2 : dir - 1;  // tangential directions
+  const R *vn = dir == 0 ? V.u : (dir == 1 ? V.v : V.ww), *v1 = t1 == 0 ? V.u : (t1 == 1 ? V.v : V.ww);
+  const R *v2 = t2 == 0 ? V.u : (t2 == 1 ? V.v : V.ww);
+  const long long stride = dir == 0 ? 1 : (dir == 1 ? d.sy : d.sz), ns = d.nslot[dir];
+  const unsigned *wlist = d.wlist[dir];
+  R *const dF = V.dF[dir];
   const R bq = K.gamma - R(1);
   for (unsigned e0 = B.x * blockDim.x + threadIdx.x; e0 < cnt; e0 += B.nx * blockDim.x) {
-    if (!S2_OK_IDX(d, e0, d.nslot[DIR])) break;
-    const long long slot = d.wlist[DIR][e0];
+    if (!S2_OK_IDX(d, e0, ns)) break;
+    const long long slot = wlist[e0];
     int i = 0, j = 0, k = 0, s;
     const unsigned us = (unsigned)slot;
-    if (DIR == 0) {
+    if (dir == 0) {
       unsigned t = d.fnx1.div(us), kk = d.fny.div(t);
       s = (int)(us - t * (unsigned)(d.nx + 1)) - 1;
       j = (int)(t - kk * (unsigned)d.ny);
       k = (int)kk;
       i = s;
-    } else if (DIR == 1) {
+    } else if (dir == 1) {
       unsigned t = d.fnx.div(us), kk = d.fny1.div(t);
       i = (int)(us - t * (unsigned)d.nx);
       s = (int)(t - kk * (unsigned)(d.ny + 1)) - 1;
@@ -746,23 +786,23 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
       s = (int)kk - 1;
       k = s;
     }
-    const long long stride = DIR == 0 ? 1 : (DIR == 1 ? d.sy : d.sz);
     const long long p0 = pidx(d, i, j, k);  // point s of the interface s+1/2
     // the WENO stencil and the central pairs reach p0 - 3 stride .. p0 + 4 stride
-    if (!(S2_OK_IDX(d, slot, d.nslot[DIR]) && S2_OK_IDX(d, p0 - 3 * stride, d.np) &&
+    if (!(S2_OK_IDX(d, slot, ns) && S2_OK_IDX(d, p0 - 3 * stride, d.np) &&
           S2_OK_IDX(d, p0 + 4 * stride, d.np)))
       continue;
 
-    // --- central flux at this interface (order 2 npc): split form, or KEEP
+    // --- central flux at this interface (order 2 npc): split form, or KEEP,
+    // components rho, normal, tangential 1 and 2, E
     R FC[5] = {R(0), R(0), R(0), R(0), R(0)}, fp = R(0);
     if (d.keep) {
       for (int l = 1; l <= d.npc; ++l)
         for (int m = 0; m < l; ++m) {
           const long long a = p0 - m * stride, b = p0 + (l - m) * stride;
           R f[5];
-          keep_pair<DIR, R>(__ldg(V.rho + a), __ldg(V.u + a), __ldg(V.v + a), __ldg(V.ww + a), __ldg(V.p + a),
-                            __ldg(V.rho + b), __ldg(V.u + b), __ldg(V.v + b), __ldg(V.ww + b), __ldg(V.p + b),
-                            K.gamma - R(1), d.keep, f);
+          keep_pair<0, R>(__ldg(V.rho + a), __ldg(vn + a), __ldg(v1 + a), __ldg(v2 + a), __ldg(V.p + a),
+                          __ldg(V.rho + b), __ldg(vn + b), __ldg(v1 + b), __ldg(v2 + b), __ldg(V.p + b),
+                          K.gamma - R(1), d.keep, f);
           const R al2 = R(2) * K.acen[l];
 #pragma unroll
           for (int c = 0; c < 5; ++c) FC[c] = fma(al2, f[c], FC[c]);
@@ -776,15 +816,14 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
       for (int m = 0; m < l; ++m) {
         long long a = p0 - m * stride, b = p0 + (l - m) * stride;
         R sr = __ldg(V.rho + a) + __ldg(V.rho + b);
-        R su = __ldg(V.u + a) + __ldg(V.u + b), sv = __ldg(V.v + a) + __ldg(V.v + b);
-        R sw = __ldg(V.ww + a) + __ldg(V.ww + b);
+        R sn = __ldg(vn + a) + __ldg(vn + b), s1 = __ldg(v1 + a) + __ldg(v1 + b);
+        R s2 = __ldg(v2 + a) + __ldg(v2 + b);
         R sh = __ldg(V.H + a) + __ldg(V.H + b);
-        R sun = DIR == 0 ? su : (DIR == 1 ? sv : sw);
-        R mm = sr * sun;
+        R mm = sr * sn;
         acc[0] += mm;
-        acc[1] += mm * su;
-        acc[2] += mm * sv;
-        acc[3] += mm * sw;
+        acc[1] += mm * sn;
+        acc[2] += mm * s1;
+        acc[3] += mm * s2;
         acc[4] += mm * sh;
         ps += __ldg(V.p + a) + __ldg(V.p + b);
       }
@@ -794,15 +833,15 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
       for (int f = 1; f < 5; ++f) FC[f] += R(0.25) * al * acc[f];
       fp += al * ps;
     }
-    FC[1 + DIR] += fp;
+    FC[1] += fp;
 
     // --- Roe average of the two interface states
     const long long ia = p0, ib = p0 + stride;
-    R ra = sqrt(__ldg(V.rho + ia)), rb = sqrt(__ldg(V.rho + ib));
+    R ra = sqrt_pos(__ldg(V.rho + ia)), rb = sqrt_pos(__ldg(V.rho + ib));
     R inv = recip_pos(ra + rb);
-    R un = (ra * __ldg(vel[DIR] + ia) + rb * __ldg(vel[DIR] + ib)) * inv;
-    R ut1 = (ra * __ldg(vel[T1] + ia) + rb * __ldg(vel[T1] + ib)) * inv;
-    R ut2 = (ra * __ldg(vel[T2] + ia) + rb * __ldg(vel[T2] + ib)) * inv;
+    R un = (ra * __ldg(vn + ia) + rb * __ldg(vn + ib)) * inv;
+    R ut1 = (ra * __ldg(v1 + ia) + rb * __ldg(v1 + ib)) * inv;
+    R ut2 = (ra * __ldg(v2 + ia) + rb * __ldg(v2 + ib)) * inv;
     R Ht = (ra * __ldg(V.H + ia) + rb * __ldg(V.H + ib)) * inv;
     R q2 = un * un + ut1 * ut1 + ut2 * ut2;
     // chi = (1/rho) dp/de, c~^2, the entropy wave's energy entry hs and
@@ -823,7 +862,7 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
       hs = Ht - c2 * recip_pos(chi);
       qa = q2 - hs;
     }
-    R cs = sqrt(c2);
+    R cs = sqrt_pos(c2);
     R h2 = R(0.5) * recip_pos(c2);
     R hb = h2 * chi, hc = h2 * cs;
 
@@ -833,11 +872,11 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
 #pragma unroll
     for (int m = 0; m < NP; ++m) {
       long long q = p0 + (m - WR + 1) * stride;
-      R r = __ldg(V.rho + q), unm = __ldg(vel[DIR] + q);
-      R u1 = __ldg(vel[T1] + q), u2 = __ldg(vel[T2] + q);
+      R r = __ldg(V.rho + q), unm = __ldg(vn + q);
+      R u1 = __ldg(v1 + q), u2 = __ldg(v2 + q);
       R pm = __ldg(V.p + q), hm = __ldg(V.H + q);
       const R Tm = __ldg(V.T + q);
-      R cm = sqrt(K.tp ? tp_sound2(K, Tm) : K.gR * Tm);
+      R cm = sqrt_pos(K.tp ? tp_sound2(K, Tm) : K.gR * Tm);
       R mn = r * unm, m1 = r * u1, m2 = r * u2, E = r * hm - pm;
       R A = hb * (qa * r - un * mn - ut1 * m1 - ut2 * m2 + E);
       R B = hc * (un * r - mn);
@@ -852,9 +891,9 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
       G[2][m] = unm * Vv[2][m];
       G[3][m] = unm * Vv[3][m];
       G[4][m] = unm * Vv[4][m] + PA + PB;
-      al0 = fmax(al0, fabs(unm - cm));
-      al1 = fmax(al1, fabs(unm));
-      al4 = fmax(al4, fabs(unm + cm));
+      al0 = max_mag(al0, unm - cm);
+      al1 = max_mag(al1, unm);
+      al4 = max_mag(al4, unm + cm);
     }
     // Lax-Friedrichs split g+- = (G +- alpha V) / 2, reconstructed as
     // G +- alpha V with 4 eps (exactly twice the result), halved once
@@ -875,27 +914,36 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
     // --- back to conserved fluxes with the right eigenvectors
     R s014 = gh[0] + gh[1] + gh[4];
     R dn = gh[4] - gh[0];
-    R Fr[5];
-    Fr[0] = s014;
-    Fr[1 + DIR] = un * s014 + cs * dn;
-    Fr[1 + T1] = ut1 * s014 + gh[2];
-    Fr[1 + T2] = ut2 * s014 + gh[3];
-    Fr[4] = Ht * (gh[0] + gh[4]) + un * cs * dn + hs * gh[1] + ut1 * gh[2] + ut2 * gh[3];
-    const long long ns = d.nslot[DIR];
-#pragma unroll
-    for (int f = 0; f < 5; ++f) V.dF[DIR][f * ns + slot] = Fr[f] - FC[f];
+    const R Fr[5] = {s014, un * s014 + cs * dn, ut1 * s014 + gh[2], ut2 * s014 + gh[3],
+                     Ht * (gh[0] + gh[4]) + un * cs * dn + hs * gh[1] + ut1 * gh[2] + ut2 * gh[3]};
+    R *const o = dF + slot;
+    o[0] = Fr[0] - FC[0];
+    o[(1 + dir) * ns] = Fr[1] - FC[1];
+    o[(1 + t1) * ns] = Fr[2] - FC[2];
+    o[(1 + t2) * ns] = Fr[3] - FC[3];
+    o[4 * ns] = Fr[4] - FC[4];
   }
 }
 
-template <int DIR, int WR, class R>
-__global__ void __launch_bounds__(WENO_NT) k_weno(Dev d) {
-  weno_body<DIR, WR, R>(d, grid_blk());
+// dir < 0: the direction is the grid's y index (one launch for all three).
+template <int WR, class R>
+__global__ void __launch_bounds__(WENO_NT) k_weno(Dev d, int dir) {
+  pdl_wait();
+  weno_body<WR, R>(d, grid_blk(), dir < 0 ? (int)blockIdx.y : dir);
 }
 
-template <int DIR, int WR, class R>
+// Batched: the work list's boxes have three rows of CTAs, one per
+// direction.  A CTA beyond the list (flows that flag nothing have none)
+// leaves before it copies the box's parameters.
+template <int WR, class R>
 __global__ void __launch_bounds__(WENO_NT) kb_weno(BatchArgs ba) {
-  S2_BATCH_ENTER(ba, sd, B, b_box);
-  weno_body<DIR, WR, R>(sd, B);
+  __shared__ Dev sd;
+  Blk B;
+  const int b = batch_locate(ba, B);
+  pdl_wait();
+  if (B.x * WENO_NT >= __ldcg(&ba.dev[b].scal->nlist[B.y])) return;
+  batch_params(ba, b, sd);
+  weno_body<WR, R>(sd, B, (int)B.y);
 }
 
 // A persistent grid, as many CTAs as fit on the device at once, each
@@ -903,7 +951,7 @@ __global__ void __launch_bounds__(WENO_NT) kb_weno(BatchArgs ba) {
 // double-precision unit): one tile per CTA, so that more CTAs at different
 // phases share each multiprocessor and keep that unit busy.
 template <int DIR, bool HASW, class R, int TV, int NP>
-cudaError_t launch_one(const Dev &d, const FluxMaps &maps, int accumulate, cudaStream_t st) {
+cudaError_t launch_one(const Dev &d, const FluxMaps &maps, int accumulate, const Lane &st) {
   static int per_sm = 0;  // resident CTAs per multiprocessor (per instantiation)
   const size_t smem = flux_smem<DIR, HASW, R, TV, NP>(TV == 2);
   if (per_sm == 0) {
@@ -918,12 +966,12 @@ cudaError_t launch_one(const Dev &d, const FluxMaps &maps, int accumulate, cudaS
   const int ntiles = tg.count();
   const int cps = d.flux_cps[DIR] > 0 && d.flux_cps[DIR] < per_sm ? d.flux_cps[DIR] : per_sm;
   const int nb = FluxLayout<DIR, R, TV>::NBUF == 1 ? ntiles : (ntiles < cps * d.nsm ? ntiles : cps * d.nsm);
-  k_flux<DIR, HASW, R, TV, NP><<<nb, NTHREADS, smem, st>>>(maps, d, tg, accumulate);
+  st.run(k_flux<DIR, HASW, R, TV, NP>, nb, NTHREADS, smem, maps, d, tg, accumulate);
   return cudaGetLastError();
 }
 
 template <int DIR, bool HASW, class R, int TV>
-cudaError_t launch_np(const Dev &d, const FluxMaps &maps, int accumulate, cudaStream_t st) {
+cudaError_t launch_np(const Dev &d, const FluxMaps &maps, int accumulate, const Lane &st) {
   switch (d.npc) {
     case 1: return launch_one<DIR, HASW, R, TV, 1>(d, maps, accumulate, st);
     case 2: return launch_one<DIR, HASW, R, TV, 2>(d, maps, accumulate, st);
@@ -934,24 +982,31 @@ cudaError_t launch_np(const Dev &d, const FluxMaps &maps, int accumulate, cudaSt
 }
 
 template <int DIR, bool HASW, class R>
-cudaError_t launch_tv(const Dev &d, const FluxMaps (&maps)[2], int accumulate, cudaStream_t st) {
+cudaError_t launch_tv(const Dev &d, const FluxMaps (&maps)[3], int accumulate, const Lane &st) {
   if (d.keep) return launch_np<DIR, HASW, R, 2>(d, maps[0], accumulate, st);  // KEEP: the default tile
-  return d.tile[DIR] ? launch_np<DIR, HASW, R, 1>(d, maps[1], accumulate, st)
-                     : launch_np<DIR, HASW, R, 0>(d, maps[0], accumulate, st);
+  const int tile = flux_auto_tile(&d, 1, DIR);
+  if constexpr (DIR == 0)
+    if (tile == 2) return launch_np<DIR, HASW, R, 3>(d, maps[2], accumulate, st);
+  return tile ? launch_np<DIR, HASW, R, 1>(d, maps[1], accumulate, st)
+              : launch_np<DIR, HASW, R, 0>(d, maps[0], accumulate, st);
 }
 
-template <int DIR, int WR, class R>
-cudaError_t launch_weno_one(const Dev &d, cudaStream_t st) {
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // small CTAs: the flagged interfaces (a device-side count, often a few
-  // per cent of the slots) then spread evenly over the multiprocessors
-  long long need = (d.nslot[DIR] + WENO_NT - 1) / WENO_NT;
-  long long cap = (long long)(d.weno_cps > 0 ? d.weno_cps : 16) * sms;
-  unsigned nb = (unsigned)(need < cap ? need : cap);
-  if (nb == 0) nb = 1;
-  k_weno<DIR, WR, R><<<nb, WENO_NT, 0, st>>>(d);
+template <class R>
+cudaError_t weno_dispatch(const Dev &d, int dir, const Lane &st) {
+  unsigned nb = 1;
+  for (int a = 0; a < 3; ++a)
+    if (dir < 0 || a == dir) {
+      const unsigned k = weno_blocks(d, a, dir < 0);
+      nb = k > nb ? k : nb;
+    }
+  const dim3 grid(nb, dir < 0 ? 3 : 1);
+  switch ((d.weno + 1) / 2) {
+    case 1: st.run(k_weno<1, R>, grid, WENO_NT, 0, d, dir); break;
+    case 2: st.run(k_weno<2, R>, grid, WENO_NT, 0, d, dir); break;
+    case 3: st.run(k_weno<3, R>, grid, WENO_NT, 0, d, dir); break;
+    case 4: st.run(k_weno<4, R>, grid, WENO_NT, 0, d, dir); break;
+    default: return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 
@@ -975,12 +1030,16 @@ cudaError_t set_attr() {
   S2_A(true, 1, 1) S2_A(true, 1, 2) S2_A(true, 1, 3) S2_A(true, 1, 4)
   S2_A(false, 2, 1) S2_A(false, 2, 2) S2_A(false, 2, 3) S2_A(false, 2, 4)
   S2_A(true, 2, 1) S2_A(true, 2, 2) S2_A(true, 2, 3) S2_A(true, 2, 4)
+  if constexpr (DIR == 0) {
+    S2_A(false, 3, 1) S2_A(false, 3, 2) S2_A(false, 3, 3) S2_A(false, 3, 4)
+    S2_A(true, 3, 1) S2_A(true, 3, 2) S2_A(true, 3, 3) S2_A(true, 3, 4)
+  }
 #undef S2_A
   return e;
 }
 
 template <class R>
-cudaError_t flux_dispatch(const Dev &d, const FluxMaps (&maps)[2], int dir, int accumulate, cudaStream_t st) {
+cudaError_t flux_dispatch(const Dev &d, const FluxMaps (&maps)[3], int dir, int accumulate, const Lane &st) {
   const bool w = d.weno > 0;
   switch (dir) {
     case 0: return w ? launch_tv<0, true, R>(d, maps, accumulate, st) : launch_tv<0, false, R>(d, maps, accumulate, st);
@@ -1029,26 +1088,6 @@ cudaError_t make_map(const Dev &d, void *base, CUtensorMap *out) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <class R>
-cudaError_t weno_dispatch(const Dev &d, int dir, cudaStream_t st) {
-  const int wr = (d.weno + 1) / 2;
-  switch (dir * 10 + wr) {
-    case 1: return launch_weno_one<0, 1, R>(d, st);
-    case 2: return launch_weno_one<0, 2, R>(d, st);
-    case 3: return launch_weno_one<0, 3, R>(d, st);
-    case 4: return launch_weno_one<0, 4, R>(d, st);
-    case 11: return launch_weno_one<1, 1, R>(d, st);
-    case 12: return launch_weno_one<1, 2, R>(d, st);
-    case 13: return launch_weno_one<1, 3, R>(d, st);
-    case 14: return launch_weno_one<1, 4, R>(d, st);
-    case 21: return launch_weno_one<2, 1, R>(d, st);
-    case 22: return launch_weno_one<2, 2, R>(d, st);
-    case 23: return launch_weno_one<2, 3, R>(d, st);
-    case 24: return launch_weno_one<2, 4, R>(d, st);
-  }
-  return cudaErrorInvalidValue;
-}
-
 }  // namespace
 
 cudaError_t flux_set_attributes() {
@@ -1062,15 +1101,46 @@ cudaError_t flux_set_attributes() {
   return e;
 }
 
-cudaError_t launch_flux(const Dev &d, const FluxMaps (&maps)[2], int dir, int accumulate, cudaStream_t st) {
+// Tile variant 0 stands for the default: the wide tile, unless a narrower
+// one covers the boxes with a quarter fewer tiles.  64 boxes of 24^3 in
+// single precision took 46 us per x launch with 128 x 4 tiles, of which 24
+// columns were in use, and 33 us with 64 x 8.
+template <int DIR, int TV, class R>
+static long long tiles_of(const Dev *d, int count) {
+  long long t = 0;
+  for (int b = 0; b < count; ++b) t += TileGrid<DIR, TV, R>(d[b]).count();
+  return t;
+}
+
+template <int DIR, class R>
+static int auto_tile(const Dev *d, int count) {
+  const long long t0 = tiles_of<DIR, 0, R>(d, count), t1 = tiles_of<DIR, 1, R>(d, count);
+  int best = 4 * t1 <= 3 * t0;
+  if constexpr (DIR == 0)
+    if (4 * tiles_of<0, 3, R>(d, count) <= 3 * (best ? t1 : t0)) best = 2;
+  return best;
+}
+
+template <class R>
+static int auto_tile_dir(const Dev *d, int count, int dir) {
+  return dir == 0 ? auto_tile<0, R>(d, count) : (dir == 1 ? auto_tile<1, R>(d, count) : auto_tile<2, R>(d, count));
+}
+
+int flux_auto_tile(const Dev *d, int count, int dir) {
+  if (d->tile[dir] || d->keep || !d->auto_shape) return d->tile[dir];
+  return d->mixed ? auto_tile_dir<float>(d, count, dir) : auto_tile_dir<double>(d, count, dir);
+}
+
+cudaError_t launch_flux(const Dev &d, const FluxMaps (&maps)[3], int dir, int accumulate, const Lane &st) {
   return d.mixed ? flux_dispatch<float>(d, maps, dir, accumulate, st)
                  : flux_dispatch<double>(d, maps, dir, accumulate, st);
 }
 
 template <class R>
-cudaError_t make_maps_dir(const Dev &d, void *field, int f, FluxMaps (&maps)[3][2]) {
+cudaError_t make_maps_dir(const Dev &d, void *field, int f, FluxMaps (&maps)[3][3]) {
   cudaError_t e = make_map<0, 0, R>(d, field, &maps[0][0].m[f]);
   if (e == cudaSuccess) e = make_map<0, 1, R>(d, field, &maps[0][1].m[f]);
+  if (e == cudaSuccess) e = make_map<0, 3, R>(d, field, &maps[0][2].m[f]);
   if (e == cudaSuccess) e = make_map<1, 0, R>(d, field, &maps[1][0].m[f]);
   if (e == cudaSuccess) e = make_map<1, 1, R>(d, field, &maps[1][1].m[f]);
   if (e == cudaSuccess) e = make_map<2, 0, R>(d, field, &maps[2][0].m[f]);
@@ -1078,7 +1148,7 @@ cudaError_t make_maps_dir(const Dev &d, void *field, int f, FluxMaps (&maps)[3][
   return e;
 }
 
-cudaError_t flux_make_maps(const Dev &d, FluxMaps (&maps)[3][2]) {
+cudaError_t flux_make_maps(const Dev &d, FluxMaps (&maps)[3][3]) {
   void *fields[7] = {d.rho, d.u, d.v, d.ww, d.H, d.p, d.sens};
   const bool dbl = !d.mixed;
   cudaError_t e = cudaSuccess;
@@ -1090,7 +1160,7 @@ cudaError_t flux_make_maps(const Dev &d, FluxMaps (&maps)[3][2]) {
   return e;
 }
 
-cudaError_t launch_weno(const Dev &d, int dir, cudaStream_t st) {
+cudaError_t launch_weno(const Dev &d, int dir, const Lane &st) {
   return d.mixed ? weno_dispatch<float>(d, dir, st) : weno_dispatch<double>(d, dir, st);
 }
 
@@ -1113,6 +1183,8 @@ cudaError_t sel_np(const Dev &d, F &f) {
 template <class F, int DIR, class R>
 cudaError_t sel_w(const Dev &d, F &f) {
   if (d.keep) return d.weno > 0 ? sel_np<F, DIR, true, R, 2>(d, f) : sel_np<F, DIR, false, R, 2>(d, f);
+  if constexpr (DIR == 0)
+    if (d.tile[DIR] == 2) return d.weno > 0 ? sel_np<F, DIR, true, R, 3>(d, f) : sel_np<F, DIR, false, R, 3>(d, f);
   if (d.weno > 0) return d.tile[DIR] ? sel_np<F, DIR, true, R, 1>(d, f) : sel_np<F, DIR, true, R, 0>(d, f);
   return d.tile[DIR] ? sel_np<F, DIR, false, R, 1>(d, f) : sel_np<F, DIR, false, R, 0>(d, f);
 }
@@ -1163,35 +1235,24 @@ struct FluxBatchLaunch {
   const FluxMaps *maps;
   const void *tgs;
   int accumulate;
-  cudaStream_t st;
+  const Lane &st;
   template <int DIR, bool HASW, class R, int TV, int NP>
   cudaError_t run() {
-    kb_flux<DIR, HASW, R, TV, NP><<<total, NTHREADS, flux_smem<DIR, HASW, R, TV, NP>(TV == 2), st>>>(
-        ba, maps, (const TileGrid<DIR, TV, R> *)tgs, accumulate);
+    st.run(kb_flux<DIR, HASW, R, TV, NP>, total, NTHREADS, flux_smem<DIR, HASW, R, TV, NP>(TV == 2), ba, maps, (const TileGrid<DIR, TV, R> *)tgs, accumulate);
     return cudaGetLastError();
   }
 };
 
-template <int DIR, class R>
-cudaError_t weno_batch_wr(const Dev &d0, const BatchArgs &ba, unsigned total, cudaStream_t st) {
+template <class R>
+cudaError_t weno_batch_wr(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st) {
   switch ((d0.weno + 1) / 2) {
-    case 1: kb_weno<DIR, 1, R><<<total, WENO_NT, 0, st>>>(ba); break;
-    case 2: kb_weno<DIR, 2, R><<<total, WENO_NT, 0, st>>>(ba); break;
-    case 3: kb_weno<DIR, 3, R><<<total, WENO_NT, 0, st>>>(ba); break;
-    case 4: kb_weno<DIR, 4, R><<<total, WENO_NT, 0, st>>>(ba); break;
+    case 1: st.run(kb_weno<1, R>, total, WENO_NT, 0, ba); break;
+    case 2: st.run(kb_weno<2, R>, total, WENO_NT, 0, ba); break;
+    case 3: st.run(kb_weno<3, R>, total, WENO_NT, 0, ba); break;
+    case 4: st.run(kb_weno<4, R>, total, WENO_NT, 0, ba); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
-}
-
-template <class R>
-cudaError_t weno_batch_dir(const Dev &d0, const BatchArgs &ba, unsigned total, int dir, cudaStream_t st) {
-  switch (dir) {
-    case 0: return weno_batch_wr<0, R>(d0, ba, total, st);
-    case 1: return weno_batch_wr<1, R>(d0, ba, total, st);
-    case 2: return weno_batch_wr<2, R>(d0, ba, total, st);
-  }
-  return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -1201,22 +1262,14 @@ cudaError_t flux_batch_plan(const Dev &d, int dir, FluxBoxPlan *out) {
   return flux_select(d, dir, f);
 }
 
-unsigned weno_batch_blocks(const Dev &d, int dir) {
-  // as the single-box launch: enough 64-thread CTAs for every slot, at
-  // most 16 per multiprocessor (the list length is known on the device only)
-  long long need = (d.nslot[dir] + WENO_NT - 1) / WENO_NT;
-  long long cap = (long long)(d.weno_cps > 0 ? d.weno_cps : 16) * d.nsm;
-  return (unsigned)(need < 1 ? 1 : (need < cap ? need : cap));
-}
-
 cudaError_t launch_flux_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const FluxMaps *maps,
-                              const void *tgs, int dir, int accumulate, cudaStream_t st) {
+                              const void *tgs, int dir, int accumulate, const Lane &st) {
   FluxBatchLaunch f{ba, total, maps, tgs, accumulate, st};
   return flux_select(d0, dir, f);
 }
 
-cudaError_t launch_weno_batch(const Dev &d0, const BatchArgs &ba, unsigned total, int dir, cudaStream_t st) {
-  return d0.mixed ? weno_batch_dir<float>(d0, ba, total, dir, st) : weno_batch_dir<double>(d0, ba, total, dir, st);
+cudaError_t launch_weno_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st) {
+  return d0.mixed ? weno_batch_wr<float>(d0, ba, total, st) : weno_batch_wr<double>(d0, ba, total, st);
 }
 
 }  // namespace s2

@@ -128,10 +128,13 @@ struct Dev {
   double vol_inv;          // 1 / sum(dV) / (dx dz) for the forcing
   int viscous, wall_y, weno, force;
   int fx;                  // 1: FP64 with 1/dx, eta_y, 1/dz in the range of the fixed-point path (s2_fixed.cuh)
+  int fx_tx;               // tile width of its gradient and viscous passes (fx_auto_tx)
   int mixed;               // 0: FP64 everywhere; 1: FP32 primitives and flux arithmetic, FP64 state
-  int tile[3];             // flux tile variant per direction (0 default, 1 narrow)
+  int tile[3];             // flux tile variant per direction (0 default, 1 narrow; 2 narrowest, by flux_auto_tile only)
   int flux_cps[3];         // persistent flux grids, per direction: resident CTAs per SM to use (0: all that fit)
   int zs;                  // planes per CTA of the z-marching passes (mixed path)
+  int auto_shape;          // 1: tiles and planes left at their defaults are chosen from the grid
+  int zs_set;              // the same as asked for by the user (ZS_DEFAULT: chosen by z_auto_planes)
   int weno_cps;            // WENO grids: CTAs per SM
   int nsm;                 // multiprocessors of the device
   unsigned long long wait_ns;  // limit of a kernel's wait for an asynchronous copy
@@ -195,18 +198,22 @@ struct BatchArgs {
   int nbox;
 };
 
-// The box of this CTA (binary search of the work list) and its box-local
-// block coordinates.
+// The box of this CTA (search of the work list) and its box-local block
+// coordinates.
 __device__ __forceinline__ int batch_locate(const BatchArgs &ba, Blk &B) {
   __shared__ int sbox;
-  if (threadIdx.x == 0) {
-    int lo = 0, hi = ba.nbox - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (ba.grid[mid].start <= blockIdx.x) lo = mid;
-      else hi = mid - 1;
+  if (threadIdx.x < 32) {
+    // the last entry whose start is not beyond this CTA: 32 entries are
+    // tried per round, so 1024 boxes take two dependent loads
+    int lo = 0, n = ba.nbox;
+    while (n > 1) {
+      const int step = (n + 31) / 32, at = (int)threadIdx.x * step;
+      const unsigned in = __ballot_sync(0xffffffffu, at < n && ba.grid[lo + at].start <= blockIdx.x);
+      const int h = (31 - __clz(in)) * step;
+      lo += h;
+      n = min(step, n - h);
     }
-    sbox = lo;
+    if (threadIdx.x == 0) sbox = lo;
   }
   __syncthreads();
   const int b = sbox;
@@ -222,14 +229,19 @@ __device__ __forceinline__ int batch_locate(const BatchArgs &ba, Blk &B) {
   return b;
 }
 
-// The same, and the box's parameters copied to shared memory (sd).
-__device__ __forceinline__ int batch_enter(const BatchArgs &ba, Dev &sd, Blk &B) {
-  const int b = batch_locate(ba, B);
+// The parameters of box b copied to shared memory (sd).
+__device__ __forceinline__ void batch_params(const BatchArgs &ba, int b, Dev &sd) {
   static_assert(sizeof(Dev) % 8 == 0, "Dev is copied in 8-byte words");
   const unsigned long long *src = (const unsigned long long *)(ba.dev + b);
   unsigned long long *dst = (unsigned long long *)&sd;
   for (int i = threadIdx.x; i < (int)(sizeof(Dev) / 8); i += blockDim.x) dst[i] = src[i];
   __syncthreads();
+}
+
+// Both.
+__device__ __forceinline__ int batch_enter(const BatchArgs &ba, Dev &sd, Blk &B) {
+  const int b = batch_locate(ba, B);
+  batch_params(ba, b, sd);
   return b;
 }
 
@@ -241,7 +253,8 @@ __device__ __forceinline__ int batch_enter(const BatchArgs &ba, Dev &sd, Blk &B)
   Blk BL;                                     \
   const int BOX = batch_enter(BA, D##_s, BL); \
   const Dev &D = D##_s;                       \
-  (void)BOX
+  (void)BOX;                                  \
+  pdl_wait()
 
 // Typed views of the fields of a Dev in the arithmetic type R.
 template <class R>
@@ -393,6 +406,31 @@ __device__ __forceinline__ double rcp_pos(double x) {
   return fma(r, e, r);
 }
 __device__ __forceinline__ float rcp_pos(float x) { return 1.0f / x; }
+
+// sqrt(x) for x > 0 in double precision: a single-precision approximate
+// 1/sqrt(x) gives s = x r, and two steps s <- s + (x - s^2) r/2 square its
+// relative error (2^-22 -> 2^-44 -> below rounding): 5 FP64 operations, about
+// half of the library's.  Outside [2^-100, 2^100], and for what is not
+// positive, the library root.
+__device__ __forceinline__ double sqrt_pos(double x) {
+  const int ex = (int)((unsigned)__double2hiint(x) >> 20) - 1023;  // the sign bit makes it large
+  if (ex < -100 || ex > 100) return sqrt(x);
+  float rf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(d2f_int(x)));
+  const double r = f2d_int(rf), h = f2d_int(0.5f * rf);
+  double s = x * r;
+  s = fma(fma(-s, s, x), h, s);
+  return fma(fma(-s, s, x), h, s);
+}
+__device__ __forceinline__ float sqrt_pos(float x) { return sqrtf(x); }
+
+// The larger magnitude, compared on the integer pipe (a NaN counts as
+// larger than every number).
+__device__ __forceinline__ double max_mag(double m, double x) {
+  const long long a = __double_as_longlong(m), b = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return __longlong_as_double(a > b ? a : b);
+}
+__device__ __forceinline__ float max_mag(float m, float x) { return fmaxf(m, fabsf(x)); }
 
 // x^e for e >= 0 by binary powering, starting from the lowest set bit
 // (no multiplications by 1, no square after the last bit).
@@ -670,17 +708,52 @@ struct FluxMaps {
   CUtensorMap m[7];
 };
 
+// Programmatic dependent launch: a kernel of the step sequence may be put on
+// the device as soon as the one before it has ended, its launch overlapping
+// that kernel's last writes, and waits here, before it touches anything a
+// kernel wrote, until they are visible.  Every thread of every kernel of the
+// sequence waits, so a kernel that has finished vouches for all those before
+// it.  Without the launch attribute the instruction does nothing.  A step of
+// 27 or 34 short launches went from 125.8 to 121.8 us (32^3, FP64) and from
+// 142.1 to 136.6 us (37 x 29 x 19, mixed); letting the next kernel's CTAs in
+// from the start of the one before (launch_dependents) instead made them
+// 201 and 176 us.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A stream and whether the next launch on it may overlap the end of the
+// kernel before it (not the first of a sequence, nor one with further
+// dependencies from other streams, nor under the per-kernel profile, whose
+// events would then bracket the overlap).
+struct Lane {
+  cudaStream_t st;
+  bool pdl;
+  template <class... P, class... A>
+  void run(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, A &&...args) const {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // the callers read the error
+  }
+};
+
 // Launch helpers (defined in the kernel translation units).
-cudaError_t flux_make_maps(const Dev &d, FluxMaps (&maps)[3][2]);
-cudaError_t launch_flux(const Dev &d, const FluxMaps (&maps)[2], int dir, int accumulate, cudaStream_t st);
-cudaError_t launch_weno(const Dev &d, int dir, cudaStream_t st);
-cudaError_t launch_grad(const Dev &d, cudaStream_t st);
-cudaError_t launch_visc(const Dev &d, cudaStream_t st);
+cudaError_t flux_make_maps(const Dev &d, FluxMaps (&maps)[3][3]);
+cudaError_t launch_flux(const Dev &d, const FluxMaps (&maps)[3], int dir, int accumulate, const Lane &st);
+cudaError_t launch_weno(const Dev &d, int dir, const Lane &st);  // dir < 0: all three
+cudaError_t launch_grad(const Dev &d, const Lane &st);
+cudaError_t launch_visc(const Dev &d, const Lane &st);
 // Forcing partials the viscous launch writes itself (mixed path), else 0;
 // CTAs of the mixed path's z-marching passes.
 int visc_force_partials(const Dev &d);
 long long z_pass_blocks(const Dev &d);
-cudaError_t launch_apply(const Dev &d, cudaStream_t st);
+cudaError_t launch_apply(const Dev &d, const Lane &st);
 cudaError_t flux_set_attributes();
 
 // Batched launches (one launch for every box of a batch group; the boxes
@@ -694,18 +767,23 @@ struct FluxBoxPlan {
   bool persistent;  // CTAs walk several tiles
 };
 cudaError_t flux_batch_plan(const Dev &d, int dir, FluxBoxPlan *out);
-unsigned weno_batch_blocks(const Dev &d, int dir);
+unsigned weno_blocks(const Dev &d, int dir, bool all);
 cudaError_t launch_flux_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const FluxMaps *maps,
-                              const void *tgs, int dir, int accumulate, cudaStream_t st);
-cudaError_t launch_weno_batch(const Dev &d0, const BatchArgs &ba, unsigned total, int dir, cudaStream_t st);
+                              const void *tgs, int dir, int accumulate, const Lane &st);
+cudaError_t launch_weno_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st);
 // gradient and viscous passes: grid of one box (x, y, z blocks)
 void z_pass_grid(const Dev &d, unsigned g[3]);
-// Planes per CTA of the z-marching passes: compiled for 4, 8, 12, 16 and
-// 24 (the forcing partials are sized for the smallest).
-constexpr int ZS_MIN = 4, ZS_DEFAULT = 12;
-cudaError_t launch_grad_batch(const Dev &d0, const BatchArgs &ba, unsigned total, cudaStream_t st);
-cudaError_t launch_visc_batch(const Dev &d0, const BatchArgs &ba, unsigned total, cudaStream_t st);
-cudaError_t launch_apply_batch(const Dev &d0, const BatchArgs &ba, unsigned total, cudaStream_t st);
+// Planes per CTA of the z-marching passes: compiled for 1, 2, 4, 8, 12, 16
+// and 24 (the forcing partials are sized for the smallest), and the choice
+// for boxes that share their launches.
+constexpr int ZS_MIN = 1, ZS_DEFAULT = 12;
+int z_auto_planes(const Dev *d, int count);
+int fx_auto_tx(const Dev *d, int count);  // the same for the FP64 tiles
+// The tile variant of a direction for boxes that share their launches.
+int flux_auto_tile(const Dev *d, int count, int dir);
+cudaError_t launch_grad_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st);
+cudaError_t launch_visc_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st);
+cudaError_t launch_apply_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st);
 
 // Gas constants (R, c_v, c_p, viscosity law) of a Dev from s2_gas.
 void set_gas(Dev &d, const s2_gas *gas);

@@ -167,6 +167,16 @@ __device__ __forceinline__ void dt_block_max(const Dev &d, double sr, int want_d
   }
 }
 
+// The per-RHS counters of the hybrid scheme (flagged interfaces and the
+// three list lengths) start at zero with the primitive pass, which runs
+// after every reader of the evaluation before.
+__device__ __forceinline__ void reset_counts(const Dev &d, long long q) {
+  if (q == 0 && d.weno) {
+    d.scal->wcount = 0;
+    for (int a = 0; a < 4; ++a) d.scal->nlist[a] = 0;
+  }
+}
+
 // Whether this launch computes the CFL partials: decided once per CTA (the
 // step counter is 64-bit, and a 64-bit remainder per thread would go
 // through the double-precision unit).
@@ -210,6 +220,7 @@ template <bool TP>
 __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk &B, int stage0) {
   long long q = (long long)B.x * NT + threadIdx.x;
   const View<double> V = view<double>(d);
+  reset_counts(d, q);
   const int want_dt = block_want_dt(d, stage0);
   double sr = 0.0;
   unsigned fe[FX_TH] = {0}, fm[FX_NMIN] = {0};
@@ -267,6 +278,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
 
 template <bool TP>
 __global__ void __launch_bounds__(NT) k_prims(Dev d, int stage0) {
+  pdl_wait();
   prims_body<TP>(d, grid_blk(), stage0);
 }
 
@@ -286,6 +298,7 @@ __global__ void __launch_bounds__(NT) kb_prims(BatchArgs ba, int stage0) {
 __device__ __forceinline__ void prims_mixed_body(const Dev &__restrict__ d, const Blk &B, int stage0) {
   long long q = (long long)B.x * NT + threadIdx.x;
   const View<float> V = view<float>(d);
+  reset_counts(d, q);
   const int want_dt = block_want_dt(d, stage0);
   const Consts<float> &K = d.kf;
   double sr = 0.0;
@@ -346,7 +359,10 @@ __device__ __forceinline__ void prims_mixed_body(const Dev &__restrict__ d, cons
   dt_block_max(d, sr, want_dt, B.x);
 }
 
-__global__ void __launch_bounds__(NT) k_prims_mixed(Dev d, int stage0) { prims_mixed_body(d, grid_blk(), stage0); }
+__global__ void __launch_bounds__(NT) k_prims_mixed(Dev d, int stage0) {
+  pdl_wait();
+  prims_mixed_body(d, grid_blk(), stage0);
+}
 
 __global__ void __launch_bounds__(NT) kb_prims_mixed(BatchArgs ba, int stage0) {
   S2_BATCH_ENTER(ba, sd, B, b_box);
@@ -374,7 +390,10 @@ __device__ __forceinline__ void dt_final_body(const Dev &__restrict__ d, int npa
   }
 }
 
-__global__ void k_dt_final(Dev d, int nparts) { dt_final_body(d, nparts); }
+__global__ void k_dt_final(Dev d, int nparts) {
+  pdl_wait();
+  dt_final_body(d, nparts);
+}
 
 // one CTA per box; nparts[b]: box b's CFL partials
 __global__ void __launch_bounds__(NT) kb_dt_final(BatchArgs ba, const int *nparts) {
@@ -474,6 +493,7 @@ __device__ __forceinline__ void ghost_prim_body(const Dev &__restrict__ d, const
 
 template <class R>
 __global__ void __launch_bounds__(NT) k_ghost_prim(Dev d) {
+  pdl_wait();
   ghost_prim_body<R>(d, grid_blk());
 }
 
@@ -516,6 +536,7 @@ __device__ __forceinline__ void ghost_aux_body(const Dev &__restrict__ d, const 
 
 template <class R>
 __global__ void __launch_bounds__(NT) k_ghost_aux(Dev d) {
+  pdl_wait();
   ghost_aux_body<R>(d, grid_blk());
 }
 
@@ -551,6 +572,7 @@ __device__ __forceinline__ void force_partial_body(const Dev &__restrict__ d, co
 
 template <class R>
 __global__ void __launch_bounds__(NT) k_force_partial(Dev d) {
+  pdl_wait();
   force_partial_body<R>(d, grid_blk());
 }
 
@@ -569,22 +591,15 @@ __device__ __forceinline__ void force_final_body(const Dev &__restrict__ d, int 
   if (threadIdx.x == 0) d.scal->force = -v[0] * d.vol_inv;
 }
 
-__global__ void k_force_final(Dev d, int nparts) { force_final_body(d, nparts); }
+__global__ void k_force_final(Dev d, int nparts) {
+  pdl_wait();
+  force_final_body(d, nparts);
+}
 
 // one CTA per box; nparts[b]: box b's forcing partials
 __global__ void __launch_bounds__(NT) kb_force_final(BatchArgs ba, const int *nparts) {
   S2_BATCH_ENTER(ba, sd, B, b);
   force_final_body(sd, nparts[b]);
-}
-
-// The per-RHS counters of the hybrid scheme (flagged interfaces and the
-// three list lengths), zeroed for every box of a batch in one launch.
-__global__ void __launch_bounds__(NT) kb_reset_counts(BatchArgs ba) {
-  S2_BATCH_ENTER(ba, sd, B, b_box);
-  if (threadIdx.x == 0) {
-    sd.scal->wcount = 0;
-    for (int a = 0; a < 4; ++a) sd.scal->nlist[a] = 0;
-  }
 }
 
 // ----------------------------------------------------------------- update
@@ -634,6 +649,7 @@ __device__ __forceinline__ void update_body(const Dev &__restrict__ d, const Blk
 }
 
 __global__ void __launch_bounds__(NT) k_update(Dev d, double gk, double rk1, int stage) {
+  pdl_wait();
   update_body(d, grid_blk(), gk, rk1, stage);
 }
 
@@ -695,6 +711,7 @@ __device__ __forceinline__ void update_mixed_body(const Dev &__restrict__ d, con
 }
 
 __global__ void __launch_bounds__(NT) k_update_mixed(Dev d, double gk, double rk1, int stage) {
+  pdl_wait();
   update_mixed_body(d, grid_blk(), gk, rk1, stage);
 }
 
@@ -832,7 +849,7 @@ struct s2_solver {
   long long launches;
   size_t rsize;         // bytes of the arithmetic type (8 FP64, 4 mixed)
   double *rhs_stage;    // staging of s2_rhs output
-  FluxMaps fmaps[3][2];  // tensor maps of the staged fields, per direction and tile variant
+  FluxMaps fmaps[3][3];  // tensor maps of the staged fields, per direction and tile variant
   // second stream for the WENO corrections of a direction, which run while
   // the flux kernels of the next directions do (fork after each flux
   // kernel, join before the viscous pass)
@@ -911,48 +928,45 @@ cudaError_t run(Trace *tr, cudaStream_t st, int kind, int nkernels, F f) {
 }
 
 // One RHS evaluation (all terms up to the forcing reduction).
-cudaError_t enqueue_rhs(s2_solver *s, int stage0, Trace *tr) {
+// first: nothing was launched on the stream by this sequence yet.
+cudaError_t enqueue_rhs(s2_solver *s, int stage0, Trace *tr, bool first) {
   const Dev &d = s->d;
-  cudaStream_t st = s->stream;
+  const bool pdl = !(tr && tr->timed) && d.auto_shape;
+  Lane st{s->stream, pdl && !first};
   cudaError_t e;
   unsigned nb = (unsigned)((d.n + NT - 1) / NT);
   long long nghost = 2LL * GH * ((long long)d.ny * d.nz + (long long)d.nx * d.nz + (long long)d.nx * d.ny);
   unsigned ngb = (unsigned)((nghost + NT - 1) / NT);
-  e = run(tr, st, S2_PROF_PRIMS, 1, [&] {
-    if (d.mixed) k_prims_mixed<<<nb, NT, 0, st>>>(d, stage0);
-    else if (d.kd.tp) k_prims<true><<<nb, NT, 0, st>>>(d, stage0);
-    else k_prims<false><<<nb, NT, 0, st>>>(d, stage0);
+  e = run(tr, st.st, S2_PROF_PRIMS, 1, [&] {
+    if (d.mixed) st.run(k_prims_mixed, nb, NT, 0, d, stage0);
+    else if (d.kd.tp) st.run(k_prims<true>, nb, NT, 0, d, stage0);
+    else st.run(k_prims<false>, nb, NT, 0, d, stage0);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
+  st.pdl = pdl;
   if (stage0 && d.cfl > 0.0) {
-    e = run(tr, st, S2_PROF_DT, 1, [&] {
-      k_dt_final<<<1, NT, 0, st>>>(d, (int)nb);
+    e = run(tr, st.st, S2_PROF_DT, 1, [&] {
+      st.run(k_dt_final, 1, NT, 0, d, (int)nb);
       return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
   }
-  e = run(tr, st, S2_PROF_GHOST, 1, [&] {
-    if (d.mixed) k_ghost_prim<float><<<ngb, NT, 0, st>>>(d);
-    else k_ghost_prim<double><<<ngb, NT, 0, st>>>(d);
+  e = run(tr, st.st, S2_PROF_GHOST, 1, [&] {
+    if (d.mixed) st.run(k_ghost_prim<float>, ngb, NT, 0, d);
+    else st.run(k_ghost_prim<double>, ngb, NT, 0, d);
     return cudaGetLastError();
   });
   if (e != cudaSuccess) return e;
   if (d.viscous || d.weno) {
-    e = run(tr, st, S2_PROF_GRAD, 1, [&] { return launch_grad(d, st); });
+    e = run(tr, st.st, S2_PROF_GRAD, 1, [&] { return launch_grad(d, st); });
     if (e != cudaSuccess) return e;
-    e = run(tr, st, S2_PROF_GHOST_AUX, 1, [&] {
-      if (d.mixed) k_ghost_aux<float><<<ngb, NT, 0, st>>>(d);
-      else k_ghost_aux<double><<<ngb, NT, 0, st>>>(d);
+    e = run(tr, st.st, S2_PROF_GHOST_AUX, 1, [&] {
+      if (d.mixed) st.run(k_ghost_aux<float>, ngb, NT, 0, d);
+      else st.run(k_ghost_aux<double>, ngb, NT, 0, d);
       return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
-  }
-  if (d.weno) {
-    // wcount and the three list lengths are adjacent
-    if ((e = cudaMemsetAsync(&d.scal->wcount, 0, sizeof(unsigned long long) + 4 * sizeof(unsigned), st)) !=
-        cudaSuccess)
-      return e;
   }
   // Outside the per-kernel profile, each direction's WENO corrections run
   // on the side stream as soon as its flux kernel has listed the flagged
@@ -964,20 +978,24 @@ cudaError_t enqueue_rhs(s2_solver *s, int stage0, Trace *tr) {
   // and measured slower with the extra branch.
   const bool overlap = d.weno && !d.mixed && !(tr && tr->timed);
   for (int dir = 0; dir < 3; ++dir) {
-    e = run(tr, st, S2_PROF_FLUX_X + dir, 1, [&] { return launch_flux(d, s->fmaps[dir], dir, dir > 0, st); });
+    e = run(tr, st.st, S2_PROF_FLUX_X + dir, 1, [&] { return launch_flux(d, s->fmaps[dir], dir, dir > 0, st); });
     if (e != cudaSuccess) return e;
     if (overlap) {
-      if ((e = cudaEventRecord(s->ev_flux[dir], st)) != cudaSuccess) return e;
+      if ((e = cudaEventRecord(s->ev_flux[dir], st.st)) != cudaSuccess) return e;
       if ((e = cudaStreamWaitEvent(s->side, s->ev_flux[dir], 0)) != cudaSuccess) return e;
-      if ((e = launch_weno(d, dir, s->side)) != cudaSuccess) return e;
+      if ((e = launch_weno(d, dir, Lane{s->side, false})) != cudaSuccess) return e;
       if (tr) tr->count[S2_PROF_WENO] += 1;
     }
   }
   if (overlap) {
     if ((e = cudaEventRecord(s->ev_join, s->side)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(st, s->ev_join, 0)) != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(st.st, s->ev_join, 0)) != cudaSuccess) return e;
+    st.pdl = false;  // the next kernel waits for the side stream too
   } else if (d.weno) {
-    e = run(tr, st, S2_PROF_WENO, 3, [&] {
+    // one launch for the three directions (not in branch mode, see
+    // enqueue_member)
+    e = run(tr, st.st, S2_PROF_WENO, d.auto_shape ? 1 : 3, [&] {
+      if (d.auto_shape) return launch_weno(d, -1, st);
       cudaError_t r = cudaSuccess;
       for (int dir = 0; dir < 3 && r == cudaSuccess; ++dir) r = launch_weno(d, dir, st);
       return r;
@@ -985,22 +1003,23 @@ cudaError_t enqueue_rhs(s2_solver *s, int stage0, Trace *tr) {
     if (e != cudaSuccess) return e;
   }
   if (d.viscous) {
-    e = run(tr, st, S2_PROF_VISC, 1, [&] { return launch_visc(d, st); });
+    e = run(tr, st.st, S2_PROF_VISC, 1, [&] { return launch_visc(d, st); });
     if (e != cudaSuccess) return e;
   } else if (d.weno) {
-    e = run(tr, st, S2_PROF_APPLY, 1, [&] { return launch_apply(d, st); });
+    e = run(tr, st.st, S2_PROF_APPLY, 1, [&] { return launch_apply(d, st); });
     if (e != cudaSuccess) return e;
   }
+  st.pdl = pdl;
   if (d.force) {
     const int fused = visc_force_partials(d);  // partials already written by the viscous pass
-    e = run(tr, st, S2_PROF_FORCE, fused ? 1 : 2, [&] {
+    e = run(tr, st.st, S2_PROF_FORCE, fused ? 1 : 2, [&] {
       if (fused) {
-        k_force_final<<<1, NT, 0, st>>>(d, fused);
+        st.run(k_force_final, 1, NT, 0, d, fused);
         return cudaGetLastError();
       }
-      if (d.mixed) k_force_partial<float><<<NRED, NT, 0, st>>>(d);
-      else k_force_partial<double><<<NRED, NT, 0, st>>>(d);
-      k_force_final<<<1, NT, 0, st>>>(d, NRED);
+      if (d.mixed) st.run(k_force_partial<float>, NRED, NT, 0, d);
+      else st.run(k_force_partial<double>, NRED, NT, 0, d);
+      st.run(k_force_final, 1, NT, 0, d, NRED);
       return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
@@ -1012,11 +1031,12 @@ cudaError_t enqueue_step(s2_solver *s, Trace *tr) {
   const Dev &d = s->d;
   unsigned nb = (unsigned)((d.n + NT - 1) / NT);
   cudaError_t e;
-  for (int st = 0; st < 3; ++st) {
-    if ((e = enqueue_rhs(s, st == 0, tr)) != cudaSuccess) return e;
+  const Lane st{s->stream, !(tr && tr->timed) && d.auto_shape};
+  for (int stage = 0; stage < 3; ++stage) {
+    if ((e = enqueue_rhs(s, stage == 0, tr, stage == 0)) != cudaSuccess) return e;
     e = run(tr, s->stream, S2_PROF_UPDATE, 1, [&] {
-      if (d.mixed) k_update_mixed<<<nb, NT, 0, s->stream>>>(d, RK_G[st], RK_R[st + 1], st);
-      else k_update<<<nb, NT, 0, s->stream>>>(d, RK_G[st], RK_R[st + 1], st);
+      if (d.mixed) st.run(k_update_mixed, nb, NT, 0, d, RK_G[stage], RK_R[stage + 1], stage);
+      else st.run(k_update, nb, NT, 0, d, RK_G[stage], RK_R[stage + 1], stage);
       return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
@@ -1319,7 +1339,10 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.tile[0] = 0;
   d.tile[1] = d.tile[2] = d.mixed;
   for (int a = 0; a < 3; ++a) d.flux_cps[a] = 0;
-  d.zs = ZS_DEFAULT;
+  d.auto_shape = 1;
+  d.zs_set = ZS_DEFAULT;
+  d.zs = z_auto_planes(&d, 1);
+  d.fx_tx = fx_auto_tx(&d, 1);
   d.weno_cps = 16;
   // scheme constants in both arithmetic types
   {
@@ -1718,7 +1741,8 @@ int s2_set_tuning(s2_solver *s, const s2_tuning *t) {
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) return S2_ECUDA;
   for (int a = 0; a < 3; ++a) s->d.tile[a] = t->tiles[a];
   for (int a = 0; a < 3; ++a) s->d.flux_cps[a] = t->flux_ctas_per_sm[a];
-  s->d.zs = t->z_planes ? t->z_planes : ZS_DEFAULT;
+  s->d.zs_set = t->z_planes ? t->z_planes : ZS_DEFAULT;
+  s->d.zs = s->d.zs_set == ZS_DEFAULT ? z_auto_planes(&s->d, 1) : s->d.zs_set;
   s->d.weno_cps = t->weno_ctas_per_sm ? t->weno_ctas_per_sm : 16;
   if (s->graph_ready) {
     cudaGraphExecDestroy(s->graph);
@@ -1731,7 +1755,7 @@ int s2_get_tuning(const s2_solver *s, s2_tuning *t) {
   if (!s || !t) return S2_EINVAL;
   for (int a = 0; a < 3; ++a) t->tiles[a] = s->d.tile[a];
   for (int a = 0; a < 3; ++a) t->flux_ctas_per_sm[a] = s->d.flux_cps[a];
-  t->z_planes = s->d.zs;
+  t->z_planes = s->d.zs_set;
   t->weno_ctas_per_sm = s->d.weno_cps;
   return S2_OK;
 }
@@ -1767,7 +1791,7 @@ int s2_set_clock(s2_solver *s, double t, long long step, double dt) {
 int s2_rhs(s2_solver *s, double *rhs, int where) {
   if (!s || !rhs || (where != S2_HOST && where != S2_DEVICE)) return S2_EINVAL;
   DeviceGuard guard(s->device);
-  cudaError_t e = enqueue_rhs(s, 0, nullptr);
+  cudaError_t e = enqueue_rhs(s, 0, nullptr, true);
   if (e != cudaSuccess) return S2_ECUDA;
   unsigned nb = (unsigned)((s->d.n + NT - 1) / NT);
   size_t bytes = NV * (size_t)s->d.n * sizeof(double);
@@ -1886,9 +1910,7 @@ enum BatchClass {
   BC_FLUX0,
   BC_FLUX1,
   BC_FLUX2,
-  BC_WENO0,
-  BC_WENO1,
-  BC_WENO2,
+  BC_WENO,   // three rows of CTAs per box, one per direction
   BC_FORCE,  // grid-stride forcing partials (NRED CTAs per box)
   BC_ONE,    // one CTA per box
   BC_COUNT
@@ -1896,6 +1918,7 @@ enum BatchClass {
 
 struct BatchGroup {
   std::vector<s2_solver *> members;
+  Dev d0;               // parameters that select the kernels: the first member's, with the group's tiles and planes
   cudaStream_t stream;  // the first member's: this group's branch of the step graph
   void *mem;            // the device tables, one block
   Dev *dev;             // [n] parameters of the boxes
@@ -1927,7 +1950,8 @@ namespace {
 bool same_kernels(const Dev &a, const Dev &b) {
   return a.mixed == b.mixed && a.npc == b.npc && a.npv == b.npv && a.weno == b.weno && a.kd.tp == b.kd.tp &&
          a.tile[0] == b.tile[0] && a.tile[1] == b.tile[1] && a.tile[2] == b.tile[2] && a.viscous == b.viscous &&
-         a.force == b.force && (a.cfl > 0.0) == (b.cfl > 0.0) && a.zs == b.zs;
+         a.force == b.force && (a.cfl > 0.0) == (b.cfl > 0.0) && a.zs_set == b.zs_set &&
+         (!a.force || !a.mixed || a.zs == b.zs);  // the forcing is summed by plane groups, so those keep their solo planes
 }
 
 void *batch_alloc(s2_solver *s, size_t bytes) {
@@ -1951,9 +1975,20 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // The group's work lists and tables, built on the host and copied once.
 int group_setup(BatchGroup &g) {
   const int n = (int)g.members.size();
-  const Dev &d0 = g.members[0]->d;
   std::vector<Dev> devs(n);
   for (int b = 0; b < n; ++b) devs[b] = g.members[b]->d;
+  // launch shapes for all boxes of the group together
+  int tile[3];
+  for (int dir = 0; dir < 3; ++dir) tile[dir] = flux_auto_tile(devs.data(), n, dir);
+  const int zs = devs[0].zs_set != ZS_DEFAULT || devs[0].force ? devs[0].zs : z_auto_planes(devs.data(), n);
+  const int tx = fx_auto_tx(devs.data(), n);
+  for (Dev &d : devs) {
+    d.fx_tx = tx;
+    for (int dir = 0; dir < 3; ++dir) d.tile[dir] = tile[dir];
+    d.zs = zs;
+  }
+  g.d0 = devs[0];
+  const Dev &d0 = g.d0;
   std::vector<std::vector<BoxGrid>> grids(BC_COUNT, std::vector<BoxGrid>(n + 1));
   std::vector<int> ndt(n), nforce(n);
   FluxBoxPlan fp[3];
@@ -1983,6 +2018,7 @@ int group_setup(BatchGroup &g) {
     z_pass_grid(d, zg);
     set(BC_GRAD, b, zg[0], zg[1], zg[2]);
     set(BC_VISC, b, zg[0], zg[1], zg[2]);
+    unsigned nweno = 1;
     for (int dir = 0; dir < 3; ++dir) {
       const FluxBoxPlan &pl = plans[3 * b + dir];
       unsigned c = (unsigned)pl.tiles;
@@ -1995,10 +2031,11 @@ int group_setup(BatchGroup &g) {
       }
       set(BC_FLUX0 + dir, b, c, 1, 1);
       // WENO: the solo launch's CTAs shared out by interface slots
-      const unsigned solo = weno_batch_blocks(d, dir);
-      unsigned w = (unsigned)(16.0 * d.nsm * (double)d.nslot[dir] / (double)slots_sum[dir]) + 1;
-      set(BC_WENO0 + dir, b, w < solo ? w : solo, 1, 1);
+      const unsigned solo = weno_blocks(d, dir, true);
+      const unsigned w = (unsigned)(8.0 * d.nsm * (double)d.nslot[dir] / (double)slots_sum[dir]) + 1;
+      if ((w < solo ? w : solo) > nweno) nweno = w < solo ? w : solo;
     }
+    set(BC_WENO, b, nweno, 3, 1);
     set(BC_FORCE, b, NRED, 1, 1);
     set(BC_ONE, b, 1, 1, 1);
     ndt[b] = (int)nb;
@@ -2040,7 +2077,7 @@ int group_setup(BatchGroup &g) {
   for (int b = 0; b < n; ++b)
     for (int dir = 0; dir < 3; ++dir) {
       const s2_solver *m = g.members[b];
-      memcpy(host.data() + o_maps[dir] + sizeof(FluxMaps) * b, &m->fmaps[dir][d0.tile[dir] && !d0.keep ? 1 : 0],
+      memcpy(host.data() + o_maps[dir] + sizeof(FluxMaps) * b, &m->fmaps[dir][d0.keep ? 0 : d0.tile[dir]],
              sizeof(FluxMaps));
       memcpy(host.data() + o_tg[dir] + (size_t)fp[dir].tg_size * b, plans[3 * b + dir].tg, fp[dir].tg_size);
     }
@@ -2070,61 +2107,95 @@ int group_setup(BatchGroup &g) {
 // One RK3 step of every box of a group: the stage sequence of
 // enqueue_step, each kernel launched once for all boxes.
 cudaError_t enqueue_group_step(BatchGroup &g) {
-  const Dev &d0 = g.members[0]->d;
+  const Dev &d0 = g.d0;
   const int n = (int)g.members.size();
-  cudaStream_t st = g.stream;
+  Lane st{g.stream, false};  // the first kernel follows the fork
   auto ba = [&](int c) { return BatchArgs{g.dev, g.grid[c], n}; };
   long long cnt = 0;
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) {
     ++cnt;
+    st.pdl = true;
     if (e == cudaSuccess) e = r;
   };
   for (int stage = 0; stage < 3 && e == cudaSuccess; ++stage) {
     const int stage0 = stage == 0;
-    if (d0.mixed) kb_prims_mixed<<<g.total[BC_PRIMS], NT, 0, st>>>(ba(BC_PRIMS), stage0);
-    else if (d0.kd.tp) kb_prims<true><<<g.total[BC_PRIMS], NT, 0, st>>>(ba(BC_PRIMS), stage0);
-    else kb_prims<false><<<g.total[BC_PRIMS], NT, 0, st>>>(ba(BC_PRIMS), stage0);
+    if (d0.mixed) st.run(kb_prims_mixed, g.total[BC_PRIMS], NT, 0, ba(BC_PRIMS), stage0);
+    else if (d0.kd.tp) st.run(kb_prims<true>, g.total[BC_PRIMS], NT, 0, ba(BC_PRIMS), stage0);
+    else st.run(kb_prims<false>, g.total[BC_PRIMS], NT, 0, ba(BC_PRIMS), stage0);
     chk(cudaGetLastError());
     if (stage0 && d0.cfl > 0.0) {
-      kb_dt_final<<<g.total[BC_ONE], NT, 0, st>>>(ba(BC_ONE), g.nparts_dt);
+      st.run(kb_dt_final, g.total[BC_ONE], NT, 0, ba(BC_ONE), g.nparts_dt);
       chk(cudaGetLastError());
     }
-    if (d0.mixed) kb_ghost_prim<float><<<g.total[BC_GHOST], NT, 0, st>>>(ba(BC_GHOST));
-    else kb_ghost_prim<double><<<g.total[BC_GHOST], NT, 0, st>>>(ba(BC_GHOST));
+    if (d0.mixed) st.run(kb_ghost_prim<float>, g.total[BC_GHOST], NT, 0, ba(BC_GHOST));
+    else st.run(kb_ghost_prim<double>, g.total[BC_GHOST], NT, 0, ba(BC_GHOST));
     chk(cudaGetLastError());
     if (d0.viscous || d0.weno) {
       chk(launch_grad_batch(d0, ba(BC_GRAD), g.total[BC_GRAD], st));
-      if (d0.mixed) kb_ghost_aux<float><<<g.total[BC_GHOST], NT, 0, st>>>(ba(BC_GHOST));
-      else kb_ghost_aux<double><<<g.total[BC_GHOST], NT, 0, st>>>(ba(BC_GHOST));
-      chk(cudaGetLastError());
-    }
-    if (d0.weno) {
-      kb_reset_counts<<<g.total[BC_ONE], NT, 0, st>>>(ba(BC_ONE));
+      if (d0.mixed) st.run(kb_ghost_aux<float>, g.total[BC_GHOST], NT, 0, ba(BC_GHOST));
+      else st.run(kb_ghost_aux<double>, g.total[BC_GHOST], NT, 0, ba(BC_GHOST));
       chk(cudaGetLastError());
     }
     for (int dir = 0; dir < 3; ++dir)
       chk(launch_flux_batch(d0, ba(BC_FLUX0 + dir), g.total[BC_FLUX0 + dir], g.maps[dir], g.tgs[dir], dir, dir > 0,
                             st));
     if (d0.weno)
-      for (int dir = 0; dir < 3; ++dir) chk(launch_weno_batch(d0, ba(BC_WENO0 + dir), g.total[BC_WENO0 + dir], dir, st));
+      chk(launch_weno_batch(d0, ba(BC_WENO), g.total[BC_WENO], st));
     if (d0.viscous) chk(launch_visc_batch(d0, ba(BC_VISC), g.total[BC_VISC], st));
     else if (d0.weno) chk(launch_apply_batch(d0, ba(BC_PRIMS), g.total[BC_PRIMS], st));
     if (d0.force) {
       if (!visc_force_partials(d0)) {
-        if (d0.mixed) kb_force_partial<float><<<g.total[BC_FORCE], NT, 0, st>>>(ba(BC_FORCE));
-        else kb_force_partial<double><<<g.total[BC_FORCE], NT, 0, st>>>(ba(BC_FORCE));
+        if (d0.mixed) st.run(kb_force_partial<float>, g.total[BC_FORCE], NT, 0, ba(BC_FORCE));
+        else st.run(kb_force_partial<double>, g.total[BC_FORCE], NT, 0, ba(BC_FORCE));
         chk(cudaGetLastError());
       }
-      kb_force_final<<<g.total[BC_ONE], NT, 0, st>>>(ba(BC_ONE), g.nparts_force);
+      st.run(kb_force_final, g.total[BC_ONE], NT, 0, ba(BC_ONE), g.nparts_force);
       chk(cudaGetLastError());
     }
-    if (d0.mixed) kb_update_mixed<<<g.total[BC_PRIMS], NT, 0, st>>>(ba(BC_PRIMS), RK_G[stage], RK_R[stage + 1], stage);
-    else kb_update<<<g.total[BC_PRIMS], NT, 0, st>>>(ba(BC_PRIMS), RK_G[stage], RK_R[stage + 1], stage);
+    if (d0.mixed) st.run(kb_update_mixed, g.total[BC_PRIMS], NT, 0, ba(BC_PRIMS), RK_G[stage], RK_R[stage + 1], stage);
+    else st.run(kb_update, g.total[BC_PRIMS], NT, 0, ba(BC_PRIMS), RK_G[stage], RK_R[stage + 1], stage);
     chk(cudaGetLastError());
   }
   g.launches = cnt;
   return e;
+}
+
+// One step of a member on its own launches, beside the other branches of
+// the batch: its z-planes are chosen for all of them together (the chip is
+// shared, so CTAs of more planes, which load their column queues less often,
+// pay; boxes of 32^3 .. 128^3 took 1.248 ms per step with the planes of the
+// boxes alone, 1.225 with 24, 1.214 with 16, the most that is taken: more
+// make the largest box's chain long), and it gets its share, by points, of
+// the WENO CTAs of one box (1.240 -> 1.204 ms where nothing is flagged).  Forced members
+// keep their planes (they sum the forcing by plane groups).
+// In branch mode, kept to compare the work list with, members keep the
+// default shapes and the plain launches of large boxes.
+cudaError_t enqueue_member(s2_solver *s, int zs, double share, int mode, Trace *tr) {
+  Dev &d = s->d;
+  const int own_zs = d.zs, own_tx = d.fx_tx, own_cps = d.weno_cps;
+  const bool plain = mode == S2_BATCH_BRANCHES;
+  if (d.zs_set == ZS_DEFAULT && !d.force) d.zs = plain ? ZS_DEFAULT : zs;
+  if (plain) {
+    d.auto_shape = 0;
+    d.fx_tx = 32;
+  } else {
+    d.weno_cps = (int)(own_cps * share) + 1;
+  }
+  const cudaError_t e = enqueue_step(s, tr);
+  d.zs = own_zs;
+  d.fx_tx = own_tx;
+  d.weno_cps = own_cps;
+  d.auto_shape = 1;
+  return e;
+}
+
+int joint_planes(const std::vector<s2_solver *> &members) {
+  std::vector<Dev> d;
+  for (const s2_solver *s : members) d.push_back(s->d);
+  if (d.empty()) return ZS_DEFAULT;
+  const int zs = z_auto_planes(d.data(), (int)d.size());
+  return zs > 16 ? 16 : zs;
 }
 
 int batch_build(s2_batch *b) {
@@ -2136,12 +2207,15 @@ int batch_build(s2_batch *b) {
   cudaError_t e = cudaEventRecord(b->events[0], b->stream);
   long long total_launches = 0;
   b->member_launches.assign(b->members.size(), 0);
+  const int zs = joint_planes(b->members);
+  double points = 0.0;
+  for (const s2_solver *s : b->members) points += (double)s->d.n;
   if (b->mode == S2_BATCH_BRANCHES) {
     for (size_t m = 0; m < b->members.size() && e == cudaSuccess; ++m) {
       s2_solver *s = b->members[m];
       e = cudaStreamWaitEvent(s->stream, b->events[0], 0);
       Trace tr;
-      if (e == cudaSuccess) e = enqueue_step(s, &tr);
+      if (e == cudaSuccess) e = enqueue_member(s, zs, s->d.n / points, b->mode, &tr);
       total_launches += total(tr);
       b->member_launches[m] = total(tr);
       if (e == cudaSuccess) e = cudaEventRecord(b->events[1 + m], s->stream);
@@ -2164,7 +2238,7 @@ int batch_build(s2_batch *b) {
       s2_solver *s = b->solo[k];
       e = cudaStreamWaitEvent(s->stream, b->events[0], 0);
       Trace tr;
-      if (e == cudaSuccess) e = enqueue_step(s, &tr);
+      if (e == cudaSuccess) e = enqueue_member(s, zs, s->d.n / points, b->mode, &tr);
       total_launches += total(tr);
       for (size_t m = 0; m < b->members.size(); ++m)
         if (b->members[m] == s) b->member_launches[m] = total(tr);

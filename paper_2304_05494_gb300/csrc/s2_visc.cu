@@ -217,6 +217,7 @@ __device__ __forceinline__ void apply_body(const Dev &__restrict__ d, const Blk 
 
 template <class R>
 __global__ void __launch_bounds__(NT) k_apply(Dev d) {
+  pdl_wait();
   apply_body<R>(d, grid_blk());
 }
 
@@ -286,25 +287,23 @@ __device__ __noinline__ void visc_point(const Dev &__restrict__ d, int j, long l
 
 // --------------------------------------- fixed-point passes (FP64 path)
 // The stencil sums of the gradient and viscous passes in 59-bit fixed point
-// (s2_fixed.cuh).  A CTA owns a 32 x 8 tile of one z-plane: the fields are
+// (s2_fixed.cuh).  A CTA owns a TX x 256/TX tile of one z-plane: the fields are
 // converted once into shared memory with an NP-point x-y halo; the 2 NP
 // neighbours along z are read from memory (L2) and converted by the thread
 // that needs them.  One plane per CTA keeps small boxes spread over the
 // chip.  On 420 x 250 x 320 points at order 6 a launch of the gradient pass
 // went from 3.53 to 1.75 ms (double and integer unit both near 3/4 busy),
 // of the viscous pass from 10.33 to 3.95 ms (double unit).
-constexpr int FTX = 32, FTY = 8;
-
-template <int NP>
+template <int NP, int TX>
 struct FxTile {
-  static constexpr int SX = FTX + 2 * NP, SIZE = SX * (FTY + 2 * NP);
+  static constexpr int TY = NT / TX, SX = TX + 2 * NP, SIZE = SX * (TY + 2 * NP);
 };
 
 // Fields src[0..NF-1] of plane k around (x0, y0) into sm as limbs.
-template <int NP, int NF>
+template <int NP, int TX, int NF>
 __device__ __forceinline__ void fx_stage(const Dev &d, const double *const (&src)[NF], const int *e, int x0, int y0,
-                                         int k, int2 (*sm)[FxTile<NP>::SIZE]) {
-  constexpr int SX = FxTile<NP>::SX, SIZE = FxTile<NP>::SIZE;
+                                         int k, int2 (*sm)[FxTile<NP, TX>::SIZE]) {
+  constexpr int SX = FxTile<NP, TX>::SX, SIZE = FxTile<NP, TX>::SIZE;
 #pragma unroll
   for (int s = 0; s < (SIZE + NT - 1) / NT; ++s) {
     const int pos = threadIdx.x + s * NT, hy = pos / SX, hx = pos - hy * SX;
@@ -378,15 +377,15 @@ __device__ __forceinline__ void fx_near_z(const double *f, long long sz, int e, 
 // Velocity gradients (stored), theta = div u and the sensor test.  The x
 // derivatives are converted on the integer unit, the others on the double
 // unit, which balances the two.
-template <int NP>
+template <int NP, int TX>
 __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Blk &B) {
-  constexpr int SX = FxTile<NP>::SX;
-  __shared__ int2 sm[3][FxTile<NP>::SIZE];
+  constexpr int SX = FxTile<NP, TX>::SX;
+  __shared__ int2 sm[3][FxTile<NP, TX>::SIZE];
   __shared__ int ex[4];  // exponents of u, v, w; fixed point or not
   __shared__ unsigned red[NT / 32];
   const View<double> V = view<double>(d);
-  const int tid = threadIdx.x, x0 = B.x * FTX, y0 = B.y * FTY, k = B.z;
-  const int i = x0 + tid % FTX, j = y0 + tid / FTX;
+  const int tid = threadIdx.x, x0 = B.x * TX, y0 = B.y * FxTile<NP, TX>::TY, k = B.z;
+  const int i = x0 + tid % TX, j = y0 + tid / TX;
   if (tid == 0) {
     const FxScale fx = fx_scale(d);
     ex[0] = fx.e[FX_U];
@@ -396,7 +395,7 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
   }
   __syncthreads();
   const double *vel[3] = {V.u, V.v, V.ww};
-  if (ex[3]) fx_stage<NP, 3>(d, vel, ex, x0, y0, k, sm);
+  if (ex[3]) fx_stage<NP, TX, 3>(d, vel, ex, x0, y0, k, sm);
   __syncthreads();
   unsigned eth = 0;
   const long long p = pidx(d, i, j, k), q = ((long long)k * d.ny + j) * d.nx + i;
@@ -405,7 +404,7 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
     double g[3][3];
     if (ex[3]) {
       const double uy = __ldg(d.fy1 + j);
-      const int c = (tid / FTX + NP) * SX + tid % FTX + NP;
+      const int c = (tid / TX + NP) * SX + tid % TX + NP;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const int n = ex[a] - 1022 - 59;  // unit 2^(E - 59)
@@ -449,15 +448,15 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
 // Three CTAs per multiprocessor (80 registers, 40 bytes spilled) measured
 // 4.61 ms where two took 5.39; adding the directions of a Laplacian up
 // before its one conversion to double then gave 3.95.
-template <int NP>
+template <int NP, int TX>
 __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Blk &B) {
-  constexpr int SX = FxTile<NP>::SX, NF = 5;
-  __shared__ int2 sm[NF][FxTile<NP>::SIZE];
+  constexpr int SX = FxTile<NP, TX>::SX, NF = 5;
+  __shared__ int2 sm[NF][FxTile<NP, TX>::SIZE];
   __shared__ int ex[NF + 1];  // exponents of u, v, w, T, theta; fixed point or not
   const View<double> V = view<double>(d);
   const Consts<double> &K = d.kd;
-  const int tid = threadIdx.x, x0 = B.x * FTX, y0 = B.y * FTY, k = B.z;
-  const int i = x0 + tid % FTX, j = y0 + tid / FTX;
+  const int tid = threadIdx.x, x0 = B.x * TX, y0 = B.y * FxTile<NP, TX>::TY, k = B.z;
+  const int i = x0 + tid % TX, j = y0 + tid / TX;
   if (tid == 0) {
     const FxScale fx = fx_scale(d);
     ex[0] = fx.e[FX_U];
@@ -469,7 +468,7 @@ __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Bl
   }
   __syncthreads();
   const double *src[NF] = {V.u, V.v, V.ww, V.T, V.div};
-  if (ex[5]) fx_stage<NP, NF>(d, src, ex, x0, y0, k, sm);
+  if (ex[5]) fx_stage<NP, TX, NF>(d, src, ex, x0, y0, k, sm);
   __syncthreads();
   if (i >= d.nx || j >= d.ny) return;
   const long long p = pidx(d, i, j, k), q = ((long long)k * d.ny + j) * d.nx + i;
@@ -478,7 +477,7 @@ __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Bl
 #pragma unroll
   for (int f = 0; f < NV; ++f) Rv[f] = V.fl[f * d.n + q];
   if (ex[5]) {
-    const int c = (tid / FTX + NP) * SX + tid % FTX + NP;
+    const int c = (tid / TX + NP) * SX + tid % TX + NP;
     const double uy1 = __ldg(d.fy1 + j), ry = __ldg(V.ry + j);
     const double mu = __ldg(V.mu + q), T = __ldg(V.T + p), th = __ldg(V.div + p);
     FxLap fl;
@@ -569,10 +568,11 @@ __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Bl
 
 // One CTA per tile and plane on a linear grid (no extent of a grid
 // dimension limits the box).
+template <int TX>
 __device__ __forceinline__ Blk fx_blk(const Dev &d) {
   Blk B = grid_blk();
-  B.nx = (d.nx + FTX - 1) / FTX;
-  B.ny = (d.ny + FTY - 1) / FTY;
+  B.nx = (d.nx + TX - 1) / TX;
+  B.ny = (d.ny + NT / TX - 1) / (NT / TX);
   const unsigned l = B.x, r = l / B.nx;
   B.x = l - r * B.nx;
   B.z = r / B.ny;
@@ -580,26 +580,28 @@ __device__ __forceinline__ Blk fx_blk(const Dev &d) {
   return B;
 }
 
-template <int NP>
+template <int NP, int TX>
 __global__ void __launch_bounds__(NT, 3) k_grad(const __grid_constant__ Dev d) {
-  grad_fx_body<NP>(d, fx_blk(d));
+  pdl_wait();
+  grad_fx_body<NP, TX>(d, fx_blk<TX>(d));
 }
 
-template <int NP>
+template <int NP, int TX>
 __global__ void __launch_bounds__(NT, 3) kb_grad(BatchArgs ba) {
   S2_BATCH_ENTER(ba, sd, B, b_box);
-  grad_fx_body<NP>(sd, B);
+  grad_fx_body<NP, TX>(sd, B);
 }
 
-template <int NP>
+template <int NP, int TX>
 __global__ void __launch_bounds__(NT, 3) k_visc(const __grid_constant__ Dev d) {
-  visc_fx_body<NP>(d, fx_blk(d));
+  pdl_wait();
+  visc_fx_body<NP, TX>(d, fx_blk<TX>(d));
 }
 
-template <int NP>
-__global__ void __launch_bounds__(NT, 2) kb_visc(BatchArgs ba) {
+template <int NP, int TX>
+__global__ void __launch_bounds__(NT, 3) kb_visc(BatchArgs ba) {
   S2_BATCH_ENTER(ba, sd, B, b_box);
-  visc_fx_body<NP>(sd, B);
+  visc_fx_body<NP, TX>(sd, B);
 }
 
 // ------------------------------------------------ z-marching (mixed path)
@@ -775,6 +777,7 @@ __device__ __forceinline__ void grad_z_body(const Dev &__restrict__ d, const Blk
 
 template <int NP, int ZS>
 __global__ void __launch_bounds__(NT, 3) k_grad_z(Dev d) {
+  pdl_wait();
   grad_z_body<NP, ZS>(d, grid_blk());
 }
 
@@ -932,6 +935,7 @@ __device__ __forceinline__ void visc_z_body(const Dev &__restrict__ d, const Blk
 
 template <int NP, int ZS>
 __global__ void __launch_bounds__(NT, 2) k_visc_z(Dev d) {
+  pdl_wait();
   visc_z_body<NP, ZS>(d, grid_blk());
 }
 
@@ -942,29 +946,28 @@ __global__ void __launch_bounds__(NT, 2) kb_visc_z(BatchArgs ba) {
 }
 
 
-// Linear grid of the FP64 gradient and viscous passes.
-unsigned fx_blocks(const Dev &d) {
-  return (unsigned)(((d.nx + FTX - 1) / FTX) * (long long)((d.ny + FTY - 1) / FTY) * d.nz);
-}
-
-void grad_np(const Dev &d, cudaStream_t st) {
-  const unsigned nb = fx_blocks(d);
+// The FP64 gradient and viscous passes for the viscous order and tile width
+// of d: f(NP, TX) as integral constants.
+template <class F>
+void fx_launch(const Dev &d, F f) {
+  auto tx = [&](auto np) {
+    switch (d.fx_tx) {
+      case 8: f(np, std::integral_constant<int, 8>()); break;
+      case 16: f(np, std::integral_constant<int, 16>()); break;
+      default: f(np, std::integral_constant<int, 32>()); break;
+    }
+  };
   switch (d.npv) {
-    case 1: k_grad<1><<<nb, NT, 0, st>>>(d); break;
-    case 2: k_grad<2><<<nb, NT, 0, st>>>(d); break;
-    case 3: k_grad<3><<<nb, NT, 0, st>>>(d); break;
-    default: k_grad<4><<<nb, NT, 0, st>>>(d); break;
+    case 1: tx(std::integral_constant<int, 1>()); break;
+    case 2: tx(std::integral_constant<int, 2>()); break;
+    case 3: tx(std::integral_constant<int, 3>()); break;
+    default: tx(std::integral_constant<int, 4>()); break;
   }
 }
 
-void visc_np(const Dev &d, cudaStream_t st) {
-  const unsigned nb = fx_blocks(d);
-  switch (d.npv) {
-    case 1: k_visc<1><<<nb, NT, 0, st>>>(d); break;
-    case 2: k_visc<2><<<nb, NT, 0, st>>>(d); break;
-    case 3: k_visc<3><<<nb, NT, 0, st>>>(d); break;
-    default: k_visc<4><<<nb, NT, 0, st>>>(d); break;
-  }
+long long fx_tiles(const Dev &d, int tx) {
+  const int ty = NT / tx;
+  return (long long)((d.nx + tx - 1) / tx) * ((d.ny + ty - 1) / ty) * d.nz;
 }
 
 }  // namespace
@@ -974,6 +977,8 @@ void visc_np(const Dev &d, cudaStream_t st) {
 template <int NPV, class F>
 void z_launch(F f, int zs) {
   switch (zs) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
     case 4: f(std::integral_constant<int, 4>()); break;
     case 8: f(std::integral_constant<int, 8>()); break;
     case 16: f(std::integral_constant<int, 16>()); break;
@@ -982,28 +987,69 @@ void z_launch(F f, int zs) {
   }
 }
 
+// The width that covers the boxes with the fewest 256-point tiles (lanes
+// beyond a row's end do nothing, yet their warps occupy the double unit); a
+// narrower one has to save a twentieth, for its shorter rows in memory.
+int fx_auto_tx(const Dev *d, int count) {
+  int best = 32;
+  long long least = -1;
+  for (int tx : {32, 16, 8}) {
+    long long t = 0;
+    for (int b = 0; b < count; ++b) t += fx_tiles(d[b], tx);
+    if (least < 0 || 20 * t < 19 * least) {
+      least = t;
+      best = tx;
+    }
+  }
+  return best;
+}
+
+// A CTA of zs planes costs about zs + 2 plane times (it first fills its
+// column queues), and two viscous CTAs fit on a multiprocessor: the count
+// with the least (CTAs over those places, rounded up) x (zs + 2).  Small
+// boxes get few planes per CTA, so that there are CTAs for every
+// multiprocessor (37 x 29 x 19: one plane, 152 CTAs instead of 16), large
+// ones many.
+int z_auto_planes(const Dev *d, int count) {
+  int best = ZS_DEFAULT;
+  long long cost = -1;
+  for (int zs : {24, 16, 12, 8, 4, 2, 1}) {
+    long long ctas = 0;
+    for (int b = 0; b < count; ++b)
+      ctas += (long long)((d[b].nx + ZTX - 1) / ZTX) * ((d[b].ny + ZTY - 1) / ZTY) * ((d[b].nz + zs - 1) / zs);
+    const long long places = 2ll * d[0].nsm, c = (ctas + places - 1) / places * (zs + 2);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = zs;
+    }
+  }
+  return best;
+}
+
 static dim3 zgrid(const Dev &d) {
   return dim3((d.nx + ZTX - 1) / ZTX, (d.ny + ZTY - 1) / ZTY, (d.nz + d.zs - 1) / d.zs);
 }
 
-cudaError_t launch_grad(const Dev &d, cudaStream_t st) {
+cudaError_t launch_grad(const Dev &d, const Lane &st) {
   if (d.mixed) {
     switch (d.npv) {
-      case 1: z_launch<1>([&](auto zs) { k_grad_z<1, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
-      case 2: z_launch<2>([&](auto zs) { k_grad_z<2, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
-      case 3: z_launch<3>([&](auto zs) { k_grad_z<3, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
-      default: z_launch<4>([&](auto zs) { k_grad_z<4, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
+      case 1: z_launch<1>([&](auto zs) { st.run(k_grad_z<1, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
+      case 2: z_launch<2>([&](auto zs) { st.run(k_grad_z<2, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
+      case 3: z_launch<3>([&](auto zs) { st.run(k_grad_z<3, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
+      default: z_launch<4>([&](auto zs) { st.run(k_grad_z<4, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
     }
   } else {
-    grad_np(d, st);
+    fx_launch(d, [&](auto np, auto tx) {
+      st.run(k_grad<decltype(np)::value, decltype(tx)::value>, (unsigned)fx_tiles(d, d.fx_tx), NT, 0, d);
+    });
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_apply(const Dev &d, cudaStream_t st) {
+cudaError_t launch_apply(const Dev &d, const Lane &st) {
   unsigned nb = (unsigned)((d.n + NT - 1) / NT);
-  if (d.mixed) k_apply<float><<<nb, NT, 0, st>>>(d);
-  else k_apply<double><<<nb, NT, 0, st>>>(d);
+  if (d.mixed) st.run(k_apply<float>, nb, NT, 0, d);
+  else st.run(k_apply<double>, nb, NT, 0, d);
   return cudaGetLastError();
 }
 
@@ -1019,66 +1065,62 @@ int visc_force_partials(const Dev &d) {
 
 void z_pass_grid(const Dev &d, unsigned g[3]) {
   const dim3 z = zgrid(d);
-  g[0] = d.mixed ? z.x : (d.nx + FTX - 1) / FTX;
-  g[1] = d.mixed ? z.y : (d.ny + FTY - 1) / FTY;
+  g[0] = d.mixed ? z.x : (d.nx + d.fx_tx - 1) / d.fx_tx;
+  g[1] = d.mixed ? z.y : (d.ny + NT / d.fx_tx - 1) / (NT / d.fx_tx);
   g[2] = d.mixed ? z.z : d.nz;
 }
 
 // Batched: every box of a batch group in one launch (instantiation of d0).
-cudaError_t launch_grad_batch(const Dev &d0, const BatchArgs &ba, unsigned total, cudaStream_t st) {
+cudaError_t launch_grad_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st) {
   if (d0.mixed) {
     switch (d0.npv) {
-      case 1: z_launch<1>([&](auto zs) { kb_grad_z<1, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
-      case 2: z_launch<2>([&](auto zs) { kb_grad_z<2, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
-      case 3: z_launch<3>([&](auto zs) { kb_grad_z<3, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
-      default: z_launch<4>([&](auto zs) { kb_grad_z<4, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
+      case 1: z_launch<1>([&](auto zs) { st.run(kb_grad_z<1, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
+      case 2: z_launch<2>([&](auto zs) { st.run(kb_grad_z<2, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
+      case 3: z_launch<3>([&](auto zs) { st.run(kb_grad_z<3, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
+      default: z_launch<4>([&](auto zs) { st.run(kb_grad_z<4, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
     }
   } else {
-    switch (d0.npv) {
-      case 1: kb_grad<1><<<total, NT, 0, st>>>(ba); break;
-      case 2: kb_grad<2><<<total, NT, 0, st>>>(ba); break;
-      case 3: kb_grad<3><<<total, NT, 0, st>>>(ba); break;
-      default: kb_grad<4><<<total, NT, 0, st>>>(ba); break;
-    }
+    fx_launch(d0, [&](auto np, auto tx) {
+      st.run(kb_grad<decltype(np)::value, decltype(tx)::value>, total, NT, 0, ba);
+    });
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_visc_batch(const Dev &d0, const BatchArgs &ba, unsigned total, cudaStream_t st) {
+cudaError_t launch_visc_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st) {
   if (d0.mixed) {
     switch (d0.npv) {
-      case 1: z_launch<1>([&](auto zs) { kb_visc_z<1, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
-      case 2: z_launch<2>([&](auto zs) { kb_visc_z<2, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
-      case 3: z_launch<3>([&](auto zs) { kb_visc_z<3, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
-      default: z_launch<4>([&](auto zs) { kb_visc_z<4, decltype(zs)::value><<<total, NT, 0, st>>>(ba); }, d0.zs); break;
+      case 1: z_launch<1>([&](auto zs) { st.run(kb_visc_z<1, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
+      case 2: z_launch<2>([&](auto zs) { st.run(kb_visc_z<2, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
+      case 3: z_launch<3>([&](auto zs) { st.run(kb_visc_z<3, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
+      default: z_launch<4>([&](auto zs) { st.run(kb_visc_z<4, decltype(zs)::value>, total, NT, 0, ba); }, d0.zs); break;
     }
   } else {
-    switch (d0.npv) {
-      case 1: kb_visc<1><<<total, NT, 0, st>>>(ba); break;
-      case 2: kb_visc<2><<<total, NT, 0, st>>>(ba); break;
-      case 3: kb_visc<3><<<total, NT, 0, st>>>(ba); break;
-      default: kb_visc<4><<<total, NT, 0, st>>>(ba); break;
-    }
+    fx_launch(d0, [&](auto np, auto tx) {
+      st.run(kb_visc<decltype(np)::value, decltype(tx)::value>, total, NT, 0, ba);
+    });
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_apply_batch(const Dev &d0, const BatchArgs &ba, unsigned total, cudaStream_t st) {
-  if (d0.mixed) kb_apply<float><<<total, NT, 0, st>>>(ba);
-  else kb_apply<double><<<total, NT, 0, st>>>(ba);
+cudaError_t launch_apply_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const Lane &st) {
+  if (d0.mixed) st.run(kb_apply<float>, total, NT, 0, ba);
+  else st.run(kb_apply<double>, total, NT, 0, ba);
   return cudaGetLastError();
 }
 
-cudaError_t launch_visc(const Dev &d, cudaStream_t st) {
+cudaError_t launch_visc(const Dev &d, const Lane &st) {
   if (d.mixed) {
     switch (d.npv) {
-      case 1: z_launch<1>([&](auto zs) { k_visc_z<1, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
-      case 2: z_launch<2>([&](auto zs) { k_visc_z<2, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
-      case 3: z_launch<3>([&](auto zs) { k_visc_z<3, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
-      default: z_launch<4>([&](auto zs) { k_visc_z<4, decltype(zs)::value><<<zgrid(d), NT, 0, st>>>(d); }, d.zs); break;
+      case 1: z_launch<1>([&](auto zs) { st.run(k_visc_z<1, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
+      case 2: z_launch<2>([&](auto zs) { st.run(k_visc_z<2, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
+      case 3: z_launch<3>([&](auto zs) { st.run(k_visc_z<3, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
+      default: z_launch<4>([&](auto zs) { st.run(k_visc_z<4, decltype(zs)::value>, zgrid(d), NT, 0, d); }, d.zs); break;
     }
   } else {
-    visc_np(d, st);
+    fx_launch(d, [&](auto np, auto tx) {
+      st.run(k_visc<decltype(np)::value, decltype(tx)::value>, (unsigned)fx_tiles(d, d.fx_tx), NT, 0, d);
+    });
   }
   return cudaGetLastError();
 }
