@@ -640,43 +640,85 @@ __global__ void __launch_bounds__(NTHREADS, 4) kb_flux(BatchArgs ba, const FluxM
 // ------------------------------------------------------------------ WENO
 // Reconstruction at i+1/2 from 2r-1 values g[0..2r-2] centred on g[r-1]:
 // Jiang & Shu (r=3), Balsara & Shu (r=4), alpha_k = d_k/(eps+beta_k)^2.
-// Everything but the centre value is formed from the undivided differences
-// d_i = g[i+1] - g[i] and, for the indicators, theirs: the substencil
-// polynomials are q_k = g[r-1] + (a combination of differences)/6 or /12.
 // The normalisation sum alpha_k q_k / sum alpha_k is evaluated with one
 // reciprocal by multiplying through by prod_k (eps+beta_k)^2, and the
-// polynomials' common denominator joins that reciprocal.  Factors common to
-// eps and all beta_k, and to all alpha_k, cancel: in double precision they
-// are chosen to save multiplications (in single precision they would shift
-// the range in which the products neither overflow nor vanish).  The caller passes eps: reconstructing 2 g with eps' = 4
-// eps gives exactly twice the reconstruction of g with eps (beta is
-// quadratic in g), which lets the flux splitting skip its factor 1/2.
+// substencil polynomials' common denominator (6, 12) joins that
+// reciprocal.  The caller passes eps: reconstructing 2 g with eps' = 4 eps
+// gives exactly twice the reconstruction of g with eps (beta is quadratic
+// in g), which lets the flux splitting skip its factor 1/2.
+// In double precision, bound by that unit, everything but the centre value
+// is formed from the undivided differences (q_k = g[r-1] + a combination of
+// them), and factors common to eps and all beta_k, and to all alpha_k, are
+// chosen to save multiplications; single precision keeps the direct form,
+// whose rounding decides with the sensor which interfaces a run flags.
 template <class R>
 __device__ __forceinline__ R recip_pos(R x) {
   return rcp_pos(x);
 }
 
-template <class R>
-__device__ __forceinline__ R weno5(const R *g, R eps) {
-  const R d0 = g[1] - g[0], d1 = g[2] - g[1], d2 = g[3] - g[2], d3 = g[4] - g[3];
-  // 6 (q_k - g[2])
-  const R q0 = R(5) * d1 - R(2) * d0, q1 = d1 + R(2) * d2, q2 = R(4) * d2 - d3;
-  const R t0 = d1 - d0, t1 = d2 - d1, t2 = d3 - d2;
-  const R u0 = R(3) * d1 - d0, u1 = d1 + d2, u2 = d3 - R(3) * d2;
-  constexpr bool DBL = sizeof(R) == 8;
-  const R e = DBL ? R(4) * eps : eps, c = DBL ? R(13.0 / 3.0) : R(13.0 / 12.0), f = DBL ? R(1) : R(0.25);
-  R s0 = fma(c * t0, t0, fma(f * u0, u0, e));
-  R s1 = fma(c * t1, t1, fma(f * u1, u1, e));
-  R s2 = fma(c * t2, t2, fma(f * u2, u2, e));
+__device__ __forceinline__ float weno5(const float *g, float eps) {
+  float q0 = float(2) * g[0] - float(7) * g[1] + float(11) * g[2];
+  float q1 = -g[1] + float(5) * g[2] + float(2) * g[3];
+  float q2 = float(2) * g[2] + float(5) * g[3] - g[4];
+  float t, b0, b1, b2;
+  t = g[0] - float(2) * g[1] + g[2]; b0 = float(13.0 / 12.0) * t * t;
+  t = g[0] - float(4) * g[1] + float(3) * g[2]; b0 += float(0.25) * t * t;
+  t = g[1] - float(2) * g[2] + g[3]; b1 = float(13.0 / 12.0) * t * t;
+  t = g[1] - g[3]; b1 += float(0.25) * t * t;
+  t = g[2] - float(2) * g[3] + g[4]; b2 = float(13.0 / 12.0) * t * t;
+  t = float(3) * g[2] - float(4) * g[3] + g[4]; b2 += float(0.25) * t * t;
+  float s0 = eps + b0, s1 = eps + b1, s2 = eps + b2;
   s0 *= s0; s1 *= s1; s2 *= s2;
-  const R w = DBL ? R(1) : R(0.1);
-  const R a0 = w * (s1 * s2), a1 = (R(6) * w) * (s0 * s2), a2 = (R(3) * w) * (s0 * s1);
-  return fma(a0 * q0 + a1 * q1 + a2 * q2, recip_pos(R(6) * (a0 + a1 + a2)), g[2]);
+  float a0 = float(0.1) * s1 * s2, a1 = float(0.6) * s0 * s2, a2 = float(0.3) * s0 * s1;
+  return (a0 * q0 + a1 * q1 + a2 * q2) * recip_pos(float(6) * (a0 + a1 + a2));
 }
 
-template <class R>
-__device__ __forceinline__ R weno7(const R *g, R eps) {
-  R d[6], e2[5], e3[4];
+__device__ __forceinline__ double weno5(const double *g, double eps) {
+  const double d0 = g[1] - g[0], d1 = g[2] - g[1], d2 = g[3] - g[2], d3 = g[4] - g[3];
+  // 6 (q_k - g[2])
+  const double q0 = 5.0 * d1 - 2.0 * d0, q1 = d1 + 2.0 * d2, q2 = 4.0 * d2 - d3;
+  // 4 (eps + beta_k)
+  const double t0 = d1 - d0, t1 = d2 - d1, t2 = d3 - d2;
+  const double u0 = 3.0 * d1 - d0, u1 = d1 + d2, u2 = d3 - 3.0 * d2;
+  const double e = 4.0 * eps, c = 13.0 / 3.0;
+  double s0 = fma(c * t0, t0, fma(u0, u0, e));
+  double s1 = fma(c * t1, t1, fma(u1, u1, e));
+  double s2 = fma(c * t2, t2, fma(u2, u2, e));
+  s0 *= s0; s1 *= s1; s2 *= s2;
+  const double a0 = s1 * s2, a1 = 6.0 * (s0 * s2), a2 = 3.0 * (s0 * s1);
+  return fma(a0 * q0 + a1 * q1 + a2 * q2, rcp_pos(6.0 * (a0 + a1 + a2)), g[2]);
+}
+
+__device__ __forceinline__ float weno7(const float *g, float eps) {
+  float q0 = float(-3) * g[0] + float(13) * g[1] - float(23) * g[2] + float(25) * g[3];
+  float q1 = g[1] - float(5) * g[2] + float(13) * g[3] + float(3) * g[4];
+  float q2 = -g[2] + float(7) * g[3] + float(7) * g[4] - g[5];
+  float q3 = float(3) * g[3] + float(13) * g[4] - float(5) * g[5] + g[6];
+  // smoothness indicators: 240 x the Jiang-Shu measure as sums of squares
+  // of the undivided differences of each 4-point substencil
+  float bk[4];
+  const float c10[4] = {float(5.0 / 2.0), float(3.0 / 2.0), float(1.0 / 2.0), float(-1.0 / 2.0)};
+  const float c11[4] = {float(11.0 / 6.0), float(1.0 / 3.0), float(-1.0 / 6.0), float(1.0 / 3.0)};
+  const float c2[4] = {float(2), float(1), float(0), float(-1)};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float e1 = g[k + 1] - g[k];
+    float e2 = g[k + 2] - float(2) * g[k + 1] + g[k];
+    float e3 = g[k + 3] - float(3) * g[k + 2] + float(3) * g[k + 1] - g[k];
+    float t1 = e1 + c10[k] * e2 + c11[k] * e3;
+    float t2 = e2 + c2[k] * e3;
+    bk[k] = float(240) * t1 * t1 + float(260) * t2 * t2 + float(781.0 / 3.0) * e3 * e3;
+  }
+  float s0 = eps + bk[0], s1 = eps + bk[1], s2 = eps + bk[2], s3 = eps + bk[3];
+  s0 *= s0; s1 *= s1; s2 *= s2; s3 *= s3;
+  float p01 = s0 * s1, p23 = s2 * s3;
+  float a0 = float(1.0 / 35.0) * s1 * p23, a1 = float(12.0 / 35.0) * s0 * p23;
+  float a2 = float(18.0 / 35.0) * p01 * s3, a3 = float(4.0 / 35.0) * p01 * s2;
+  return (a0 * q0 + a1 * q1 + a2 * q2 + a3 * q3) * recip_pos(float(12) * (a0 + a1 + a2 + a3));
+}
+
+__device__ __forceinline__ double weno7(const double *g, double eps) {
+  double d[6], e2[5], e3[4];
 #pragma unroll
   for (int i = 0; i < 6; ++i) d[i] = g[i + 1] - g[i];
 #pragma unroll
@@ -684,28 +726,25 @@ __device__ __forceinline__ R weno7(const R *g, R eps) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) e3[i] = e2[i + 1] - e2[i];
   // 12 (q_k - g[3])
-  const R q0 = R(3) * d[0] - R(10) * d[1] + R(13) * d[2], q1 = R(4) * d[2] - d[1] + R(3) * d[3];
-  const R q2 = d[2] + R(6) * d[3] - d[4], q3 = R(9) * d[3] - R(4) * d[4] + d[5];
-  // smoothness indicators: 240 x the Jiang-Shu measure (in double precision
-  // the measure itself) as sums of squares of the undivided differences of
-  // each 4-point substencil
-  const R c10[4] = {R(5.0 / 2.0), R(3.0 / 2.0), R(1.0 / 2.0), R(-1.0 / 2.0)};
-  const R c11[4] = {R(11.0 / 6.0), R(1.0 / 3.0), R(-1.0 / 6.0), R(1.0 / 3.0)};
-  const R c2[4] = {R(2), R(1), R(0), R(-1)};
-  constexpr bool DBL = sizeof(R) == 8;
-  const R m = DBL ? R(1) : R(240), e = DBL ? eps * R(1.0 / 240.0) : eps;
-  R s[4];
+  const double q0 = 3.0 * d[0] - 10.0 * d[1] + 13.0 * d[2], q1 = 4.0 * d[2] - d[1] + 3.0 * d[3];
+  const double q2 = d[2] + 6.0 * d[3] - d[4], q3 = 9.0 * d[3] - 4.0 * d[4] + d[5];
+  // eps + beta_k: the Jiang-Shu measure as sums of squares of the undivided
+  // differences of each 4-point substencil
+  const double c10[4] = {5.0 / 2.0, 3.0 / 2.0, 1.0 / 2.0, -1.0 / 2.0};
+  const double c11[4] = {11.0 / 6.0, 1.0 / 3.0, -1.0 / 6.0, 1.0 / 3.0};
+  const double c2[4] = {2.0, 1.0, 0.0, -1.0};
+  const double e = eps / 240.0;
+  double s[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const R t1 = fma(c11[k], e3[k], fma(c10[k], e2[k], d[k]));
-    const R t2 = k == 2 ? e2[k] : fma(c2[k], e3[k], e2[k]);
-    const R b = fma(m * t1, t1, fma(m * R(13.0 / 12.0) * t2, t2, fma(m * R(781.0 / 720.0) * e3[k], e3[k], e)));
+    const double t1 = fma(c11[k], e3[k], fma(c10[k], e2[k], d[k]));
+    const double t2 = k == 2 ? e2[k] : fma(c2[k], e3[k], e2[k]);
+    const double b = fma(t1, t1, fma((13.0 / 12.0) * t2, t2, fma((781.0 / 720.0) * e3[k], e3[k], e)));
     s[k] = b * b;
   }
-  const R p01 = s[0] * s[1], p23 = s[2] * s[3];
-  const R w = DBL ? R(1) : R(1.0 / 35.0);
-  const R a0 = w * s[1] * p23, a1 = R(12) * w * s[0] * p23, a2 = R(18) * w * p01 * s[3], a3 = R(4) * w * p01 * s[2];
-  return fma(a0 * q0 + a1 * q1 + a2 * q2 + a3 * q3, recip_pos(R(12) * (a0 + a1 + a2 + a3)), g[3]);
+  const double p01 = s[0] * s[1], p23 = s[2] * s[3];
+  const double a0 = s[1] * p23, a1 = 12.0 * (s[0] * p23), a2 = 18.0 * (p01 * s[3]), a3 = 4.0 * (p01 * s[2]);
+  return fma(a0 * q0 + a1 * q1 + a2 * q2 + a3 * q3, rcp_pos(12.0 * (a0 + a1 + a2 + a3)), g[3]);
 }
 
 // Order 3: two substencils, d = (1/3, 2/3), beta_k = (undivided difference)^2.
@@ -724,8 +763,8 @@ template <int WR, class R>
 __device__ __forceinline__ R weno_rec(const R *g, R eps) {
   if constexpr (WR == 1) return g[0];  // order 1: upwind value
   else if constexpr (WR == 2) return weno3<R>(g, eps);
-  else if constexpr (WR == 3) return weno5<R>(g, eps);
-  else return weno7<R>(g, eps);
+  else if constexpr (WR == 3) return weno5(g, eps);
+  else return weno7(g, eps);
 }
 
 // F_weno - F_central at every listed interface of direction dir.  The
@@ -787,6 +826,10 @@ __device__ __forceinline__ void weno_body(const Dev &__restrict__ d, const Blk &
       k = s;
     }
     const long long p0 = pidx(d, i, j, k);  // point s of the interface s+1/2
+    // the points on both sides get a correction
+    if (s >= 0) d.wmap[wmap_of(d, i, j, k)] = 1;
+    if (s + 1 < (dir == 0 ? d.nx : (dir == 1 ? d.ny : d.nz)))
+      d.wmap[wmap_of(d, dir == 0 ? s + 1 : i, dir == 1 ? s + 1 : j, dir == 2 ? s + 1 : k)] = 1;
     // the WENO stencil and the central pairs reach p0 - 3 stride .. p0 + 4 stride
     if (!(S2_OK_IDX(d, slot, ns) && S2_OK_IDX(d, p0 - 3 * stride, d.np) &&
           S2_OK_IDX(d, p0 + 4 * stride, d.np)))

@@ -170,6 +170,11 @@ struct Dev {
   unsigned int *wlist[3];
   void *dF[3];             // R
   long long nslot[3];
+  // which blocks of 32 x 8 points of a plane have a flagged interface at one
+  // of their points (wbx x wby blocks per plane): set by the WENO kernels,
+  // cleared by the primitive pass
+  unsigned char *wmap;
+  int wbx, wby;
 };
 
 // Block coordinates of a kernel body.  A launch for one box uses the CUDA
@@ -310,6 +315,11 @@ __host__ __device__ inline View<R> view(const Dev &d) {
 // the value (exact comparisons on the integer pipe).
 __device__ __forceinline__ long long order_bits(double x) { return __double_as_longlong(x); }
 __device__ __forceinline__ int order_bits(float x) { return __float_as_int(x); }
+
+// Entry of Dev::wmap of point (i, j, k).
+__host__ __device__ inline unsigned wmap_of(const Dev &d, int i, int j, int k) {
+  return ((unsigned)k * d.wby + (unsigned)(j >> 3)) * d.wbx + (unsigned)(i >> 5);
+}
 
 __host__ __device__ inline long long pidx(const Dev &d, int i, int j, int k) {
   return d.off0 + (long long)k * d.sz + (long long)j * d.sy + i;

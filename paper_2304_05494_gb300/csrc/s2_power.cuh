@@ -31,17 +31,31 @@ struct PowTab {
 constexpr long long POW_LN2_Q63 = 0x58b90bfbe8e7bcd6ll;  // ln 2
 constexpr long long POW_LN2_Q58 = POW_LN2_Q63 >> 5;
 
+// The part of the table that does not depend on omega, and the logarithms
+// (base 2) for the rest: evaluated once per process (128 extended-precision
+// logarithms and exponentials take 0.5 ms where they are done in software).
+struct PowBase {
+  PowTab t;
+  long double lg[128];
+  PowBase() {
+    const long double ln2 = logl(2.0L);
+    for (int i = 0; i < 128; ++i) {
+      t.r[i] = (int)floorl(1024.0L / (1.0L + (i + 0.5L) / 128.0L) + 0.5L);
+      const long double lr = logl(t.r[i] / 1024.0L);
+      lg[i] = lr / ln2;
+      t.ll[i] = llroundl(ldexpl(-lr, 58));
+      t.b[i] = llroundl(ldexpl(expl(ln2 * i / 128.0L), 62));
+    }
+  }
+};
+
 // The table, and omega and the range of its use in d (visc_exp set).
 inline void pow_setup(Dev &d, PowTab &t) {
+  static const PowBase base;
   const long double ln2 = logl(2.0L), w = d.visc_exp;
   const bool inside = fabs(d.visc_exp) <= 4.0;
-  for (int i = 0; i < 128; ++i) {
-    t.r[i] = (int)floorl(1024.0L / (1.0L + (i + 0.5L) / 128.0L) + 0.5L);
-    const long double lr = logl(t.r[i] / 1024.0L);
-    t.wl[i] = inside ? llroundl(ldexpl(-w * lr / ln2, 58)) : 0;
-    t.ll[i] = llroundl(ldexpl(-lr, 58));
-    t.b[i] = llroundl(ldexpl(expl(ln2 * i / 128.0L), 62));
-  }
+  t = base.t;
+  for (int i = 0; i < 128; ++i) t.wl[i] = inside ? llroundl(ldexpl(-w * base.lg[i], 58)) : 0;
   d.pow_emax = -1;  // no exponent is in range
   if (inside) {
     d.pow_w = llroundl(ldexpl(w, 58));

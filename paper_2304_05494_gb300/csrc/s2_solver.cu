@@ -168,10 +168,12 @@ __device__ __forceinline__ void dt_block_max(const Dev &d, double sr, int want_d
 }
 
 // The per-RHS counters of the hybrid scheme (flagged interfaces and the
-// three list lengths) start at zero with the primitive pass, which runs
-// after every reader of the evaluation before.
+// three list lengths) and the map of blocks with flags start at zero with the
+// primitive pass, which runs after every reader of the evaluation before.
 __device__ __forceinline__ void reset_counts(const Dev &d, long long q) {
-  if (q == 0 && d.weno) {
+  if (!d.weno) return;
+  if (q < (long long)d.wbx * d.wby * d.nz) d.wmap[q] = 0;
+  if (q == 0) {
     d.scal->wcount = 0;
     for (int a = 0; a < 4; ++a) d.scal->nlist[a] = 0;
   }
@@ -1427,17 +1429,24 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   // s2_rhs stages its double output in fln when that is double, else here
   s->rhs_stage = d.mixed ? A(NV * nn) : (double *)d.fln;
   double *eta = A(grid->ny), *ay = A(4 * grid->ny), *by = A(5 * grid->ny), *ry = A(grid->ny), *dvy = A(grid->ny);
-  // table of the power law and the logarithm (FP64: mu of viscous runs, the
-  // thermally perfect e(T))
+  // one block: units of the fixed-point stencils; table of the power law and
+  // the logarithm (FP64: mu of viscous runs, the thermally perfect e(T)); the
+  // map of blocks with flags
+  d.wbx = (grid->nx + 31) / 32;
+  d.wby = (grid->ny + 7) / 8;
+  const size_t map_bytes = scheme->weno_order ? (size_t)d.wbx * d.wby * grid->nz : 1;
+  const size_t o_fy = sizeof(FxLap) * grid->ny, o_pow = o_fy + sizeof(double) * grid->ny;
+  const size_t o_map = o_pow + sizeof(PowTab);
+  unsigned char *tables = (unsigned char *)dalloc(s, o_map + map_bytes);
+  if (!tables) ok = false;
+  FxLap *fxl = (FxLap *)tables;
+  double *fy = (double *)(tables + o_fy);
+  d.wmap = tables + o_map;
   std::vector<PowTab> powt(1);
   if (!d.mixed && (d.viscous || d.kd.tp)) {
-    d.powt = (PowTab *)dalloc(s, sizeof(PowTab));
-    if (!d.powt) ok = false;
+    d.powt = (PowTab *)(tables + o_pow);
     pow_setup(d, powt[0]);
   }
-  double *fy = A(grid->ny);
-  FxLap *fxl = (FxLap *)dalloc(s, sizeof(FxLap) * grid->ny);
-  if (!fxl) ok = false;
   float *etaf = (float *)dalloc(s, sizeof(float) * grid->ny), *ayf = (float *)dalloc(s, sizeof(float) * 4 * grid->ny);
   float *byf = (float *)dalloc(s, sizeof(float) * 5 * grid->ny), *ryf = (float *)dalloc(s, sizeof(float) * grid->ny);
   if (!etaf || !ayf || !byf || !ryf) ok = false;
