@@ -297,8 +297,10 @@ __device__ __noinline__ void visc_point(const Dev &__restrict__ d, int j, long l
 // neighbours along z are read from memory (L2) and converted by the thread
 // that needs them.  One plane per CTA keeps small boxes spread over the
 // chip.  On 420 x 250 x 320 points at order 6 a launch of the gradient pass
-// went from 3.53 to 1.75 ms (double and integer unit both near 3/4 busy),
-// of the viscous pass from 10.33 to 3.95 ms (double unit).
+// went from 3.53 to 1.51 ms (double and integer unit both near 3/4 busy),
+// of the viscous pass from 10.33 to 3.85 ms (double unit).  Four CTAs per
+// multiprocessor (64 registers) hide the latencies better than three, though
+// the viscous pass spills: 1.69 -> 1.51 and 3.97 -> 3.85 ms.
 template <int NP, int TX>
 struct FxTile {
   static constexpr int TY = NT / TX, SX = TX + 2 * NP, SIZE = SX * (TY + 2 * NP);
@@ -450,9 +452,8 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
 //   u_a X_a + tau_ab d_b u_a / mu + (c_p / Pr) (lap T + psi . grad T)
 // so mu enters with the sum into the RHS: about 55 double operations per
 // point at order 6 (169 when the stencils were in double precision too).
-// Three CTAs per multiprocessor (80 registers, 40 bytes spilled) measured
-// 4.61 ms where two took 5.39; adding the directions of a Laplacian up
-// before its one conversion to double then gave 3.95.
+// Adding the directions of a Laplacian up before its one conversion to
+// double took it from 4.61 to 3.95 ms.
 template <int NP, int TX>
 __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Blk &B) {
   constexpr int SX = FxTile<NP, TX>::SX, NF = 5;
@@ -589,7 +590,7 @@ __device__ __forceinline__ Blk fx_blk(const Dev &d) {
 }
 
 template <int NP, int TX>
-__global__ void __launch_bounds__(NT, 3) k_grad(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(NT, 4) k_grad(const __grid_constant__ Dev d) {
   pdl_wait();
   grad_fx_body<NP, TX>(d, fx_blk<TX>(d));
 }
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(NT, 3) kb_grad(BatchArgs ba) {
 }
 
 template <int NP, int TX>
-__global__ void __launch_bounds__(NT, 3) k_visc(const __grid_constant__ Dev d) {
+__global__ void __launch_bounds__(NT, 4) k_visc(const __grid_constant__ Dev d) {
   pdl_wait();
   visc_fx_body<NP, TX>(d, fx_blk<TX>(d));
 }
@@ -1003,12 +1004,13 @@ void z_launch(F f, int zs) {
 }
 
 // The width that covers the boxes with the fewest 256-point tiles (lanes
-// beyond a row's end do nothing, yet their warps occupy the double unit); a
-// narrower one has to save a twentieth, for its shorter rows in memory.
+// beyond a row's end do nothing, yet their warps occupy the double unit).  16
+// unless another saves a twentieth: a square tile has the smallest halo to
+// convert (484 values at order 6 against 532).
 int fx_auto_tx(const Dev *d, int count) {
-  int best = 32;
+  int best = 16;
   long long least = -1;
-  for (int tx : {32, 16, 8}) {
+  for (int tx : {16, 32, 8}) {
     long long t = 0;
     for (int b = 0; b < count; ++b) t += fx_tiles(d[b], tx);
     if (least < 0 || 20 * t < 19 * least) {
