@@ -28,7 +28,7 @@
 //   4. interface flags (max sensor over the WENO stencil > threshold, from
 //      the per-point tests theta > threshold) are stored and the flagged
 //      interfaces appended to a global list.
-// k_weno<DIR>  one thread per listed interface (globally compacted, so
+// k_weno       one thread per listed interface (globally compacted, so
 //   shocks cause no divergence in the central kernel and no idle lanes
 //   here): F_weno - F_central at the interface.
 // The corrections are added per point, in a fixed order, by the viscous

@@ -192,7 +192,8 @@ __device__ __forceinline__ int block_want_dt(const Dev &d, int stage0) {
 // Exponents of a CTA's largest magnitudes (e[FX_*], 0 for threads without a
 // point) and smallest ones (m: 2047 - exponent) into Scal, for the
 // fixed-point path.  Whole warps reduce with one instruction per value and
-// one thread per value looks at the CTA's result: 0.2 % of k_prims.
+// one thread per value looks at the CTA's result: about 1 us per launch at 4M
+// points.
 __device__ __forceinline__ void fx_block_raise(const Dev &d, const unsigned *e, const unsigned *m) {
   constexpr int NE = FX_TH;  // the fields of the primitive pass
   __shared__ unsigned red[NE + FX_NMIN][NT / 32];

@@ -20,8 +20,8 @@
 // inviscid runs): per direction -scale (dF_{i+1/2} - dF_{i-1/2}) over the
 // flagged interfaces, in a fixed order.
 //
-// Every kernel is instantiated for R = double (FP64 path) and R = float
-// (arithmetic of the mixed path).
+// The FP64 path forms the stencil sums in fixed point (k_grad, k_visc); the
+// mixed path marches through z in single precision (k_grad_z, k_visc_z).
 #include <type_traits>
 
 #include "s2_fixed.cuh"
