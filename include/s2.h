@@ -340,8 +340,8 @@ void s2_destroy(s2_solver *s);
  *
  * Work-list mode (S2_BATCH_WORKLIST, the default of s2_batch_create):
  * members that share their kernels (same precision, orders, WENO order,
- * tile shapes, gas model and viscous / WENO / forcing / CFL switches) form
- * a group, and each kernel of an RK stage is one launch for the whole
+ * central flux (split form or KEEP), tile shapes, gas model and viscous /
+ * WENO / forcing / CFL switches) form a group, and each kernel of an RK stage is one launch for the whole
  * group: a work list in device memory gives every CTA of the launch its
  * box and its tile in that box, the box's parameters come from a table in
  * device memory, and the persistent single-precision flux grids are

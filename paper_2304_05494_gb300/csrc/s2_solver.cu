@@ -1902,8 +1902,8 @@ const char *s2_profile_name(int kind) {
 // Batched stepping
 // ======================================================================
 // Work-list mode (default): members whose kernels are the same
-// instantiations (precision, orders, WENO order, tile shapes, gas model,
-// and the viscous / WENO / forcing / CFL switches) form a group, and every
+// instantiations (precision, orders, WENO order, central flux, tile shapes,
+// gas model, and the viscous / WENO / forcing / CFL switches) form a group, and every
 // kernel of a stage is ONE launch over the whole group: a table in device
 // memory lists, per box, the box's parameters and the CTAs of the launch
 // that work on it (BoxGrid); each CTA finds its box, copies the box's
@@ -1959,6 +1959,7 @@ namespace {
 
 bool same_kernels(const Dev &a, const Dev &b) {
   return a.mixed == b.mixed && a.npc == b.npc && a.npv == b.npv && a.weno == b.weno && a.kd.tp == b.kd.tp &&
+         (a.keep != 0) == (b.keep != 0) &&  // (the KEEP variant is a parameter of the box)
          a.tile[0] == b.tile[0] && a.tile[1] == b.tile[1] && a.tile[2] == b.tile[2] && a.viscous == b.viscous &&
          a.force == b.force && (a.cfl > 0.0) == (b.cfl > 0.0) && a.zs_set == b.zs_set &&
          (!a.force || !a.mixed || a.zs == b.zs);  // the forcing is summed by plane groups, so those keep their solo planes

@@ -1,0 +1,44 @@
+"""Which boxes share their launches in a batch, and with which shapes."""
+import numpy as np
+import pytest
+
+from paper_2304_05494_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def s2():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2304_05494_gb300 import s2 as mod
+    return mod
+
+
+@pytest.mark.parametrize("mode", ["worklist", "worklist_all"])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("keeps", [(0, -1, 0, -1), (-1, 0, 0, 2)])
+def test_split_form_and_keep_boxes_in_one_batch(s2, precision, mode, keeps):
+    """Boxes with the split form and boxes with KEEP have other flux kernels
+    and other tiles, whichever comes first: each box equals its solo run."""
+    cases = [W.taylor_green(48, mach=0.3, seed=20 + i) for i in range(len(keeps))]
+    kw = [dict(precision=precision, keep=k, threshold=0.1) for k in keeps]
+    want = []
+    for c, k in zip(cases, kw):
+        c.weno_order = 5
+        with s2.Solver.from_case(c, **k) as sv:
+            sv.set_state(c.w0)
+            sv.step(2)
+            want.append(sv.get_state())
+    solvers = [s2.Solver.from_case(c, **k) for c, k in zip(cases, kw)]
+    for sv, c in zip(solvers, cases):
+        sv.set_state(c.w0)
+    with s2.Batch(solvers, mode=mode) as b:
+        b.step(2)
+        b.sync()
+    got = [sv.get_state() for sv in solvers]
+    for sv in solvers:
+        sv.close()
+    for k, g, w in zip(keeps, got, want):
+        assert np.array_equal(g, w), k
