@@ -148,28 +148,6 @@ __device__ __forceinline__ long long fx_sum(long long hi, long long lo, int &dro
   return (t << (FX_LIMB - drop)) + (r >> drop);
 }
 
-// Weighted sum of stencil sums (the directions of a Laplacian): each limb
-// sum times a 60-bit fraction k, collected by powers of 2^30.
-struct FxAcc {
-  long long hi = 0, lo = 0, m = 0;
-  __device__ __forceinline__ void add(long long shi, long long slo, int2 k) {
-    const long long t = shi + (slo >> FX_LIMB);
-    const int r = (int)slo & FX_MASK, t0 = (int)t & FX_MASK, t1 = (int)(t >> FX_LIMB);
-    hi += (long long)t1 * k.y;
-    lo += (long long)t1 * k.x;
-    lo += (long long)t0 * k.y;
-    m += (long long)t0 * k.x;
-    m += (long long)r * k.y;
-  }
-};
-
-// Weights 1/(D2 h^2) of the three directions in one row of the grid, as
-// 60-bit fractions of 2^n.
-struct __align__(16) FxLap {
-  int2 x, y, z;
-  int n, pad;
-};
-
 // x 2^n, x and the result being normal.
 __device__ __forceinline__ double fx_ldexp(double x, int n) {
   return __hiloint2double(__double2hiint(x) + n * (1 << 20), __double2loint(x));

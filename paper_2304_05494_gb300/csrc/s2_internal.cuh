@@ -45,7 +45,6 @@ constexpr int ERR_NONFINITE = 1;
 constexpr int ERR_TIMEOUT = 2;  // a bounded wait on an asynchronous copy gave up
 constexpr int ERR_BOUNDS = 4;   // an index left its array (checked build)
 
-struct FxLap;
 struct PowTab;
 
 // Scheme constants in the arithmetic type R of a kernel (double for the
@@ -154,12 +153,10 @@ struct Dev {
   // metrics (length ny): eta_y; a_l eta_y (4/j); b_l eta_y^2 (5/j); eta_yy/eta_y; 1/eta_y
   // (a_l, b_l of the viscous order; the metric itself uses the higher order)
   const double *eta_y, *ay, *by, *ry, *dvy;
-  // units of the fixed-point stencils (s2_fixed.cuh): the derivative of an
-  // integer stencil sum, 1/(D1 h), for x and z and per row, and the weights
-  // of the Laplacian per row
-  const double *fy1;
-  double fx1, fz1;
-  const FxLap *fxl;
+  // units of the fixed-point stencils (s2_fixed.cuh), the derivatives of an
+  // integer stencil sum: 1/(D1 h) and 1/(D2 h^2) for x and z and per row
+  const double *fy1, *fy2;
+  double fx1, fz1, fx2, fz2;
   const float *eta_yf, *ayf, *byf, *ryf;  // the same in single precision
   Scal *scal;
   double *part;            // reduction partials

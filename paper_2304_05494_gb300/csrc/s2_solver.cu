@@ -53,7 +53,6 @@ struct MetricCoef {
   double av[5], bv[5];  // viscous order
   int lm, lv;
   double fx_d1, fx_d2;  // its common denominators (FxStencil)
-  double fx_x2, fx_z2;  // 1/(D2 dx^2), 1/(D2 dz^2)
 };
 // Wray's low-storage RK3 coefficients.
 const double RK_G[3] = {8.0 / 15.0, 5.0 / 12.0, 3.0 / 4.0};
@@ -102,7 +101,7 @@ __device__ void block_sum(double *v) {
 // pre-scaled coefficient tables used by the stencil kernels, in double and
 // in single precision.
 __global__ void k_metric(const double *yn, int ny, double ly, int wall, MetricCoef mc, double *eta_y, double *ay,
-                         double *by, double *ry, double *dvy, double *fy1, FxLap *fxl, float *eta_yf, float *ayf, float *byf, float *ryf) {
+                         double *by, double *ry, double *dvy, double *fy1, double *fy2, float *eta_yf, float *ayf, float *byf, float *ryf) {
   int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= ny) return;
   const double *a = mc.am, *b = mc.bm;
@@ -134,20 +133,7 @@ __global__ void k_metric(const double *yn, int ny, double ly, int wall, MetricCo
     byf[5 * j + l] = (float)(mc.bv[l] * ey * ey);
   }
   fy1[j] = ey / mc.fx_d1;
-  // Laplacian weights of the row as 60-bit fractions of the power of two
-  // above the largest
-  const double wt[3] = {mc.fx_x2, ey * ey / mc.fx_d2, mc.fx_z2};
-  int n = 0;
-  frexp(fmax(fmax(wt[0], wt[1]), wt[2]), &n);
-  int2 k[3];
-  for (int c = 0; c < 3; ++c) {
-    const long long q = (long long)ldexp(wt[c], 60 - n);
-    k[c] = make_int2((int)q & FX_MASK, (int)(q >> FX_LIMB));
-  }
-  fxl[j].x = k[0];
-  fxl[j].y = k[1];
-  fxl[j].z = k[2];
-  fxl[j].n = n;
+  fy2[j] = ey * ey / mc.fx_d2;
   ry[j] = eyy / ey;
   ryf[j] = (float)(eyy / ey);
   dvy[j] = d1;
@@ -1436,12 +1422,11 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.wbx = (grid->nx + 31) / 32;
   d.wby = (grid->ny + 7) / 8;
   const size_t map_bytes = scheme->weno_order ? (size_t)d.wbx * d.wby * grid->nz : 1;
-  const size_t o_fy = sizeof(FxLap) * grid->ny, o_pow = o_fy + sizeof(double) * grid->ny;
+  const size_t o_pow = 2 * sizeof(double) * grid->ny;
   const size_t o_map = o_pow + sizeof(PowTab);
   unsigned char *tables = (unsigned char *)dalloc(s, o_map + map_bytes);
   if (!tables) ok = false;
-  FxLap *fxl = (FxLap *)tables;
-  double *fy = (double *)(tables + o_fy);
+  double *fy = (double *)tables;
   d.wmap = tables + o_map;
   std::vector<PowTab> powt(1);
   if (!d.mixed && (d.viscous || d.kd.tp)) {
@@ -1492,7 +1477,7 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.ry = ry;
   d.dvy = dvy;
   d.fy1 = fy;
-  d.fxl = fxl;
+  d.fy2 = fy + grid->ny;
   d.eta_yf = etaf;
   d.ayf = ayf;
   d.byf = byf;
@@ -1538,10 +1523,10 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
     mc.fx_d2 = den2[d.npv];
     d.fx1 = 1.0 / (d.dx * mc.fx_d1);
     d.fz1 = 1.0 / (d.dz * mc.fx_d1);
-    mc.fx_x2 = 1.0 / (d.dx * d.dx * mc.fx_d2);
-    mc.fx_z2 = 1.0 / (d.dz * d.dz * mc.fx_d2);
+    d.fx2 = 1.0 / (d.dx * d.dx * mc.fx_d2);
+    d.fz2 = 1.0 / (d.dz * d.dz * mc.fx_d2);
     k_metric<<<(grid->ny + 127) / 128, 128, 0, s->stream>>>(ynd, grid->ny, grid->ly, d.wall_y, mc, eta, ay, by, ry,
-                                                             dvy, fy, fxl, etaf, ayf, byf, ryf);
+                                                             dvy, fy, fy + grid->ny, etaf, ayf, byf, ryf);
     e = cudaGetLastError();
   }
   std::vector<double> dv(grid->ny);

@@ -344,8 +344,9 @@ __device__ __forceinline__ double fx_d1(const int2 (&up)[NP], const int2 (&dn)[N
   return (HW ? __ll2double_rn(v) : fx_i2d(v)) * fx_ldexp(unit, drop);
 }
 
+// (in units of 2^n)
 template <int NP>
-__device__ __forceinline__ void fx_d2(FxAcc &acc, int2 c, const int2 (&up)[NP], const int2 (&dn)[NP], int2 k) {
+__device__ __forceinline__ double fx_d2(int2 c, const int2 (&up)[NP], const int2 (&dn)[NP], int n) {
   using S = FxStencil<NP>;
   long long hi = (long long)S::c2(0) * c.y, lo = (long long)S::c2(0) * c.x;
 #pragma unroll
@@ -353,7 +354,9 @@ __device__ __forceinline__ void fx_d2(FxAcc &acc, int2 c, const int2 (&up)[NP], 
     hi += (long long)S::c2(l) * (up[l - 1].y + dn[l - 1].y);
     lo += (long long)S::c2(l) * (up[l - 1].x + dn[l - 1].x);
   }
-  acc.add(hi, lo, k);
+  int drop;
+  const long long v = fx_sum<S::W2>(hi, lo, drop);
+  return fx_i2d(v, n + drop);
 }
 
 // Neighbours along x (step 1) or y (step SX) in shared memory, along z in
@@ -452,8 +455,11 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
 //   u_a X_a + tau_ab d_b u_a / mu + (c_p / Pr) (lap T + psi . grad T)
 // so mu enters with the sum into the RHS: about 55 double operations per
 // point at order 6 (169 when the stencils were in double precision too).
-// Adding the directions of a Laplacian up before its one conversion to
-// double took it from 4.61 to 3.95 ms.
+// Each direction of a Laplacian becomes a double by itself and is weighted
+// there: in one integer sum of all three, the weights and the sum's last
+// place are relative to the finest spacing, and the direction of the
+// longest cells loses the square of the cells' aspect ratio (7e-9 of it at
+// 1e5).
 template <int NP, int TX>
 __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Blk &B) {
   constexpr int SX = FxTile<NP, TX>::SX, NF = 5;
@@ -484,11 +490,8 @@ __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Bl
   for (int f = 1; f < NV; ++f) Rv[f] = V.fl[f * d.n + q];
   if (ex[5]) {
     const int c = (tid / TX + NP) * SX + tid % TX + NP;
-    const double uy1 = __ldg(d.fy1 + j), ry = __ldg(V.ry + j);
+    const double uy1 = __ldg(d.fy1 + j), uy2 = __ldg(d.fy2 + j), ry = __ldg(V.ry + j);
     const double mu = __ldg(V.mu + q), T = __ldg(V.T + p), th = __ldg(V.div + p);
-    FxLap fl;
-    ((int4 *)&fl)[0] = __ldg((const int4 *)(d.fxl + j));
-    ((int4 *)&fl)[1] = __ldg((const int4 *)(d.fxl + j) + 1);
     int2 up[NP], dn[NP];
     // Laplacians of u, v, w, T in the computational coordinates, gradients
     // of T and theta
@@ -497,22 +500,19 @@ __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Bl
     for (int f = 0; f < NF; ++f) {
       const int n = ex[f] - 1022 - 59;
       const int2 *S = sm[f] + c;
-      FxAcc acc;
 #pragma unroll
       for (int dir = 0; dir < 3; ++dir) {
         if (dir == 0) fx_near<NP>(S, 1, up, dn);
         else if (dir == 1) fx_near<NP>(S, SX, up, dn);
         else fx_near_z<NP>(src[f] + p, d.sz, ex[f], up, dn);
-        if (f < 4) fx_d2<NP>(acc, S[0], up, dn, dir == 0 ? fl.x : (dir == 1 ? fl.y : fl.z));
+        if (f < 4) {
+          const double s = fx_d2<NP>(S[0], up, dn, n);
+          lap[f] = dir == 0 ? d.fx2 * s : fma(dir == 1 ? uy2 : d.fz2, s, lap[f]);
+        }
         if (f >= 3) {
           const double unit = fx_ldexp(dir == 0 ? d.fx1 : (dir == 1 ? uy1 : d.fz1), n);
           (f == 3 ? gT : gth)[dir] = fx_d1<NP, false>(up, dn, unit);
         }
-      }
-      if (f < 4) {
-        int drop;
-        const long long v = fx_sum<FxStencil<NP>::W2 + 2>(acc.hi, acc.lo + (acc.m >> FX_LIMB), drop);
-        lap[f] = fx_i2d(v, fl.n + n + drop);
       }
     }
     double g[3][3];
