@@ -216,7 +216,10 @@ __device__ __forceinline__ void keep_pairs_tile(const R *S, R *TP, R gm1, int n)
 // the double unit executed 61 operations (64 issue clocks each); here it
 // executes 12 (the pressure difference and the sums into the RHS), the
 // integer unit the rest beside them.  On 420 x 250 x 320 points a launch
-// went from 3.85 / 3.70 / 3.64 ms (x / y / z) to 1.28 / 1.25 / 1.27.
+// takes 1.66 / 1.76 / 1.72 ms (x / y / z) instead of 3.85 / 3.70 / 3.64; of
+// these, quiet stencils (a third of v's and w's in that channel) and looking
+// for them cost 0.4 to 0.5 (1.28 / 1.25 / 1.27 with the grid's exponents for
+// every stencil, which loses the digits of quiet regions).
 // With the double unit no longer the bound, the persistent grid that
 // prefetches the next tile pays here too: with one tile per CTA the same
 // arithmetic took 2.67 / 2.77 / 2.72 ms (waiting at barriers and for the
@@ -251,8 +254,16 @@ __device__ __forceinline__ constexpr int2 acoef_limbs(int l) {
 // Pair mass fluxes m_l(a), a = -NP .. L-1, in units of 2^(E_rho + E_n - 59).
 // (rho_a + rho_b)(un_a + un_b) is formed to 2^-60 of its largest value, and
 // so is its product with a_l / 4.
+__device__ __forceinline__ int2 fx_pair(int2 r0, int2 r1, int2 n0, int2 n1, int2 k) {
+  const long long P = fx_mulhi(r0.x + r1.x, r0.y + r1.y, n0.x + n1.x, n0.y + n1.y);
+  const long long m = fx_mulhi((int)P & FX_MASK, (int)(P >> FX_LIMB), k.x, k.y);
+  return make_int2((int)m & FX_MASK, (int)(m >> FX_LIMB));
+}
+
+// loud: the fields' thresholds (FxField).  Q gets, per position a, whether
+// density (bit 0) and normal velocity (bit 1) are loud in a .. a+NP.
 template <int DIR, int NP, int LT, int W, int SA, int SCS, int SCT, int SFA>
-__device__ __forceinline__ void fx_pairs_tile(const int2 *S, int2 *TP) {
+__device__ __forceinline__ void fx_pairs_tile(const int2 *S, int2 *TP, unsigned char *Q, const int *loud) {
   constexpr int ST = LT * W;
   for (int idx = threadIdx.x; idx < ST; idx += NTHREADS) {
     int a, cc;
@@ -261,15 +272,35 @@ __device__ __forceinline__ void fx_pairs_tile(const int2 *S, int2 *TP) {
     const int2 *Sr = S + F_RHO * SFA, *Sn = S + (F_U + DIR) * SFA;
     const int q0 = (a - NP + GH) * SA + cc * SCS;
     const int2 r0 = Sr[q0], n0 = Sn[q0];
+    int rmax = r0.y, nmax = n0.y, nmin = n0.y;
 #pragma unroll
     for (int l = 1; l <= NP; ++l) {
       const int2 r1 = Sr[q0 + l * SA], n1 = Sn[q0 + l * SA];
-      const long long P = fx_mulhi(r0.x + r1.x, r0.y + r1.y, n0.x + n1.x, n0.y + n1.y);
-      const int2 k = acoef_limbs<NP>(l);
-      const long long m = fx_mulhi((int)P & FX_MASK, (int)(P >> FX_LIMB), k.x, k.y);
-      TP[(l - 1) * ST + a * SA + cc * SCT] = make_int2((int)m & FX_MASK, (int)(m >> FX_LIMB));
+      TP[(l - 1) * ST + a * SA + cc * SCT] = fx_pair(r0, r1, n0, n1, acoef_limbs<NP>(l));
+      rmax = max(rmax, r1.y);
+      nmax = max(nmax, n1.y);
+      nmin = min(nmin, n1.y);
     }
+    Q[a * SA + cc * SCT] =
+        (rmax >= loud[F_RHO] ? 1 : 0) | (nmax >= loud[F_U + DIR] || nmin <= -loud[F_U + DIR] ? 2 : 0);
   }
+}
+
+// The 2 NP + 1 values of f around point p, converted with their own exponent,
+// which is returned.
+template <int NP>
+__device__ __forceinline__ int fx_own(const double *f, long long p, long long stride, int2 (&v)[2 * NP + 1]) {
+  double x[2 * NP + 1];
+  int mag = 0;
+#pragma unroll
+  for (int l = 0; l <= 2 * NP; ++l) {
+    x[l] = __ldg(f + p + (l - NP) * stride);
+    mag = max(mag, fx_mag(x[l]));
+  }
+  const int e = fx_own_exponent(mag);
+#pragma unroll
+  for (int l = 0; l <= 2 * NP; ++l) v[l] = fx_split(x[l], e);
+  return e;
 }
 
 // The flux difference of one point: D_rho = 2 M, D_phi = phi_a M + sum_l
@@ -277,33 +308,70 @@ __device__ __forceinline__ void fx_pairs_tile(const int2 *S, int2 *TP) {
 // largest value: A collects the hi hi products, B the mixed ones.  |m| is
 // below 2^59 sum |a_l| and the lo limbs of m are not negative, so with 8
 // pairs (order 8) |B| stays below 2^59 (8 + 2.1 + 1 + 2.1) < 2^63.
+// The field values of a quiet stencil (s2_fixed.cuh) come from memory with
+// their own exponent; p: the point's padded offset.
 template <int DIR, int NP, int ST, int SA, int SFA>
-__device__ __forceinline__ void fx_flux_point(const int2 *S, const int2 *TP, int at, int ap, const int *e,
-                                              double dp, double scale, const double *prev, double *out,
-                                              long long n) {
-  int2 mp[NP], mm[NP];  // m_l(a), -m_l(a-l)
+__device__ __forceinline__ void fx_flux_point(const Dev &__restrict__ d, const int2 *S, const int2 *TP,
+                                              const unsigned char *Q, int at, int ap, const int *e, const int *loud,
+                                              long long p, double dp, double scale, const double *prev, double *out) {
+  const View<double> V = view<double>(d);
+  const double *src[5] = {V.rho, V.u, V.v, V.ww, V.H};  // by F_*
+  const long long stride = DIR == 0 ? 1 : (DIR == 1 ? d.sy : d.sz);
+  const int q = Q[at] | Q[at - NP * SA];
+  int2 mp[NP], mm[NP], v[2 * NP + 1];  // m_l(a), -m_l(a-l), values of a field
+  const int2 *Sr = S + F_RHO * SFA, *Sn = S + (F_U + DIR) * SFA;
+  int er = e[F_RHO], en = e[F_U + DIR];
+#pragma unroll
+  for (int l = 0; l <= 2 * NP; ++l) v[l] = Sn[ap + (l - NP) * SA];
+  if (q == 3) {
+#pragma unroll
+    for (int l = 1; l <= NP; ++l) {
+      mp[l - 1] = TP[(l - 1) * ST + at];
+      mm[l - 1] = TP[(l - 1) * ST + at - l * SA];
+    }
+  } else {
+    int2 r[2 * NP + 1];
+#pragma unroll
+    for (int l = 0; l <= 2 * NP; ++l) r[l] = Sr[ap + (l - NP) * SA];
+    if (!(q & 1)) er = fx_own<NP>(src[F_RHO], p, stride, r);
+    if (!(q & 2)) en = fx_own<NP>(src[F_U + DIR], p, stride, v);
+#pragma unroll
+    for (int l = 1; l <= NP; ++l) {
+      mp[l - 1] = fx_pair(r[NP], r[NP + l], v[NP], v[NP + l], acoef_limbs<NP>(l));
+      mm[l - 1] = fx_pair(r[NP - l], r[NP], v[NP - l], v[NP], acoef_limbs<NP>(l));
+    }
+  }
   int Ml = 0, Mh = 0;
 #pragma unroll
   for (int l = 1; l <= NP; ++l) {
-    mp[l - 1] = TP[(l - 1) * ST + at];
-    const int2 m = TP[(l - 1) * ST + at - l * SA];
-    mm[l - 1] = make_int2(-m.x, -m.y);
+    mm[l - 1] = make_int2(-mm[l - 1].x, -mm[l - 1].y);
     Ml += mp[l - 1].x + mm[l - 1].x;
     Mh += mp[l - 1].y + mm[l - 1].y + (Ml >> FX_LIMB);
     Ml &= FX_MASK;
   }
-  const int eM = e[F_RHO] + e[F_U + DIR] - 2 * 1022 - 59;  // unit of m
-  const double M = fx_i2d((long long)Mh * (1 << FX_LIMB) + Ml);
-  out[0] = fma(-fx_ldexp(scale, eM + 1), M, prev[0]);
+  const int eM = er + en - (2 * 1022 + 59);  // unit of m
+  out[0] = fma(-fx_ldexp(scale, eM + 1), fx_i2d((long long)Mh * (1 << FX_LIMB) + Ml), prev[0]);
+  // (the normal velocity first, whose values are at hand)
 #pragma unroll
-  for (int f = 1; f < 5; ++f) {
-    const int2 *Sf = S + f * SFA;  // F_U .. F_H follow F_RHO
-    const int2 c = Sf[ap];
-    long long A = (long long)Mh * c.y;
-    long long B = (long long)Mh * c.x + (long long)Ml * c.y;
+  for (int g = 0; g < 4; ++g) {
+    const int f = g == 0 ? F_U + DIR : (g <= DIR ? g : g + 1);
+    int ef = en;
+    if (g > 0) {
+      const int2 *Sf = S + f * SFA;  // F_U .. F_H follow F_RHO
+      ef = e[f];
+      unsigned any = 0;  // bits from 2 loud on: a value outside -loud .. loud
+#pragma unroll
+      for (int l = 0; l <= 2 * NP; ++l) {
+        v[l] = Sf[ap + (l - NP) * SA];
+        any |= (unsigned)(v[l].y + loud[f]);
+      }
+      if (any < 2u * (unsigned)loud[f]) ef = fx_own<NP>(src[f], p, stride, v);
+    }
+    long long A = (long long)Mh * v[NP].y;
+    long long B = (long long)Mh * v[NP].x + (long long)Ml * v[NP].y;
 #pragma unroll
     for (int l = 1; l <= NP; ++l) {
-      const int2 vp = Sf[ap + l * SA], vm = Sf[ap - l * SA];
+      const int2 vp = v[NP + l], vm = v[NP - l];
       A += (long long)mp[l - 1].y * vp.y;
       B += (long long)mp[l - 1].y * vp.x;
       B += (long long)mp[l - 1].x * vp.y;
@@ -313,10 +381,10 @@ __device__ __forceinline__ void fx_flux_point(const int2 *S, const int2 *TP, int
     }
     const double D = fx_i2d(A + (B >> FX_LIMB));
     // unit of D: 2^60 times the units of m and phi
-    const int eD = eM + e[f] - 1022 + 1;
+    const int eD = eM + ef - 1022 + 1;
     double r = fma(-fx_ldexp(scale, eD), D, prev[f]);
     if (f == 1 + DIR) r = fma(-scale, dp, r);
-    out[f * n] = r;
+    out[f * d.n] = r;
   }
 }
 
@@ -350,7 +418,8 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
   const int ntiles = tg.count();
   // split form in double precision: fixed point where the fields allow it
   constexpr bool FX = sizeof(R) == 8 && TV != 2;
-  __shared__ int fx_e[8];  // exponents of rho, u, v, w, H by F_*; [5]: fixed point
+  __shared__ int fx_e[6], fx_l[5];  // exponents and thresholds of rho, u, v, w, H by F_*; [5]: fixed point
+  __shared__ unsigned char fx_q[FX ? ST : 1];
 
   const int tid = threadIdx.x;
   const int n = DIR == 0 ? d.nx : (DIR == 1 ? d.ny : d.nz);
@@ -386,13 +455,14 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
       if ((int)B.x + j * G < ntiles) issue((int)B.x + j * G, j);
   }
   if (FX && tid == 32) {
-    const FxScale fx = fx_scale(d);
-    fx_e[F_RHO] = fx.e[FX_RHO];
-    fx_e[F_U] = fx.e[FX_U];
-    fx_e[F_V] = fx.e[FX_V];
-    fx_e[F_W] = fx.e[FX_W];
-    fx_e[F_H] = fx.e[FX_H];
-    fx_e[5] = fx.ok;
+    const int field[5] = {FX_RHO, FX_U, FX_V, FX_W, FX_H};
+    bool ok = fx_flux_ok(d);
+    fx_e[5] = ok;
+    for (int f = 0; f < 5; ++f) {
+      const FxField x = fx_field(d, field[f], ok);
+      fx_e[f] = x.e;
+      fx_l[f] = f == 0 ? 8 * x.loud : x.loud;
+    }
   }
   __syncthreads();
   const bool fixed = FX && fx_e[5];
@@ -456,7 +526,7 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
     if constexpr (TV == 2) {
       keep_pairs_tile<DIR, R, NP, LT, W, SA, SCS, SCT, SFA>(S, TP, K.gamma - R(1), d.keep);
     } else if (fixed) {
-      if constexpr (FX) fx_pairs_tile<DIR, NP, LT, W, SA, SCS, SCT, SFA>((const int2 *)S, (int2 *)TP);
+      if constexpr (FX) fx_pairs_tile<DIR, NP, LT, W, SA, SCS, SCT, SFA>((const int2 *)S, (int2 *)TP, fx_q, fx_l);
     } else
     for (int idx = tid; idx < ST; idx += NTHREADS) {
       int a, cc;                            // a in 0..LT-1 <-> position a-NP
@@ -574,8 +644,11 @@ __device__ __forceinline__ void flux_body(const FluxMaps &maps, const Dev &__res
       R scale = DIR == 0 ? K.idx : (DIR == 1 ? (FX ? ey[pp] : __ldg(V.eta_y + pj)) : K.idz);
       if constexpr (FX) {
         if (fixed) {
-          fx_flux_point<DIR, NP, ST, SA, SFA>((const int2 *)S, (const int2 *)TP, at, ap, fx_e, dp, scale, prev[pp],
-                                              V.fl + q[pp], d.n);
+          const long long p = pidx(d, DIR == 0 ? x0 + ta[pp] : x0 + tc, pj, DIR == 2 ? z0 + ta[pp] : z0);
+          const long long s = DIR == 0 ? 1 : (DIR == 1 ? d.sy : d.sz);
+          if (!(S2_OK_IDX(d, p - NP * s, d.np) && S2_OK_IDX(d, p + NP * s, d.np))) continue;
+          fx_flux_point<DIR, NP, ST, SA, SFA>(d, (const int2 *)S, (const int2 *)TP, fx_q, at, ap, fx_e, fx_l, p, dp,
+                                              scale, prev[pp], V.fl + q[pp]);
           continue;
         }
       }

@@ -14,10 +14,9 @@ namespace s2 {
 constexpr int GH = 4;
 constexpr int NV = 5;
 
-// Fields with a fixed-point exponent (s2_fixed.cuh); the first FX_NMIN also
-// record their smallest magnitude.
-enum { FX_RHO = 0, FX_T, FX_P, FX_U, FX_V, FX_W, FX_H, FX_TH, FX_NF };
-constexpr int FX_NMIN = 3;
+// Fields with a fixed-point exponent (s2_fixed.cuh); all but the dilatation
+// FX_TH come from the primitive pass.
+enum { FX_RHO = 0, FX_T, FX_U, FX_V, FX_W, FX_H, FX_TH, FX_NF };
 
 // Device-side scalars of one solver.
 struct Scal {
@@ -32,11 +31,11 @@ struct Scal {
   long long nstep;        // completed RK3 steps (decides the dt recomputation on the device)
   double red[8];          // results of the last stats reduction
   // biased exponent of the largest magnitude of each field of this RHS
-  // evaluation, and 2047 - that of the smallest (0: nothing seen yet); the
-  // primitive, ghost and gradient passes raise them, the pass that ends
-  // the evaluation clears them
-  unsigned int fx_e[FX_NF], fx_m[FX_NMIN];
-  unsigned int fx_pad;
+  // evaluation, and 2047 - that of the smallest density (0: nothing seen
+  // yet); the primitive, ghost and gradient passes raise them, the pass that
+  // ends the evaluation clears them
+  unsigned int fx_e[FX_NF];
+  unsigned int fx_m;
 };
 
 // Error bits kernels OR into Scal::status (mapped on the host to

@@ -176,25 +176,24 @@ __device__ __forceinline__ int block_want_dt(const Dev &d, int stage0) {
 }
 
 // Exponents of a CTA's largest magnitudes (e[FX_*], 0 for threads without a
-// point) and smallest ones (m: 2047 - exponent) into Scal, for the
+// point) and of its smallest density (m: 2047 - exponent) into Scal, for the
 // fixed-point path.  Whole warps reduce with one instruction per value and
 // one thread per value looks at the CTA's result: about 1 us per launch at 4M
 // points.
-__device__ __forceinline__ void fx_block_raise(const Dev &d, const unsigned *e, const unsigned *m) {
+__device__ __forceinline__ void fx_block_raise(const Dev &d, const unsigned *e, unsigned m) {
   constexpr int NE = FX_TH;  // the fields of the primitive pass
-  __shared__ unsigned red[NE + FX_NMIN][NT / 32];
+  __shared__ unsigned red[NE + 1][NT / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-  for (int f = 0; f < NE + FX_NMIN; ++f) {
-    const unsigned r = __reduce_max_sync(0xffffffffu, f < NE ? e[f] : m[f - NE]);
+  for (int f = 0; f <= NE; ++f) {
+    const unsigned r = __reduce_max_sync(0xffffffffu, f < NE ? e[f] : m);
     if (lane == 0) red[f][wid] = r;
   }
   __syncthreads();
-  if (threadIdx.x < NE + FX_NMIN) {
+  if (threadIdx.x <= NE) {
     unsigned r = 0;
     for (int w = 0; w < NT / 32; ++w) r = max(r, red[threadIdx.x][w]);
-    unsigned *at = threadIdx.x < NE ? &d.scal->fx_e[threadIdx.x] : &d.scal->fx_m[threadIdx.x - NE];
-    if (__ldcg(at) < r) atomicMax(at, r);
+    fx_raise(threadIdx.x < NE ? &d.scal->fx_e[threadIdx.x] : &d.scal->fx_m, r);
   }
 }
 
@@ -212,7 +211,7 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
   reset_counts(d, q);
   const int want_dt = block_want_dt(d, stage0);
   double sr = 0.0;
-  unsigned fe[FX_TH] = {0}, fm[FX_NMIN] = {0};
+  unsigned fe[FX_TH] = {0}, fm = 0;
   if (q < d.n) {
     int i, j, k;
     point_of(d, q, i, j, k);
@@ -247,11 +246,10 @@ __device__ __forceinline__ void prims_body(const Dev &__restrict__ d, const Blk 
       V.p[p] = pr;
       V.H[p] = H;
     }
-    const double fv[FX_TH] = {rho, T, pr, u, v, ww, H};  // by FX_*
+    const double fv[FX_TH] = {rho, T, u, v, ww, H};  // by FX_*
 #pragma unroll
     for (int f = 0; f < FX_TH; ++f) fe[f] = fx_exponent(fv[f]);
-#pragma unroll
-    for (int f = 0; f < FX_NMIN; ++f) fm[f] = 2047u - fe[f];
+    fm = 2047u - fe[FX_RHO];
     double mu = 0.0;
     if (d.viscous) {
       mu = viscosity_fixed(d, T);
@@ -471,10 +469,11 @@ __device__ __forceinline__ void ghost_prim_body(const Dev &__restrict__ d, const
     const R h = K.tp ? fma(K.R_gas, T, tp_e(K, T, rcp_pos(T))) : K.cp * T;
     const R H = h + R(0.5) * (u * u + v * v + ww * ww);
     V.H[dp] = H;
-    if (sizeof(R) == 8 && d.fx) {  // the mirrored u, v, w and p have their interior magnitudes
-      fx_raise(d.scal, FX_RHO, fx_exponent(r));
-      fx_raise(d.scal, FX_T, fx_exponent(T));
-      fx_raise(d.scal, FX_H, fx_exponent(H));
+    if (sizeof(R) == 8 && d.fx) {  // the mirrored u, v and w have their interior magnitudes
+      fx_raise(&d.scal->fx_e[FX_RHO], fx_exponent(r));
+      fx_raise(&d.scal->fx_m, 2047 - fx_exponent(r));
+      fx_raise(&d.scal->fx_e[FX_T], fx_exponent(T));
+      fx_raise(&d.scal->fx_e[FX_H], fx_exponent(H));
     }
     if (!(T > R(0))) atomicOr(&d.scal->status, ERR_NONFINITE);
   }
@@ -519,7 +518,7 @@ __device__ __forceinline__ void ghost_aux_body(const Dev &__restrict__ d, const 
     R ux = V.g[0 * d.n + q], vy = V.g[4 * d.n + q], wz = V.g[8 * d.n + q];
     const R dv = -ux + vy - wz;
     V.div[dp] = dv;
-    if (sizeof(R) == 8 && d.fx) fx_raise(d.scal, FX_TH, fx_exponent(dv));
+    if (sizeof(R) == 8 && d.fx) fx_raise(&d.scal->fx_e[FX_TH], fx_exponent(dv));
   }
 }
 

@@ -291,25 +291,30 @@ __device__ __noinline__ void visc_point(const Dev &__restrict__ d, int j, long l
 }
 
 // --------------------------------------- fixed-point passes (FP64 path)
-// The stencil sums of the gradient and viscous passes in 59-bit fixed point
+// The stencil sums of the gradient and viscous passes in 62-bit fixed point
 // (s2_fixed.cuh).  A CTA owns a TX x 256/TX tile of one z-plane: the fields are
-// converted once into shared memory with an NP-point x-y halo; the 2 NP
-// neighbours along z are read from memory (L2) and converted by the thread
-// that needs them.  One plane per CTA keeps small boxes spread over the
-// chip.  On 420 x 250 x 320 points at order 6 a launch of the gradient pass
-// went from 3.53 to 1.51 ms (double and integer unit both near 3/4 busy),
-// of the viscous pass from 10.33 to 3.85 ms (double unit).  Four CTAs per
-// multiprocessor (64 registers) hide the latencies better than three, though
-// the viscous pass spills: 1.69 -> 1.51 and 3.97 -> 3.85 ms.
+// converted once into shared memory with an NP-point x-y halo; the values
+// along z are read from memory (L2) and converted, with their own exponent, by
+// the thread that needs them.  One plane per CTA keeps small boxes spread over
+// the chip.  On 420 x 250 x 320 points (a channel, a tenth of whose v and w
+// stencils are quiet) at order 6 a launch of the gradient pass takes 1.96 ms,
+// 3.53 in double (integer unit 72 % busy, double unit 61 %), of the viscous
+// pass 5.18 ms, 10.33 in double (double unit 62 %, integer unit 58 %).  With
+// the grid's exponents for every stencil, which loses the digits of quiet
+// regions, they took 1.51 and 4.2 ms.  Four CTAs per multiprocessor (64
+// registers) hide the latencies better than three: 1.96 for 2.31 ms, 5.18 for
+// 5.3.
 template <int NP, int TX>
 struct FxTile {
   static constexpr int TY = NT / TX, SX = TX + 2 * NP, SIZE = SX * (TY + 2 * NP);
 };
 
-// Fields src[0..NF-1] of plane k around (x0, y0) into sm as limbs.
+// Fields src[0..NF-1] of plane k around (x0, y0) into sm as words; bit f of lq
+// says whether the value of field f is loud (s2_fixed.cuh).
 template <int NP, int TX, int NF>
-__device__ __forceinline__ void fx_stage(const Dev &d, const double *const (&src)[NF], const int *e, int x0, int y0,
-                                         int k, int2 (*sm)[FxTile<NP, TX>::SIZE]) {
+__device__ __forceinline__ void fx_stage(const Dev &d, const double *const (&src)[NF], const int *e, const int *loud,
+                                         int x0, int y0, int k, long long (*sm)[FxTile<NP, TX>::SIZE],
+                                         unsigned char *lq) {
   constexpr int SX = FxTile<NP, TX>::SX, SIZE = FxTile<NP, TX>::SIZE;
 #pragma unroll
   for (int s = 0; s < (SIZE + NT - 1) / NT; ++s) {
@@ -319,93 +324,164 @@ __device__ __forceinline__ void fx_stage(const Dev &d, const double *const (&src
       const long long p = pidx(d, i, j, k);
       if (S2_OK_IDX(d, p, d.np)) {
         double x[NF];
+        unsigned bits = 0;
 #pragma unroll
         for (int f = 0; f < NF; ++f) x[f] = __ldg(src[f] + p);
 #pragma unroll
-        for (int f = 0; f < NF; ++f) sm[f][pos] = fx_split(x[f], e[f]);
+        for (int f = 0; f < NF; ++f) {
+          const long long v = fx_word(x[f], e[f]);
+          sm[f][pos] = v;
+          bits |= (unsigned)(fx_hi(v) + loud[f]) >= 2u * (unsigned)loud[f] ? 1u << f : 0u;
+        }
+        lq[pos] = (unsigned char)bits;
       }
     }
   }
 }
 
-// Limb sums of the first and second derivative along one direction from the
-// neighbours up[l-1] = f_{+l} and dn[l-1] = f_{-l}.
-template <int NP, bool HW>
-__device__ __forceinline__ double fx_d1(const int2 (&up)[NP], const int2 (&dn)[NP], double unit) {
-  using S = FxStencil<NP>;
-  long long hi = 0, lo = 0;
+// Fields with a loud value among the neighbours along x (step 1) or y (SX).
+template <int NP>
+__device__ __forceinline__ unsigned fx_near_loud(const unsigned char *lq, int step) {
+  unsigned b = 0;
 #pragma unroll
-  for (int l = 1; l <= NP; ++l) {
-    hi += (long long)S::c1(l) * (up[l - 1].y - dn[l - 1].y);
-    lo += (long long)S::c1(l) * (up[l - 1].x - dn[l - 1].x);
-  }
-  int drop;
-  const long long v = fx_sum<S::W1>(hi, lo, drop);
-  return (HW ? __ll2double_rn(v) : fx_i2d(v)) * fx_ldexp(unit, drop);
+  for (int l = 1; l <= NP; ++l) b |= lq[l * step] | lq[-l * step];
+  return b;
 }
 
-// (in units of 2^n)
-template <int NP>
-__device__ __forceinline__ double fx_d2(int2 c, const int2 (&up)[NP], const int2 (&dn)[NP], int n) {
+// First derivative along one direction, from the neighbours up[l-1] = f_{+l}
+// and dn[l-1] = f_{-l} in units of 2^n; h = 1/(D1 spacing).  HW: converted on
+// the double unit.
+template <int NP, bool HW>
+__device__ __forceinline__ double fx_d1(const long long (&up)[NP], const long long (&dn)[NP], int n, double h) {
   using S = FxStencil<NP>;
-  long long hi = (long long)S::c2(0) * c.y, lo = (long long)S::c2(0) * c.x;
+  FxSum s;
 #pragma unroll
   for (int l = 1; l <= NP; ++l) {
-    hi += (long long)S::c2(l) * (up[l - 1].y + dn[l - 1].y);
-    lo += (long long)S::c2(l) * (up[l - 1].x + dn[l - 1].x);
+    s.add(S::c1(l), up[l - 1] - dn[l - 1]);
   }
   int drop;
-  const long long v = fx_sum<S::W2>(hi, lo, drop);
+  const long long v = s.value<S::W1>(drop);
+  return HW ? __ll2double_rn(v) * fx_ldexp(h, n + drop) : fx_i2d(v, n + drop) * h;
+}
+
+// Second derivative times D2 spacing^2.
+template <int NP>
+__device__ __forceinline__ double fx_d2(long long c, const long long (&up)[NP], const long long (&dn)[NP], int n) {
+  using S = FxStencil<NP>;
+  FxSum s;
+  s.add(S::c2(0), c);
+#pragma unroll
+  for (int l = 1; l <= NP; ++l) {
+    s.add(S::c2(l), up[l - 1] + dn[l - 1]);
+  }
+  int drop;
+  const long long v = s.value<S::W2>(drop);
   return fx_i2d(v, n + drop);
 }
 
-// Neighbours along x (step 1) or y (step SX) in shared memory, along z in
-// memory.
+// Neighbours along x (step 1) or y (step SX) in shared memory.
 template <int NP>
-__device__ __forceinline__ void fx_near(const int2 *S, int step, int2 (&up)[NP], int2 (&dn)[NP]) {
+__device__ __forceinline__ void fx_near(const long long *S, int step, long long (&up)[NP], long long (&dn)[NP]) {
 #pragma unroll
   for (int l = 1; l <= NP; ++l) {
     up[l - 1] = S[l * step];
     dn[l - 1] = S[-l * step];
   }
 }
-template <int NP>
-__device__ __forceinline__ void fx_near_z(const double *f, long long sz, int e, int2 (&up)[NP], int2 (&dn)[NP]) {
-  double a[NP], b[NP];
+
+// Neighbours (and the centre, CEN) at a stride in memory, with the exponent
+// of the largest, which is returned.
+template <int NP, bool CEN>
+__device__ __forceinline__ int fx_near_mem(const double *f, long long s, long long (&up)[NP], long long (&dn)[NP],
+                                           long long &c) {
+  double a[NP], b[NP], x = 0.0;
 #pragma unroll
   for (int l = 1; l <= NP; ++l) {
-    a[l - 1] = __ldg(f + l * sz);
-    b[l - 1] = __ldg(f - l * sz);
+    a[l - 1] = __ldg(f + l * s);
+    b[l - 1] = __ldg(f - l * s);
   }
+  if (CEN) x = __ldg(f);
+  int mag = fx_mag(x);
+#pragma unroll
+  for (int l = 0; l < NP; ++l) mag = max(mag, max(fx_mag(a[l]), fx_mag(b[l])));
+  const int e = fx_own_exponent(mag);
+#pragma unroll
+  for (int l = 0; l < NP; ++l) {
+    up[l] = fx_word(a[l], e);
+    dn[l] = fx_word(b[l], e);
+  }
+  c = fx_word(x, e);
+  return e;
+}
+
+// First (D1, times h) and second (D2, as fx_d2) derivative of a quiet stencil
+// of f, in double from memory: the divergent warps wait for the loads, and
+// with integers and the stencil's own exponent these cost the same.
+template <int NP, bool D1, bool D2>
+__device__ __noinline__ double2 fx_quiet_point(const double *f, long long s, double h) {
+  using S = FxStencil<NP>;
+  double a = 0.0, b = D2 ? (double)S::c2(0) * __ldg(f) : 0.0;
 #pragma unroll
   for (int l = 1; l <= NP; ++l) {
-    up[l - 1] = fx_split(a[l - 1], e);
-    dn[l - 1] = fx_split(b[l - 1], e);
+    const double up = __ldg(f + l * s), dn = __ldg(f - l * s);
+    if (D1) a = fma((double)S::c1(l), up - dn, a);
+    if (D2) b = fma((double)S::c2(l), up + dn, b);
+  }
+  return make_double2(a * h, b);
+}
+
+// Gradient (D1) and Laplacian (D2) of a field in the computational
+// coordinates at one point: S in shared memory, f in memory; lx, ly: the
+// stencil is loud; uy1, uy2: the row's 1/(D1 h), 1/(D2 h^2).
+template <int NP, int SX, bool D1, bool D2>
+__device__ __forceinline__ void fx_derivs(const Dev &d, const long long *S, const double *f, int e, bool lx, bool ly,
+                                          double uy1, double uy2, double (&grad)[3], double &lap) {
+  long long up[NP], dn[NP], cen = S[0];
+#pragma unroll
+  for (int dir = 0; dir < 3; ++dir) {
+    const double h = dir == 0 ? d.fx1 : (dir == 1 ? uy1 : d.fz1);
+    int n = e - FX_UNIT;
+    if (dir < 2) {
+      fx_near<NP>(S, dir == 0 ? 1 : SX, up, dn);
+    } else {
+      n = fx_near_mem<NP, D2>(f, d.sz, up, dn, cen) - FX_UNIT;
+    }
+    double2 D;
+    if (dir == 0 ? !lx : (dir == 1 ? !ly : false)) {
+      D = fx_quiet_point<NP, D1, D2>(f, dir == 0 ? 1 : d.sy, h);
+    } else {
+      if (D1) D.x = fx_d1<NP, false>(up, dn, n, h);
+      if (D2) D.y = fx_d2<NP>(cen, up, dn, n);
+    }
+    if (D1) grad[dir] = D.x;
+    if (D2) lap = dir == 0 ? d.fx2 * D.y : fma(dir == 1 ? uy2 : d.fz2, D.y, lap);
   }
 }
 
-// Velocity gradients (stored), theta = div u and the sensor test.  The x
-// derivatives are converted on the integer unit, the others on the double
-// unit, which balances the two.
+// Velocity gradients (stored), theta = div u and the sensor test, converted
+// on the double unit, which is less busy than the integer one here.
 template <int NP, int TX>
 __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Blk &B) {
   constexpr int SX = FxTile<NP, TX>::SX;
-  __shared__ int2 sm[3][FxTile<NP, TX>::SIZE];
-  __shared__ int ex[4];  // exponents of u, v, w; fixed point or not
+  __shared__ long long sm[3][FxTile<NP, TX>::SIZE];
+  __shared__ unsigned char lq[FxTile<NP, TX>::SIZE];
+  __shared__ int ex[4], loud[3];  // exponents and thresholds of u, v, w; [3]: fixed point or not
   __shared__ unsigned red[NT / 32];
   const View<double> V = view<double>(d);
   const int tid = threadIdx.x, x0 = B.x * TX, y0 = B.y * FxTile<NP, TX>::TY, k = B.z;
   const int i = x0 + tid % TX, j = y0 + tid / TX;
   if (tid == 0) {
-    const FxScale fx = fx_scale(d);
-    ex[0] = fx.e[FX_U];
-    ex[1] = fx.e[FX_V];
-    ex[2] = fx.e[FX_W];
-    ex[3] = fx.ok;
+    bool ok = fx_ok(d);
+    ex[3] = ok;
+    for (int a = 0; a < 3; ++a) {
+      const FxField f = fx_field(d, FX_U + a, ok);
+      ex[a] = f.e;
+      loud[a] = f.loud_word;
+    }
   }
   __syncthreads();
   const double *vel[3] = {V.u, V.v, V.ww};
-  if (ex[3]) fx_stage<NP, TX, 3>(d, vel, ex, x0, y0, k, sm);
+  if (ex[3]) fx_stage<NP, TX, 3>(d, vel, ex, loud, x0, y0, k, sm, lq);
   __syncthreads();
   unsigned eth = 0;
   const long long p = pidx(d, i, j, k), q = ((long long)k * d.ny + j) * d.nx + i;
@@ -415,16 +491,19 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
     if (ex[3]) {
       const double uy = __ldg(d.fy1 + j);
       const int c = (tid / TX + NP) * SX + tid % TX + NP;
+      const unsigned lx = fx_near_loud<NP>(lq + c, 1), ly = fx_near_loud<NP>(lq + c, SX);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const int n = ex[a] - 1022 - 59;  // unit 2^(E - 59)
-        int2 up[NP], dn[NP];
+        const int n = ex[a] - FX_UNIT;
+        long long up[NP], dn[NP], cen;
         fx_near<NP>(sm[a] + c, 1, up, dn);
-        g[a][0] = fx_d1<NP, false>(up, dn, fx_ldexp(d.fx1, n));
+        g[a][0] = lx >> a & 1 ? fx_d1<NP, true>(up, dn, n, d.fx1)
+                              : fx_quiet_point<NP, true, false>(vel[a] + p, 1, d.fx1).x;
         fx_near<NP>(sm[a] + c, SX, up, dn);
-        g[a][1] = fx_d1<NP, true>(up, dn, fx_ldexp(uy, n));
-        fx_near_z<NP>(vel[a] + p, d.sz, ex[a], up, dn);
-        g[a][2] = fx_d1<NP, true>(up, dn, fx_ldexp(d.fz1, n));
+        g[a][1] = ly >> a & 1 ? fx_d1<NP, true>(up, dn, n, uy)
+                              : fx_quiet_point<NP, true, false>(vel[a] + p, d.sy, uy).x;
+        const int nz = fx_near_mem<NP, false>(vel[a] + p, d.sz, up, dn, cen) - FX_UNIT;
+        g[a][2] = fx_d1<NP, true>(up, dn, nz, d.fz1);
       }
     } else {
       grad_point<NP>(d, j, p, &g[0][0]);
@@ -444,7 +523,7 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
     __syncthreads();
     if (tid == 0) {
       for (int w = 0; w < NT / 32; ++w) eth = max(eth, red[w]);
-      fx_raise(d.scal, FX_TH, (int)eth);
+      fx_raise(&d.scal->fx_e[FX_TH], eth);
     }
   }
 }
@@ -463,24 +542,30 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
 template <int NP, int TX>
 __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Blk &B) {
   constexpr int SX = FxTile<NP, TX>::SX, NF = 5;
-  __shared__ int2 sm[NF][FxTile<NP, TX>::SIZE];
-  __shared__ int ex[NF + 1];  // exponents of u, v, w, T, theta; fixed point or not
+  __shared__ long long sm[NF][FxTile<NP, TX>::SIZE];
+  __shared__ unsigned char lq[FxTile<NP, TX>::SIZE];
+  __shared__ int ex[NF + 1], loud[NF];  // exponents and thresholds of u, v, w, T, theta; [NF]: fixed point or not
   const View<double> V = view<double>(d);
   const Consts<double> &K = d.kd;
   const int tid = threadIdx.x, x0 = B.x * TX, y0 = B.y * FxTile<NP, TX>::TY, k = B.z;
   const int i = x0 + tid % TX, j = y0 + tid / TX;
+  __shared__ const double *at[3];
   if (tid == 0) {
-    const FxScale fx = fx_scale(d);
-    ex[0] = fx.e[FX_U];
-    ex[1] = fx.e[FX_V];
-    ex[2] = fx.e[FX_W];
-    ex[3] = fx.e[FX_T];
-    ex[4] = fx.e[FX_TH];
-    ex[5] = fx.ok;
+    at[0] = V.u;
+    at[1] = V.v;
+    at[2] = V.ww;
+    const int field[NF] = {FX_U, FX_V, FX_W, FX_T, FX_TH};
+    bool ok = fx_ok(d);
+    for (int f = 0; f < NF; ++f) {
+      const FxField x = fx_field(d, field[f], ok);
+      ex[f] = x.e;
+      loud[f] = x.loud_word;
+    }
+    ex[NF] = ok;
   }
   __syncthreads();
   const double *src[NF] = {V.u, V.v, V.ww, V.T, V.div};
-  if (ex[5]) fx_stage<NP, TX, NF>(d, src, ex, x0, y0, k, sm);
+  if (ex[NF]) fx_stage<NP, TX, NF>(d, src, ex, loud, x0, y0, k, sm, lq);
   __syncthreads();
   if (i >= d.nx || j >= d.ny) return;
   const long long p = pidx(d, i, j, k), q = ((long long)k * d.ny + j) * d.nx + i;
@@ -488,33 +573,26 @@ __device__ __forceinline__ void visc_fx_body(const Dev &__restrict__ d, const Bl
   double Rv[NV];
 #pragma unroll
   for (int f = 1; f < NV; ++f) Rv[f] = V.fl[f * d.n + q];
-  if (ex[5]) {
+  if (ex[NF]) {
     const int c = (tid / TX + NP) * SX + tid % TX + NP;
     const double uy1 = __ldg(d.fy1 + j), uy2 = __ldg(d.fy2 + j), ry = __ldg(V.ry + j);
     const double mu = __ldg(V.mu + q), T = __ldg(V.T + p), th = __ldg(V.div + p);
-    int2 up[NP], dn[NP];
     // Laplacians of u, v, w, T in the computational coordinates, gradients
     // of T and theta
-    double lap[4], gT[3], gth[3];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      const int n = ex[f] - 1022 - 59;
-      const int2 *S = sm[f] + c;
-#pragma unroll
-      for (int dir = 0; dir < 3; ++dir) {
-        if (dir == 0) fx_near<NP>(S, 1, up, dn);
-        else if (dir == 1) fx_near<NP>(S, SX, up, dn);
-        else fx_near_z<NP>(src[f] + p, d.sz, ex[f], up, dn);
-        if (f < 4) {
-          const double s = fx_d2<NP>(S[0], up, dn, n);
-          lap[f] = dir == 0 ? d.fx2 * s : fma(dir == 1 ? uy2 : d.fz2, s, lap[f]);
-        }
-        if (f >= 3) {
-          const double unit = fx_ldexp(dir == 0 ? d.fx1 : (dir == 1 ? uy1 : d.fz1), n);
-          (f == 3 ? gT : gth)[dir] = fx_d1<NP, false>(up, dn, unit);
-        }
-      }
+    double lap[4], gT[3], gth[3], none[3];
+    const unsigned nx = fx_near_loud<NP>(lq + c, 1), ny = fx_near_loud<NP>(lq + c, SX);
+    const unsigned lx = nx | lq[c], ly = ny | lq[c];
+    // (a loop: unrolled, the pass waits for the instruction cache)
+#pragma unroll 1
+    for (int f = 0; f < 3; ++f) {
+      double l;
+      fx_derivs<NP, SX, false, true>(d, sm[f] + c, at[f] + p, ex[f], lx >> f & 1, ly >> f & 1, uy1, uy2, none, l);
+      if (f == 0) lap[0] = l;
+      if (f == 1) lap[1] = l;
+      if (f == 2) lap[2] = l;
     }
+    fx_derivs<NP, SX, true, true>(d, sm[3] + c, src[3] + p, ex[3], lx >> 3 & 1, ly >> 3 & 1, uy1, uy2, gT, lap[3]);
+    fx_derivs<NP, SX, true, false>(d, sm[4] + c, src[4] + p, ex[4], nx >> 4 & 1, ny >> 4 & 1, uy1, uy2, gth, none[0]);
     double g[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)

@@ -84,3 +84,55 @@ def test_diffusion_along_the_long_side_of_the_cells(s2, aspect, order):
     err = np.max(np.abs(got - want)) / scale
     print("aspect %g, order %d: error %.2e" % (aspect, order, err))
     assert err < TOL
+
+
+def jet(c, contrast, unit):
+    """A state uniform along direction c whose velocities fall from 0.4 in the
+    middle of the box to 1e-30 at its edge, with the density between unit and
+    unit times the contrast.  (Along c the pressure differences are exactly
+    zero, so the c momentum shows the transport and diffusion alone.)"""
+    n = [40, 36, 44]
+    n[c] = 9
+    X = np.meshgrid(*(np.arange(m) * L / m for m in n[::-1]), indexing="ij")[::-1]
+    p, q = X[(c + 1) % 3], X[(c + 2) % 3]
+    far = np.exp(-((p - np.pi) ** 2 + (q - np.pi) ** 2) / 0.25)
+    u = [None] * 3
+    u[(c + 1) % 3] = 0.3 * far * np.sin(3 * p + q)
+    u[(c + 2) % 3] = 0.2 * far * np.cos(2 * p)
+    u[c] = 0.4 * far * np.cos(p + 2 * q)
+    rho = unit * contrast ** (0.5 + 0.5 * np.cos(p + q)) * (1.0 + 0.1 * np.sin(q))
+    return n, W.conserved(rho, *u, 1.0 + 0.1 * np.cos(p), GAMMA, MACH)
+
+
+@pytest.mark.parametrize("order", [2, 6, 8])
+@pytest.mark.parametrize("contrast,unit", [(1.0, 1.0), (1e9, 1.0), (1.0, 1e-70), (1.0, 1e50), (1.0, 1e-100)])
+@pytest.mark.parametrize("c", [0, 1, 2])
+def test_quiet_regions(s2, c, contrast, unit, order):
+    """Mass and momentum along c, each point by the values around it."""
+    half = order // 2
+    n, w0 = jet(c, contrast, unit)
+    h = [L / m for m in n]
+    re = 50.0 / unit
+    with s2.Solver(*n, L, L, L, mach=MACH, re=re, weno_order=0, cfl=0.0, dt_fixed=1e-3, central_order=order,
+                   visc_order=order) as sv:
+        sv.set_state(w0)
+        got = sv.rhs()
+    rho, u, T = prims(w0)
+    mu = np.power(T, np.full(T.shape, LD(OMEGA))) / LD(re)
+    sa, sb = sum(abs(a) for a in A1[half]), abs(B2[half][0]) + 2 * sum(abs(b) for b in B2[half][1:])
+    want = [np.zeros_like(rho), np.zeros_like(rho)]
+    scale = [np.zeros_like(rho), np.zeros_like(rho)]
+    phi = u[c]
+    for d in range(3):
+        for l, a in enumerate(A1[half], 1):
+            m = a / 4 * (rho + shift(rho, d, l)) * (u[d] + shift(u[d], d, l))
+            b = shift(m, d, -l)
+            want[0] = want[0] - 2 * (m - b) / h[d]
+            want[1] = want[1] - (m * (phi + shift(phi, d, l)) - b * (phi + shift(phi, d, -l))) / h[d]
+        flux = 4 * sa * around(rho, d, half) * around(u[d], d, half) / h[d]
+        scale[0] += flux
+        scale[1] += flux * around(phi, d, half) + mu * sb * around(phi, d, half) / h[d] ** 2
+        want[1] = want[1] + mu * d2(phi, d, h[d], half) + OMEGA * mu / T * d1(T, d, h[d], half) * d1(phi, d, h[d], half)
+    err = [np.max(np.abs(got[f] - w) / s) for f, w, s in zip((0, 1 + c), want, scale)]
+    print("along %d, contrast %g, unit %g, order %d: errors %.2e %.2e" % (c, contrast, unit, order, *err))
+    assert max(err) < TOL
