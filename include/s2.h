@@ -259,8 +259,8 @@ int s2_set_tiles(s2_solver *s, const int *tiles);
  * persistent flux grid of direction d (0: as many as fit, up to 16; KEEP
  * in S2_FP64 has no persistent grid).
  * z_planes: z-planes each CTA of the mixed path's z-marching gradient and
- * viscous passes walks (0 or 12: chosen from the grid, between 1 and 24;
- * else 4, 8, 16 or 24, compiled variants).  weno_ctas_per_sm: cap of the
+ * viscous passes walks (0: chosen from the grid, between 1 and 24; else 4,
+ * 8, 12, 16 or 24).  s2_get_tuning returns what was set.  weno_ctas_per_sm: cap of the
  * WENO kernels' 64-thread CTAs per multiprocessor (0: 16; else 1..64).
  * Takes effect at the next s2_step; results do not depend on it, except
  * that with channel forcing in S2_MIXED the viscous pass sums the forcing

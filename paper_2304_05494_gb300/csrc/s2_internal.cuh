@@ -132,7 +132,7 @@ struct Dev {
   int flux_cps[3];         // persistent flux grids, per direction: resident CTAs per SM to use (0: all that fit)
   int zs;                  // planes per CTA of the z-marching passes (mixed path)
   int auto_shape;          // 1: tiles and planes left at their defaults are chosen from the grid
-  int zs_set;              // the same as asked for by the user (ZS_DEFAULT: chosen by z_auto_planes)
+  int zs_set;              // the same as asked for by the user (0: chosen by z_auto_planes)
   int weno_cps;            // WENO grids: CTAs per SM
   int nsm;                 // multiprocessors of the device
   unsigned long long wait_ns;  // limit of a kernel's wait for an asynchronous copy
@@ -783,6 +783,7 @@ void z_pass_grid(const Dev &d, unsigned g[3]);
 // and 24 (the forcing partials are sized for the smallest), and the choice
 // for boxes that share their launches.
 constexpr int ZS_MIN = 1, ZS_DEFAULT = 12;
+constexpr int FORCED_NSM = 152;  // see z_auto_planes
 int z_auto_planes(const Dev *d, int count);
 int fx_auto_tx(const Dev *d, int count);  // the same for the FP64 tiles
 // The tile variant of a direction for boxes that share their launches.

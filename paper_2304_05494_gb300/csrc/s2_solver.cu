@@ -1328,7 +1328,7 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.tile[1] = d.tile[2] = d.mixed;
   for (int a = 0; a < 3; ++a) d.flux_cps[a] = 0;
   d.auto_shape = 1;
-  d.zs_set = ZS_DEFAULT;
+  d.zs_set = 0;
   d.zs = z_auto_planes(&d, 1);
   d.fx_tx = fx_auto_tx(&d, 1);
   d.weno_cps = 16;
@@ -1735,8 +1735,8 @@ int s2_set_tuning(s2_solver *s, const s2_tuning *t) {
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) return S2_ECUDA;
   for (int a = 0; a < 3; ++a) s->d.tile[a] = t->tiles[a];
   for (int a = 0; a < 3; ++a) s->d.flux_cps[a] = t->flux_ctas_per_sm[a];
-  s->d.zs_set = t->z_planes ? t->z_planes : ZS_DEFAULT;
-  s->d.zs = s->d.zs_set == ZS_DEFAULT ? z_auto_planes(&s->d, 1) : s->d.zs_set;
+  s->d.zs_set = t->z_planes;
+  s->d.zs = t->z_planes ? t->z_planes : z_auto_planes(&s->d, 1);
   s->d.weno_cps = t->weno_ctas_per_sm ? t->weno_ctas_per_sm : 16;
   if (s->graph_ready) {
     cudaGraphExecDestroy(s->graph);
@@ -1975,7 +1975,7 @@ int group_setup(BatchGroup &g) {
   // launch shapes for all boxes of the group together
   int tile[3];
   for (int dir = 0; dir < 3; ++dir) tile[dir] = flux_auto_tile(devs.data(), n, dir);
-  const int zs = devs[0].zs_set != ZS_DEFAULT || devs[0].force ? devs[0].zs : z_auto_planes(devs.data(), n);
+  const int zs = devs[0].zs_set || devs[0].force ? devs[0].zs : z_auto_planes(devs.data(), n);
   const int tx = fx_auto_tx(devs.data(), n);
   for (Dev &d : devs) {
     d.fx_tx = tx;
@@ -2170,7 +2170,7 @@ cudaError_t enqueue_member(s2_solver *s, int zs, double share, int mode, Trace *
   Dev &d = s->d;
   const int own_zs = d.zs, own_tx = d.fx_tx, own_cps = d.weno_cps;
   const bool plain = mode == S2_BATCH_BRANCHES;
-  if (d.zs_set == ZS_DEFAULT && !d.force) d.zs = plain ? ZS_DEFAULT : zs;
+  if (!d.zs_set && !d.force) d.zs = plain ? ZS_DEFAULT : zs;
   if (plain) {
     d.auto_shape = 0;
     d.fx_tx = 32;

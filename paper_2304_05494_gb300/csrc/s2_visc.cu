@@ -1104,7 +1104,9 @@ int fx_auto_tx(const Dev *d, int count) {
 // with the least (CTAs over those places, rounded up) x (zs + 2).  Small
 // boxes get few planes per CTA, so that there are CTAs for every
 // multiprocessor (37 x 29 x 19: one plane, 152 CTAs instead of 16), large
-// ones many.
+// ones many.  A forced box sums its body force by plane groups: it is counted
+// on the multiprocessors of a GB300, so that its results depend on the grid
+// alone.
 int z_auto_planes(const Dev *d, int count) {
   int best = ZS_DEFAULT;
   long long cost = -1;
@@ -1112,7 +1114,7 @@ int z_auto_planes(const Dev *d, int count) {
     long long ctas = 0;
     for (int b = 0; b < count; ++b)
       ctas += (long long)((d[b].nx + ZTX - 1) / ZTX) * ((d[b].ny + ZTY - 1) / ZTY) * ((d[b].nz + zs - 1) / zs);
-    const long long places = 2ll * d[0].nsm, c = (ctas + places - 1) / places * (zs + 2);
+    const long long places = 2ll * (d[0].force ? FORCED_NSM : d[0].nsm), c = (ctas + places - 1) / places * (zs + 2);
     if (cost < 0 || c < cost) {
       cost = c;
       best = zs;

@@ -42,3 +42,22 @@ def test_split_form_and_keep_boxes_in_one_batch(s2, precision, mode, keeps):
         sv.close()
     for k, g, w in zip(keeps, got, want):
         assert np.array_equal(g, w), k
+
+
+def test_twelve_planes_are_what_is_asked_for(s2):
+    """z_planes = 12 is a choice of its own, not the default: a forced channel
+    of 12 planes sums its body force in one group with 12, 16 or 24 planes
+    per CTA, and in several by default."""
+    c = W.channel(40, 36, 12, seed=2)
+    out = {}
+    for z in (0, 12, 16, 24):
+        with s2.Solver.from_case(c, cfl=0.8, threshold=0.05, precision="mixed") as sv:
+            assert sv.get_tuning()["z_planes"] == 0
+            sv.set_tuning(z_planes=z)
+            sv.set_tuning(flux_ctas_per_sm=2)  # (leaves the others as they are)
+            assert sv.get_tuning()["z_planes"] == z
+            sv.set_state(c.w0)
+            sv.step(3)
+            out[z] = sv.get_state()
+    assert np.array_equal(out[12], out[16]) and np.array_equal(out[12], out[24])
+    assert not np.array_equal(out[12], out[0])
