@@ -351,7 +351,7 @@ void s2_destroy(s2_solver *s);
  * S2_BATCH_MIN_GROUP members save too few launches: those keep their own
  * launch sequence (S2_BATCH_WORKLIST_ALL puts every member in a group).  Groups and such members run as concurrent branches of the
  * step graph.  Branch mode (S2_BATCH_BRANCHES): every member's own
- * launch sequence is a concurrent branch.  Either way each box's
+ * launch sequence, in the shapes of its solo run, is a concurrent branch.  Either way each box's
  * arithmetic is exactly that of its solo run (results identical bit for
  * bit), members keep their own state, parameters, streams and clocks, and
  * no buffer is shared.

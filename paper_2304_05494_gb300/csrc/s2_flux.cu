@@ -1243,7 +1243,7 @@ static int auto_tile_dir(const Dev *d, int count, int dir) {
 }
 
 int flux_auto_tile(const Dev *d, int count, int dir) {
-  if (d->tile[dir] || d->keep || !d->auto_shape) return d->tile[dir];
+  if (d->tile[dir] || d->keep) return d->tile[dir];
   return d->mixed ? auto_tile_dir<float>(d, count, dir) : auto_tile_dir<double>(d, count, dir);
 }
 

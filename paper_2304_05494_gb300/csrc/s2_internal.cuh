@@ -131,7 +131,6 @@ struct Dev {
   int tile[3];             // flux tile variant per direction (0 default, 1 narrow; 2 narrowest, by flux_auto_tile only)
   int flux_cps[3];         // persistent flux grids, per direction: resident CTAs per SM to use (0: all that fit)
   int zs;                  // planes per CTA of the z-marching passes (mixed path)
-  int auto_shape;          // 1: tiles and planes left at their defaults are chosen from the grid
   int zs_set;              // the same as asked for by the user (0: chosen by z_auto_planes)
   int weno_cps;            // WENO grids: CTAs per SM
   int nsm;                 // multiprocessors of the device

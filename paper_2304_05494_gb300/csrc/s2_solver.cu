@@ -919,7 +919,7 @@ cudaError_t run(Trace *tr, cudaStream_t st, int kind, int nkernels, F f) {
 // first: nothing was launched on the stream by this sequence yet.
 cudaError_t enqueue_rhs(s2_solver *s, int stage0, Trace *tr, bool first) {
   const Dev &d = s->d;
-  const bool pdl = !(tr && tr->timed) && d.auto_shape;
+  const bool pdl = !(tr && tr->timed);
   Lane st{s->stream, pdl && !first};
   cudaError_t e;
   unsigned nb = (unsigned)((d.n + NT - 1) / NT);
@@ -980,14 +980,8 @@ cudaError_t enqueue_rhs(s2_solver *s, int stage0, Trace *tr, bool first) {
     if ((e = cudaStreamWaitEvent(st.st, s->ev_join, 0)) != cudaSuccess) return e;
     st.pdl = false;  // the next kernel waits for the side stream too
   } else if (d.weno) {
-    // one launch for the three directions (not in branch mode, see
-    // enqueue_member)
-    e = run(tr, st.st, S2_PROF_WENO, d.auto_shape ? 1 : 3, [&] {
-      if (d.auto_shape) return launch_weno(d, -1, st);
-      cudaError_t r = cudaSuccess;
-      for (int dir = 0; dir < 3 && r == cudaSuccess; ++dir) r = launch_weno(d, dir, st);
-      return r;
-    });
+    // one launch for the three directions
+    e = run(tr, st.st, S2_PROF_WENO, 1, [&] { return launch_weno(d, -1, st); });
     if (e != cudaSuccess) return e;
   }
   if (d.viscous) {
@@ -1019,7 +1013,7 @@ cudaError_t enqueue_step(s2_solver *s, Trace *tr) {
   const Dev &d = s->d;
   unsigned nb = (unsigned)((d.n + NT - 1) / NT);
   cudaError_t e;
-  const Lane st{s->stream, !(tr && tr->timed) && d.auto_shape};
+  const Lane st{s->stream, !(tr && tr->timed)};
   for (int stage = 0; stage < 3; ++stage) {
     if ((e = enqueue_rhs(s, stage == 0, tr, stage == 0)) != cudaSuccess) return e;
     e = run(tr, s->stream, S2_PROF_UPDATE, 1, [&] {
@@ -1327,7 +1321,6 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.tile[0] = 0;
   d.tile[1] = d.tile[2] = d.mixed;
   for (int a = 0; a < 3; ++a) d.flux_cps[a] = 0;
-  d.auto_shape = 1;
   d.zs_set = 0;
   d.zs = z_auto_planes(&d, 1);
   d.fx_tx = fx_auto_tx(&d, 1);
@@ -2157,31 +2150,22 @@ cudaError_t enqueue_group_step(BatchGroup &g) {
 }
 
 // One step of a member on its own launches, beside the other branches of
-// the batch: its z-planes are chosen for all of them together (the chip is
-// shared, so CTAs of more planes, which load their column queues less often,
-// pay; boxes of 32^3 .. 128^3 took 1.248 ms per step with the planes of the
-// boxes alone, 1.225 with 24, 1.214 with 16, the most that is taken: more
-// make the largest box's chain long), and it gets its share, by points, of
-// the WENO CTAs of one box (1.240 -> 1.204 ms where nothing is flagged).  Forced members
-// keep their planes (they sum the forcing by plane groups).
-// In branch mode, kept to compare the work list with, members keep the
-// default shapes and the plain launches of large boxes.
-cudaError_t enqueue_member(s2_solver *s, int zs, double share, int mode, Trace *tr) {
+// the batch: it gets its share, by points, of the WENO CTAs of one box (boxes
+// of 32^3 .. 128^3, mixed: 1.240 -> 1.204 ms per step where nothing is
+// flagged).  zs: beside a work list, z-planes chosen for all the members
+// together (the chip is shared, so CTAs of more planes, which load their
+// column queues less often, pay; the same boxes took 1.248 ms per step with
+// the planes of the boxes alone, 1.225 with 24, 1.214 with 16, the most that
+// is taken: more make the largest box's chain long); 0: the member's own.
+// Forced members keep their planes (they sum the forcing by plane groups).
+cudaError_t enqueue_member(s2_solver *s, int zs, double share, Trace *tr) {
   Dev &d = s->d;
-  const int own_zs = d.zs, own_tx = d.fx_tx, own_cps = d.weno_cps;
-  const bool plain = mode == S2_BATCH_BRANCHES;
-  if (!d.zs_set && !d.force) d.zs = plain ? ZS_DEFAULT : zs;
-  if (plain) {
-    d.auto_shape = 0;
-    d.fx_tx = 32;
-  } else {
-    d.weno_cps = (int)(own_cps * share) + 1;
-  }
+  const int own_zs = d.zs, own_cps = d.weno_cps;
+  if (zs && !d.zs_set && !d.force) d.zs = zs;
+  d.weno_cps = (int)(own_cps * share) + 1;
   const cudaError_t e = enqueue_step(s, tr);
   d.zs = own_zs;
-  d.fx_tx = own_tx;
   d.weno_cps = own_cps;
-  d.auto_shape = 1;
   return e;
 }
 
@@ -2210,7 +2194,7 @@ int batch_build(s2_batch *b) {
       s2_solver *s = b->members[m];
       e = cudaStreamWaitEvent(s->stream, b->events[0], 0);
       Trace tr;
-      if (e == cudaSuccess) e = enqueue_member(s, zs, s->d.n / points, b->mode, &tr);
+      if (e == cudaSuccess) e = enqueue_member(s, 0, s->d.n / points, &tr);
       total_launches += total(tr);
       b->member_launches[m] = total(tr);
       if (e == cudaSuccess) e = cudaEventRecord(b->events[1 + m], s->stream);
@@ -2233,7 +2217,7 @@ int batch_build(s2_batch *b) {
       s2_solver *s = b->solo[k];
       e = cudaStreamWaitEvent(s->stream, b->events[0], 0);
       Trace tr;
-      if (e == cudaSuccess) e = enqueue_member(s, zs, s->d.n / points, b->mode, &tr);
+      if (e == cudaSuccess) e = enqueue_member(s, zs, s->d.n / points, &tr);
       total_launches += total(tr);
       for (size_t m = 0; m < b->members.size(); ++m)
         if (b->members[m] == s) b->member_launches[m] = total(tr);

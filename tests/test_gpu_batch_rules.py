@@ -61,3 +61,18 @@ def test_twelve_planes_are_what_is_asked_for(s2):
             out[z] = sv.get_state()
     assert np.array_equal(out[12], out[16]) and np.array_equal(out[12], out[24])
     assert not np.array_equal(out[12], out[0])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_branch_mode_runs_the_solo_launches(s2, precision):
+    """A member of a branch-mode batch has the launches of its solo step."""
+    c = W.taylor_green(24, mach=0.3, seed=5)
+    c.weno_order = 5
+    with s2.Solver.from_case(c, precision=precision, threshold=0.2, cfl=0.0, dt_fixed=1e-3) as sv:
+        sv.set_state(c.w0)
+        sv.step(1)
+        before = sv.stats()["launches"]
+        sv.step(1)
+        solo = sv.stats()["launches"] - before
+        with s2.Batch([sv], mode="branches") as b:
+            assert b.launches_per_step == solo
