@@ -260,8 +260,10 @@ int s2_set_tiles(s2_solver *s, const int *tiles);
  * in S2_FP64 has no persistent grid).
  * z_planes: z-planes each CTA of the mixed path's z-marching gradient and
  * viscous passes walks (0: chosen from the grid, between 1 and 24; else 4,
- * 8, 12, 16 or 24).  s2_get_tuning returns what was set.  weno_ctas_per_sm: cap of the
- * WENO kernels' 64-thread CTAs per multiprocessor (0: 16; else 1..64).
+ * 8, 12, 16 or 24).  s2_get_tuning returns what was set.  weno_ctas_per_sm: cap of a
+ * WENO launch's 64-thread CTAs per multiprocessor (0: 16 for a launch of one
+ * direction, 24 for a launch of all three, of which each gets a third and at
+ * least one; else 1..64).
  * Takes effect at the next s2_step; results do not depend on it, except
  * that with channel forcing in S2_MIXED the viscous pass sums the forcing
  * per CTA, so z_planes changes the order of that sum (single-precision

@@ -46,14 +46,19 @@ constexpr int WENO_NT = 64;  // threads per CTA of the WENO kernels
 
 // CTAs of a direction's WENO corrections: small, so that the flagged
 // interfaces (a count known on the device only, often a few per cent of the
-// slots) spread evenly over the multiprocessors; at most weno_cps on each,
-// or half as many per direction in a launch of all three.  (Isotropic 256^3,
-// 19 % flagged, ms per step for 16 / 24 / 48 per multiprocessor over the
-// three: 3.51 / 2.79 / 2.96; 24 is three times what is resident.)
+// slots) spread evenly over the multiprocessors.  A launch has at most
+// weno_cps on each, all (a launch of all three directions) a third of them for
+// each direction; by default 16, all 24.  (Isotropic 256^3, 19 % flagged, ms
+// per step for 16 / 24 / 48 per multiprocessor over the three: 3.51 / 2.79 /
+// 2.96; 24 is three times what is resident.)
+int weno_per_sm(const Dev &d, bool all) {
+  const int cps = d.weno_cps > 0 ? d.weno_cps : (all ? 24 : 16);
+  return all ? (cps < 3 ? 1 : cps / 3) : cps;
+}
+
 unsigned weno_blocks(const Dev &d, int dir, bool all) {
   const long long need = (d.nslot[dir] + WENO_NT - 1) / WENO_NT;
-  const int cps = d.weno_cps > 0 ? d.weno_cps : 16;
-  const long long cap = (long long)(all ? (cps + 1) / 2 : cps) * d.nsm;
+  const long long cap = (long long)weno_per_sm(d, all) * d.nsm;
   return (unsigned)(need < 1 ? 1 : (need < cap ? need : cap));
 }
 

@@ -132,7 +132,7 @@ struct Dev {
   int flux_cps[3];         // persistent flux grids, per direction: resident CTAs per SM to use (0: all that fit)
   int zs;                  // planes per CTA of the z-marching passes (mixed path)
   int zs_set;              // the same as asked for by the user (0: chosen by z_auto_planes)
-  int weno_cps;            // WENO grids: CTAs per SM
+  int weno_cps;            // WENO launches: largest number of CTAs per SM (0: weno_per_sm's)
   int nsm;                 // multiprocessors of the device
   unsigned long long wait_ns;  // limit of a kernel's wait for an asynchronous copy
   unsigned tx_extra;       // bytes a staging barrier expects beyond its copies (0; test hook)
@@ -773,6 +773,7 @@ struct FluxBoxPlan {
   bool persistent;  // CTAs walk several tiles
 };
 cudaError_t flux_batch_plan(const Dev &d, int dir, FluxBoxPlan *out);
+int weno_per_sm(const Dev &d, bool all);  // all: per direction, of a launch of all three
 unsigned weno_blocks(const Dev &d, int dir, bool all);
 cudaError_t launch_flux_batch(const Dev &d0, const BatchArgs &ba, unsigned total, const FluxMaps *maps,
                               const void *tgs, int dir, int accumulate, const Lane &st);

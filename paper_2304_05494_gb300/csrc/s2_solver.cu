@@ -1324,7 +1324,7 @@ int s2_create(const s2_grid *grid, const s2_metrics *metrics, const s2_gas *gas,
   d.zs_set = 0;
   d.zs = z_auto_planes(&d, 1);
   d.fx_tx = fx_auto_tx(&d, 1);
-  d.weno_cps = 16;
+  d.weno_cps = 0;
   // scheme constants in both arithmetic types
   {
     Consts<double> &k = d.kd;
@@ -1730,7 +1730,7 @@ int s2_set_tuning(s2_solver *s, const s2_tuning *t) {
   for (int a = 0; a < 3; ++a) s->d.flux_cps[a] = t->flux_ctas_per_sm[a];
   s->d.zs_set = t->z_planes;
   s->d.zs = t->z_planes ? t->z_planes : z_auto_planes(&s->d, 1);
-  s->d.weno_cps = t->weno_ctas_per_sm ? t->weno_ctas_per_sm : 16;
+  s->d.weno_cps = t->weno_ctas_per_sm;
   if (s->graph_ready) {
     cudaGraphExecDestroy(s->graph);
     s->graph_ready = false;
@@ -2020,7 +2020,7 @@ int group_setup(BatchGroup &g) {
       set(BC_FLUX0 + dir, b, c, 1, 1);
       // WENO: the solo launch's CTAs shared out by interface slots
       const unsigned solo = weno_blocks(d, dir, true);
-      const unsigned w = (unsigned)(8.0 * d.nsm * (double)d.nslot[dir] / (double)slots_sum[dir]) + 1;
+      const unsigned w = (unsigned)((double)weno_per_sm(d, true) * d.nsm * (double)d.nslot[dir] / (double)slots_sum[dir]) + 1;
       if ((w < solo ? w : solo) > nweno) nweno = w < solo ? w : solo;
     }
     set(BC_WENO, b, nweno, 3, 1);
@@ -2162,7 +2162,8 @@ cudaError_t enqueue_member(s2_solver *s, int zs, double share, Trace *tr) {
   Dev &d = s->d;
   const int own_zs = d.zs, own_cps = d.weno_cps;
   if (zs && !d.zs_set && !d.force) d.zs = zs;
-  d.weno_cps = (int)(own_cps * share) + 1;
+  // (mixed: one launch for three directions)
+  d.weno_cps = (int)((own_cps ? own_cps : (d.mixed ? 24 : 16)) * share) + (d.mixed ? 2 : 1);
   const cudaError_t e = enqueue_step(s, tr);
   d.zs = own_zs;
   d.weno_cps = own_cps;

@@ -52,7 +52,7 @@ def test_twelve_planes_are_what_is_asked_for(s2):
     out = {}
     for z in (0, 12, 16, 24):
         with s2.Solver.from_case(c, cfl=0.8, threshold=0.05, precision="mixed") as sv:
-            assert sv.get_tuning()["z_planes"] == 0
+            assert sv.get_tuning()["z_planes"] == 0 and sv.get_tuning()["weno_ctas_per_sm"] == 0
             sv.set_tuning(z_planes=z)
             sv.set_tuning(flux_ctas_per_sm=2)  # (leaves the others as they are)
             assert sv.get_tuning()["z_planes"] == z
