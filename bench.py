@@ -63,26 +63,29 @@ ALG_FLOPS_FLUX_DIFFERENCE = 47.0 / 3  # flux difference per point and direction
 # Double-precision issue peak of the FP64 unit: 152 SMs x 2 DFMA per clock
 # (4 flop) at the 2070 MHz maximum SM clock.
 FP64_PEAK_GFLOPS = 152 * 4 * 2.070
+# (The stencil sums run on the integer unit, so that rates above this peak
+# are no share of it; profiles/channel256x128x128_fp64_kernels_full.md has how
+# busy both units are.)
 # DRAM bytes per interior point of one launch of the FP64 viscous kernel
 # (ncu dram__bytes_read.sum + dram__bytes_write.sum, 256 x 128 x 128
-# channel, scaled by the points of a launch; profiles/channel256x128x128_fp64_visc_full.md).
-FP64_DRAM_BYTES = {"visc": 207.8}
+# channel, scaled by the points of a launch; the same file).
+FP64_DRAM_BYTES = {"visc": 192.8}
 # Mixed path: algorithmic HBM bytes per interior point of one launch
 # (single-precision primitives and RHS, double-precision state; each field
 # read or written once, halos not counted):
 #   prims  w (40) -> rho, u, v, w, T, p, H, mu (32)
 #   grad   u, v, w (12) -> div u, sensor test (8)
 #   flux   rho, u, v, w, H, p, sensor (28) + RHS write (20), y and z also read it (20)
-#   visc   u, v, w, T, div u, mu (24) + RHS read and write (40)
+#   visc   u, v, w, T, div u, mu (24) + RHS of momentum and energy read and
+#          write (32; the density's only where an interface is flagged)
 #   update w read/write (80), RHS (20), RK register read and write on 2 of 3 stages (26.7), u (4)
-MIXED_BYTES = {"prims": 72, "grad": 20, "flux_x": 48, "flux_y": 68, "flux_z": 68, "visc": 64, "update": 130.7}
+MIXED_BYTES = {"prims": 72, "grad": 20, "flux_x": 48, "flux_y": 68, "flux_z": 68, "visc": 56, "update": 130.7}
 # The method's algorithmic traffic per point and RK3 step: per stage read
 # and write the state and the RK register, 4 x 40 B.
 METHOD_BYTES_PER_POINT_STEP = 480.0
 # DRAM bytes per interior point of one launch of the mixed kernels (ncu,
-# 256 x 128 x 128 channel, first stage; profiles/channel256x128x128_mixed_kernels_full.md,
-# the viscous pass profiles/channel1024x256x512_launch_list.md).
-MIXED_DRAM_BYTES = {"prims": 63.9, "visc": 65.5, "update": 110.1}
+# 256 x 128 x 128 channel; profiles/channel256x128x128_mixed_kernels_full.md).
+MIXED_DRAM_BYTES = {"prims": 63.6, "visc": 55.5, "update": 110.1}
 # Thermally perfect gas of the side measurement: a synthetic polynomial of
 # the NASA 9-coefficient form, c_p/R = sum_{l=-2..4} a_l T^l (reference
 # units of T), whose gamma falls from 1.45 at T = 0.5 through 1.40 at T = 1
@@ -338,10 +341,13 @@ def per_launch(prof, name):
 
 
 def fp64_roofline(case, prof, steps, weno_frac, step_ms, fma_gflops):
-    """FP64 path: bound by the double-precision unit.  achieved = the
+    """FP64 path: bound by arithmetic, the double-precision unit's and the
+    integer unit's, which forms the stencil sums.  achieved = the
     oracle-tallied flops of the dominant kernel class per launch / its mean
     launch time (CUDA events on the solver's stream); the whole step's
-    tallied flops / step time beside it."""
+    tallied flops / step time beside it.  The peak is that of the
+    double-precision unit alone: a frac above 1 says how much faster the
+    method's operations are than on that unit."""
     n = case.points
     flux_pp = {d: ALG_FLOPS_CENTRAL_INTERFACE * (nd + 1) / nd + ALG_FLOPS_FLUX_DIFFERENCE
                for d, nd in (("flux_x", case.nx), ("flux_y", case.ny), ("flux_z", case.nz))}
@@ -364,8 +370,8 @@ def fp64_roofline(case, prof, steps, weno_frac, step_ms, fma_gflops):
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
             "frac": achieved / FP64_PEAK_GFLOPS, "traffic": traffic * n if traffic else None, "kernel": name,
             "per_launch_ms": pl,
-            "peak_source": "152 SM x 2 DFMA/clk x 2070 MHz (FP64 unit issue rate); FMA loop measured live: "
-                           "%.0f GFLOP/s" % fma_gflops,
+            "peak_source": "152 SM x 2 DFMA/clk x 2070 MHz (FP64 unit issue rate; the stencil sums run on the "
+                           "integer unit, so frac may exceed 1); FMA loop measured live: %.0f GFLOP/s" % fma_gflops,
             "frac_of_fma_measured": achieved / fma_gflops,
             "flops_source": "oracle operation tally (oracle/tally.py)",
             "step_frac": step_flops / (step_ms * 1e-3) / 1e9 / FP64_PEAK_GFLOPS,

@@ -2157,6 +2157,11 @@ cudaError_t enqueue_group_step(BatchGroup &g) {
 // column queues less often, pay; the same boxes took 1.248 ms per step with
 // the planes of the boxes alone, 1.225 with 24, 1.214 with 16, the most that
 // is taken: more make the largest box's chain long); 0: the member's own.
+// Other mixes agree: up to 24 planes, boxes of 64^3, 96^3 and 128^3 with 19 %
+// of their interfaces flagged took 1.925 for 1.867 ms, two of 96^3 and two of
+// 128^3, three of 64^3 .. 112^3, 160^3 with 64^3, and two flagged of 128^3 the
+// same within 0.3 %; without the share of the WENO CTAs these five took 0.5
+// to 2.4 % more.
 // Forced members keep their planes (they sum the forcing by plane groups).
 cudaError_t enqueue_member(s2_solver *s, int zs, double share, Trace *tr) {
   Dev &d = s->d;
