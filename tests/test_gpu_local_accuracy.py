@@ -136,3 +136,32 @@ def test_quiet_regions(s2, c, contrast, unit, order):
     err = [np.max(np.abs(got[f] - w) / s) for f, w, s in zip((0, 1 + c), want, scale)]
     print("along %d, contrast %g, unit %g, order %d: errors %.2e %.2e" % (c, contrast, unit, order, *err))
     assert max(err) < TOL
+
+
+def test_quiet_regions_do_not_depend_on_tiles(s2):
+    """Which stencils are quiet follows from the fields alone: a jet's steps
+    are the same bit for bit with other tiles and in a batch."""
+    out = []
+    for c in (0, 2):
+        n, w0 = jet(c, 30.0, 1.0)
+        kw = dict(mach=MACH, re=50.0, weno_order=5, threshold=0.05, cfl=0.5, dt_every=1)
+        got = []
+        for tiles in ([0, 0, 0], [1, 1, 1]):
+            with s2.Solver(*n, L, L, L, **kw) as sv:
+                sv.set_tiles(tiles)
+                sv.set_state(w0)
+                sv.step(3)
+                got.append(sv.get_state())
+        out.append((n, w0, kw, got[0]))
+        assert np.array_equal(got[0], got[1])
+    solvers = [s2.Solver(*n, L, L, L, **kw) for n, _, kw, _ in out]
+    for sv, (_, w0, _, _) in zip(solvers, out):
+        sv.set_state(w0)
+    with s2.Batch(solvers, mode="worklist_all") as b:
+        b.step(3)
+        b.sync()
+    states = [sv.get_state() for sv in solvers]
+    for sv in solvers:
+        sv.close()
+    for w, (_, _, _, want) in zip(states, out):
+        assert np.array_equal(w, want)
