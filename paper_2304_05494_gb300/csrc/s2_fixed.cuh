@@ -4,8 +4,8 @@
 // and 64 integer ones (measured per warp instruction and scheduler: 64.5
 // clocks for a DFMA, 5 for a 32 x 32 + 64 bit multiply-add, 2 for an
 // integer add; the two kinds overlap).  The linear and bilinear parts of
-// the right-hand side therefore run on the integer unit, in 59-bit fixed
-// point, which carries more bits than the 53 of a double.
+// the right-hand side therefore run on the integer unit, in fixed point of 59
+// or 62 bits, more than the 53 of a double.
 //
 // A value is held as an integer F, cut towards zero, for an exponent E with
 // |f| < 2^E: f 2^(59-E) in two limbs F = hi 2^30 + lo with the sign of f on

@@ -533,7 +533,7 @@ __device__ __forceinline__ void grad_fx_body(const Dev &__restrict__ d, const Bl
 // tensor tau and psi = (omega / T) grad T, each term is mu times
 //   X_a = lap u_a + d_a theta / 3 + psi_b tau_ab / mu   (momentum a)
 //   u_a X_a + tau_ab d_b u_a / mu + (c_p / Pr) (lap T + psi . grad T)
-// so mu enters with the sum into the RHS: about 55 double operations per
+// so mu enters with the sum into the RHS: about 67 double operations per
 // point at order 6 (169 when the stencils were in double precision too).
 // Each direction of a Laplacian becomes a double by itself and is weighted
 // there: in one integer sum of all three, the weights and the sum's last
