@@ -104,10 +104,9 @@ __device__ __forceinline__ int2 fx_split(double x, int ex) {
 __device__ __forceinline__ int fx_mag(double x) { return __double2hiint(x) & 0x7fffffff; }
 __device__ __forceinline__ int fx_own_exponent(int mag) { return max(mag >> 20, FX_EMIN); }
 
-// The high part of a product of limb pairs, (a b) / 2^60 up to the dropped
-// lo lo product: hh + hl / 2^30.
-__device__ __forceinline__ long long fx_mulhi(int al, int ah, int bl, int bh) {
-  const long long hl = (long long)ah * bl + (long long)al * bh;
+// A product of limb pairs / 2^60.
+__device__ __forceinline__ long long fx_mul(int al, int ah, int bl, int bh) {
+  const long long hl = (long long)ah * bl + (long long)al * bh + (((long long)al * bl) >> FX_LIMB);
   return (long long)ah * bh + (hl >> FX_LIMB);
 }
 

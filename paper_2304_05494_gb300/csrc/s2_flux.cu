@@ -221,9 +221,9 @@ __device__ __forceinline__ void keep_pairs_tile(const R *S, R *TP, R gm1, int n)
 // the double unit executed 61 operations (64 issue clocks each); here it
 // executes 12 (the pressure difference and the sums into the RHS), the
 // integer unit the rest beside them.  On 420 x 250 x 320 points a launch
-// takes 1.66 / 1.76 / 1.72 ms (x / y / z) instead of 3.85 / 3.70 / 3.64; of
+// takes 1.94 / 2.05 / 1.99 ms (x / y / z) instead of 3.85 / 3.70 / 3.64; of
 // these, quiet stencils (a third of v's and w's in that channel) and looking
-// for them cost 0.4 to 0.5 (1.28 / 1.25 / 1.27 with the grid's exponents for
+// for them cost 0.4 to 0.5, the lo lo products 0.25 (1.28 / 1.25 / 1.27 with the grid's exponents for
 // every stencil, which loses the digits of quiet regions).
 // With the double unit no longer the bound, the persistent grid that
 // prefetches the next tile pays here too: with one tile per CTA the same
@@ -257,11 +257,11 @@ __device__ __forceinline__ constexpr int2 acoef_limbs(int l) {
 }
 
 // Pair mass fluxes m_l(a), a = -NP .. L-1, in units of 2^(E_rho + E_n - 59).
-// (rho_a + rho_b)(un_a + un_b) is formed to 2^-60 of its largest value, and
-// so is its product with a_l / 4.
+// (rho_a + rho_b)(un_a + un_b) is formed to 2^-60 of its exponents' power of
+// two, and so is its product with a_l / 4.
 __device__ __forceinline__ int2 fx_pair(int2 r0, int2 r1, int2 n0, int2 n1, int2 k) {
-  const long long P = fx_mulhi(r0.x + r1.x, r0.y + r1.y, n0.x + n1.x, n0.y + n1.y);
-  const long long m = fx_mulhi((int)P & FX_MASK, (int)(P >> FX_LIMB), k.x, k.y);
+  const long long P = fx_mul(r0.x + r1.x, r0.y + r1.y, n0.x + n1.x, n0.y + n1.y);
+  const long long m = fx_mul((int)P & FX_MASK, (int)(P >> FX_LIMB), k.x, k.y);
   return make_int2((int)m & FX_MASK, (int)(m >> FX_LIMB));
 }
 
@@ -309,10 +309,13 @@ __device__ __forceinline__ int fx_own(const double *f, long long p, long long st
 }
 
 // The flux difference of one point: D_rho = 2 M, D_phi = phi_a M + sum_l
-// [m_l(a) phi_{a+l} - m_l(a-l) phi_{a-l}], each product to 2^-60 of its
-// largest value: A collects the hi hi products, B the mixed ones.  |m| is
-// below 2^59 sum |a_l| and the lo limbs of m are not negative, so with 8
-// pairs (order 8) |B| stays below 2^59 (8 + 2.1 + 1 + 2.1) < 2^63.
+// [m_l(a) phi_{a+l} - m_l(a-l) phi_{a-l}]: A collects the hi hi products, B
+// the mixed ones, C the lo lo ones (without them, and the sum rounded to whole
+// units, operands all near their loud bounds would have 40 times a double's
+// error; they cost 0.25 ms per launch of 420 x 250 x 320 points).  |m| is below
+// 2^59 sum |a_l| and the lo limbs of m are not negative, so with 8 pairs (order
+// 8) |B| stays below 2^59 (8 + 2.1 + 1 + 2.1) < 2^63, and |C| below 8 times
+// (2^30 - 1)^2 < 2^63.
 // The field values of a quiet stencil (s2_fixed.cuh) come from memory with
 // their own exponent; p: the point's padded offset.
 template <int DIR, int NP, int ST, int SA, int SFA>
@@ -360,18 +363,16 @@ __device__ __forceinline__ void fx_flux_point(const Dev &__restrict__ d, const i
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
     const int f = g == 0 ? F_U + DIR : (g <= DIR ? g : g + 1);
-    int ef = en;
+    int ef = en, any = 0;  // bits of the values' hi limbs
     if (g > 0) {
       const int2 *Sf = S + f * SFA;  // F_U .. F_H follow F_RHO
       ef = e[f];
-      unsigned any = 0;  // bits from 2 loud on: a value outside -loud .. loud
 #pragma unroll
-      for (int l = 0; l <= 2 * NP; ++l) {
-        v[l] = Sf[ap + (l - NP) * SA];
-        any |= (unsigned)(v[l].y + loud[f]);
-      }
-      if (any < 2u * (unsigned)loud[f]) ef = fx_own<NP>(src[f], p, stride, v);
+      for (int l = 0; l <= 2 * NP; ++l) v[l] = Sf[ap + (l - NP) * SA];
     }
+#pragma unroll
+    for (int l = 0; l <= 2 * NP; ++l) any |= v[l].y ^ (v[l].y >> 31);
+    if (g > 0 && any < loud[f]) ef = fx_own<NP>(src[f], p, stride, v);
     long long A = (long long)Mh * v[NP].y;
     long long B = (long long)Mh * v[NP].x + (long long)Ml * v[NP].y;
 #pragma unroll
@@ -384,9 +385,22 @@ __device__ __forceinline__ void fx_flux_point(const Dev &__restrict__ d, const i
       B += (long long)mm[l - 1].y * vm.x;
       B += (long long)mm[l - 1].x * vm.y;
     }
-    const double D = fx_i2d(A + (B >> FX_LIMB));
-    // unit of D: 2^60 times the units of m and phi
-    const int eD = eM + ef - 1022 + 1;
+    B += (long long)Ml * v[NP].x >> FX_LIMB;
+    long long C = 0;
+#pragma unroll
+    for (int l = 1; l <= NP; ++l) {
+      C += (long long)mp[l - 1].x * v[NP + l].x;
+      C += (long long)mm[l - 1].x * v[NP - l].x;
+    }
+    B += C >> FX_LIMB;
+    // unit of D: 2^60 times the units of m and phi, 2^-30 of it for small sums
+    int eD = eM + ef - 1022 + 1;
+    A += B >> FX_LIMB;
+    if ((unsigned long long)(A + (1ll << 32)) >> 33 == 0) {
+      A = A * (1ll << FX_LIMB) + (B & FX_MASK);
+      eD -= FX_LIMB;
+    }
+    const double D = fx_i2d(A);
     double r = fma(-fx_ldexp(scale, eD), D, prev[f]);
     if (f == 1 + DIR) r = fma(-scale, dp, r);
     out[f * d.n] = r;
