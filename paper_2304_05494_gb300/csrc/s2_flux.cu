@@ -221,10 +221,10 @@ __device__ __forceinline__ void keep_pairs_tile(const R *S, R *TP, R gm1, int n)
 // the double unit executed 61 operations (64 issue clocks each); here it
 // executes 12 (the pressure difference and the sums into the RHS), the
 // integer unit the rest beside them.  On 420 x 250 x 320 points a launch
-// takes 1.94 / 2.05 / 1.99 ms (x / y / z) instead of 3.85 / 3.70 / 3.64; of
+// takes 1.98 / 2.10 / 2.05 ms (x / y / z) instead of 3.85 / 3.70 / 3.64; of
 // these, quiet stencils (a third of v's and w's in that channel) and looking
-// for them cost 0.4 to 0.5, the lo lo products 0.25 (1.28 / 1.25 / 1.27 with the grid's exponents for
-// every stencil, which loses the digits of quiet regions).
+// for them cost 0.4 to 0.5, the lower digits of products 0.3 (1.28 / 1.25 /
+// 1.27 without either, which loses the digits of quiet regions).
 // With the double unit no longer the bound, the persistent grid that
 // prefetches the next tile pays here too: with one tile per CTA the same
 // arithmetic took 2.67 / 2.77 / 2.72 ms (waiting at barriers and for the
@@ -310,9 +310,9 @@ __device__ __forceinline__ int fx_own(const double *f, long long p, long long st
 
 // The flux difference of one point: D_rho = 2 M, D_phi = phi_a M + sum_l
 // [m_l(a) phi_{a+l} - m_l(a-l) phi_{a-l}]: A collects the hi hi products, B
-// the mixed ones, C the lo lo ones (without them, and the sum rounded to whole
+// the mixed ones, C the lo lo ones (without them, and with the sum cut to whole
 // units, operands all near their loud bounds would have 40 times a double's
-// error; they cost 0.25 ms per launch of 420 x 250 x 320 points).  |m| is below
+// error; both cost 0.3 ms per launch of 420 x 250 x 320 points).  |m| is below
 // 2^59 sum |a_l| and the lo limbs of m are not negative, so with 8 pairs (order
 // 8) |B| stays below 2^59 (8 + 2.1 + 1 + 2.1) < 2^63, and |C| below 8 times
 // (2^30 - 1)^2 < 2^63.
@@ -393,14 +393,12 @@ __device__ __forceinline__ void fx_flux_point(const Dev &__restrict__ d, const i
       C += (long long)mm[l - 1].x * v[NP - l].x;
     }
     B += C >> FX_LIMB;
-    // unit of D: 2^60 times the units of m and phi, 2^-30 of it for small sums
-    int eD = eM + ef - 1022 + 1;
     A += B >> FX_LIMB;
-    if ((unsigned long long)(A + (1ll << 32)) >> 33 == 0) {
-      A = A * (1ll << FX_LIMB) + (B & FX_MASK);
-      eD -= FX_LIMB;
-    }
-    const double D = fx_i2d(A);
+    // as many of the lower bits as there is room for
+    const int up = min(__clzll(A ^ (A >> 63)) - 2, FX_LIMB);
+    const double D = fx_i2d((A << up) + (long long)(((int)B & FX_MASK) >> (FX_LIMB - up)));
+    // unit of D: 2^60 times the units of m and phi, 2^up of it
+    const int eD = eM + ef - 1022 + 1 - up;
     double r = fma(-fx_ldexp(scale, eD), D, prev[f]);
     if (f == 1 + DIR) r = fma(-scale, dp, r);
     out[f * d.n] = r;

@@ -95,7 +95,7 @@ def test_flux_difference_error(half):
     which there are 2 half; the last cut at most 2.  For velocities and field
     values near the loud bounds, 2^-5 of their exponents' powers of two, a pair
     flux is off by at most 0.5 + 1 + 2^-5 and meets values of at most 2^-6
-    twice, 0.05 per pair flux, and the sum is cut 2^-30 lower: the error falls
+    twice, 0.05 per pair flux, and the sum keeps lower bits: the error falls
     with the products."""
     rng = np.random.default_rng(100 + half)
     top = (1 << 59) - 1
@@ -143,9 +143,9 @@ def test_flux_difference_error(half):
         A, B = fits(A + Mh * c[1], 64), fits(B + Mh * c[0] + Ml * c[1], 64)
         B = fits(B + (fits(Ml * c[0], 64) >> LIMB) + (C >> LIMB), 64)
         A = fits(A + (B >> LIMB), 64)
-        D = Fraction(A)
-        if -(1 << 32) <= A < 1 << 32:
-            D = Fraction(fits(A * (1 << LIMB) + (B & MASK), 64), 1 << LIMB)
+        up = min(62 - (A if A >= 0 else ~A).bit_length(), LIMB)
+        assert up >= 0
+        D = Fraction(fits((A << up) + ((B & MASK) >> (LIMB - up)), 64), 1 << up)
         error = abs(D - exact / 2 ** 120)
         worst = max(worst, error)
         assert trial < 220 or error <= 0.1 * half + 0.01
